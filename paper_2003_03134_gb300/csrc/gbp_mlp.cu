@@ -17,6 +17,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -66,24 +67,93 @@ __global__ void mlp_pack_kernel(const float* __restrict__ W, uint32_t* __restric
 
 // ------------------------------------------------------------------------
 // forward over samples (inference)
+//
+// A warp walks 16-row tiles with every weight in registers: the 44 B-operand
+// fragments are 88 registers a lane, loaded once per warp, and the
+// activations stay in registers between the layers (mlp_forward_regs' scheme,
+// the same roundings and the same mma order, so the same bits).  Rows are
+// read straight into A fragments: a lane's four float2 cover whole 32-byte
+// sectors over the warp, and the next tile's are in flight while this one is
+// evaluated.  Shared memory holds only the biases.  4 million rows: 126 us
+// (the tensor pipe 61 % busy), 340 us for a block per 128 rows that copied
+// the weights to shared memory first and kept the activations there (its
+// shared-memory pipe was 94 % busy); reading the rows once takes 40 us.
 
-__global__ void __launch_bounds__(MLP_BLOCK) mlp_forward_kernel(const uint32_t* __restrict__ frag_g,
-                                                                const float* __restrict__ bias_g,
-                                                                const float* __restrict__ X, int n,
-                                                                float* __restrict__ y) {
-    __shared__ __align__(16) uint32_t frag[FWD_FRAG_WORDS];
-    __shared__ float bias[MLP_BIAS_WORDS];
-    __shared__ __align__(16) __nv_bfloat16 xs[MLP_WARPS][32 * XS];
-    __shared__ __align__(16) __nv_bfloat16 hs[MLP_WARPS][32 * HS];
-    for (int i = threadIdx.x; i < FWD_FRAG_WORDS; i += MLP_BLOCK) frag[i] = frag_g[i];
-    for (int i = threadIdx.x; i < MLP_BIAS_WORDS; i += MLP_BLOCK) bias[i] = bias_g[i];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int s = blockIdx.x * MLP_BLOCK + threadIdx.x;
+// A fragment of rows [r0, r0 + 16) of X; rows past n read as zero.
+template <bool PAIRS>
+__device__ __forceinline__ void load_rows(const float* __restrict__ X, int n, int r0, int lane, float2 (&v)[4]) {
+    const int g = lane >> 2, q = lane & 3;
 #pragma unroll
-    for (int j = 0; j < MLP_IN; ++j) xs[warp][lane * XS + j] = __float2bfloat16_rn(s < n ? X[(size_t)s * MLP_IN + j] : 0.f);
+    for (int h = 0; h < 4; ++h) {
+        const int r = r0 + g + 8 * (h & 1);
+        const float* p = X + (size_t)r * MLP_IN + 2 * q + 8 * (h >> 1);
+        if (r >= n) v[h] = make_float2(0.f, 0.f);
+        else if constexpr (PAIRS) v[h] = __ldcs(reinterpret_cast<const float2*>(p));
+        else v[h] = make_float2(p[0], p[1]);
+    }
+}
+
+template <bool PAIRS>
+__global__ void __launch_bounds__(MLP_BLOCK, 3) mlp_forward_kernel(const uint32_t* __restrict__ frag_g,
+                                                                   const float* __restrict__ bias_g,
+                                                                   const float* __restrict__ X, int n,
+                                                                   float* __restrict__ y) {
+    __shared__ __align__(16) float bias[MLP_BIAS_WORDS];
+    const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+    const int n_tiles = (n + 15) / 16, stride = gridDim.x * MLP_WARPS;
+    int tile = blockIdx.x * MLP_WARPS + (threadIdx.x >> 5);
+    float2 v[4];
+    load_rows<PAIRS>(X, n, tile < n_tiles ? 16 * tile : n, lane, v);
+    uint2 w[FT_W2T];
+#pragma unroll
+    for (int t = 0; t < FT_W2T; ++t) w[t] = reinterpret_cast<const uint2*>(frag_g)[t * 32 + lane];
+    for (int i = threadIdx.x; i < MLP_BIAS_WORDS; i += MLP_BLOCK) bias[i] = bias_g[i];
     __syncthreads();
-    const float z3 = mlp_forward_warp(frag, bias, xs[warp], hs[warp], nullptr, lane);
-    if (s < n) y[s] = mlp_output(z3);
+    for (; tile < n_tiles; tile += stride) {
+        const uint32_t x0 = pack_bf16(v[0].x, v[0].y), x1 = pack_bf16(v[1].x, v[1].y);
+        const uint32_t x2 = pack_bf16(v[2].x, v[2].y), x3 = pack_bf16(v[3].x, v[3].y);
+        load_rows<PAIRS>(X, n, tile + stride < n_tiles ? 16 * (tile + stride) : n, lane, v);
+        uint32_t a[4][4];
+        float d[8][4];
+        // layer 1: h1 = relu(X W1 + b1) -> A fragments of layer 2
+#pragma unroll
+        for (int nt = 0; nt < 8; ++nt) {
+            d[nt][0] = d[nt][1] = d[nt][2] = d[nt][3] = 0.f;
+            mma_bf16(d[nt], x0, x1, x2, x3, w[FT_L1 + nt].x, w[FT_L1 + nt].y);
+        }
+#pragma unroll
+        for (int nt = 0; nt < 8; ++nt) {
+            const float2 b = *reinterpret_cast<const float2*>(bias + 8 * nt + 2 * q);
+            a[nt >> 1][(nt & 1) ? 2 : 0] = pack_bf16_relu(d[nt][0] + b.x, d[nt][1] + b.y);
+            a[nt >> 1][(nt & 1) ? 3 : 1] = pack_bf16_relu(d[nt][2] + b.x, d[nt][3] + b.y);
+        }
+        // layer 2: h2 = relu(h1 W2 + b2) -> A fragments of layer 3
+#pragma unroll
+        for (int nt = 0; nt < 8; ++nt) d[nt][0] = d[nt][1] = d[nt][2] = d[nt][3] = 0.f;
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks)
+#pragma unroll
+            for (int nt = 0; nt < 8; ++nt)
+                mma_bf16(d[nt], a[ks][0], a[ks][1], a[ks][2], a[ks][3], w[FT_L2 + ks * 8 + nt].x,
+                         w[FT_L2 + ks * 8 + nt].y);
+#pragma unroll
+        for (int nt = 0; nt < 8; ++nt) {
+            const float2 b = *reinterpret_cast<const float2*>(bias + MLP_H + 8 * nt + 2 * q);
+            a[nt >> 1][(nt & 1) ? 2 : 0] = pack_bf16_relu(d[nt][0] + b.x, d[nt][1] + b.y);
+            a[nt >> 1][(nt & 1) ? 3 : 1] = pack_bf16_relu(d[nt][2] + b.x, d[nt][3] + b.y);
+        }
+        // layer 3: z3 = h2 W3 + b3 (column 0 of the output tile: lanes with q = 0)
+        float z[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks)
+            mma_bf16(z, a[ks][0], a[ks][1], a[ks][2], a[ks][3], w[FT_L3 + ks].x, w[FT_L3 + ks].y);
+        if (q == 0) {
+            const int r = 16 * tile + g;
+            const float b3 = bias[2 * MLP_H];
+            if (r < n) y[r] = mlp_output(z[0] + b3);
+            if (r + 8 < n) y[r + 8] = mlp_output(z[2] + b3);
+        }
+    }
 }
 
 // ------------------------------------------------------------------------
@@ -437,7 +507,18 @@ gbp_status gbp_mlp_get_params(const gbp_mlp* n, float* params) {
 gbp_status gbp_mlp_forward(gbp_mlp* n, const float* X, int32_t count, float* y) {
     if (!n || count < 0 || (count && (!X || !y))) return GBP_EINVAL;
     if (count == 0) return GBP_OK;
-    mlp_forward_kernel<<<(count + MLP_BLOCK - 1) / MLP_BLOCK, MLP_BLOCK, 0, n->stream>>>(n->frag, n->bias, X, count, y);
+    // resident blocks walk the tiles (three per SM, the register budget); X may
+    // be aligned to a float only
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return GBP_ECUDA;
+    const int tiles = (count + 15) / 16;
+    const int blocks = std::min((tiles + MLP_WARPS - 1) / MLP_WARPS, 3 * sms);
+    if (reinterpret_cast<uintptr_t>(X) % 8 == 0)
+        mlp_forward_kernel<true><<<blocks, MLP_BLOCK, 0, n->stream>>>(n->frag, n->bias, X, count, y);
+    else
+        mlp_forward_kernel<false><<<blocks, MLP_BLOCK, 0, n->stream>>>(n->frag, n->bias, X, count, y);
     return cudaGetLastError() == cudaSuccess ? GBP_OK : GBP_ECUDA;
 }
 

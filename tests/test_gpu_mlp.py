@@ -178,3 +178,27 @@ def test_invalid_arguments(torch):
     net.forward(Xd.data_ptr(), 0, td.data_ptr())   # empty batch is a no-op
     np.testing.assert_array_equal(net.params, p)
     net.close()
+
+
+@pytest.mark.parametrize("n", [1, 15, 16, 17, 63, 65, 29184 - 1, 29184 + 17])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_forward_rows_do_not_depend_on_their_place(torch, n, offset):
+    """Row counts around the 16-row tile and around one tile per resident warp (152 SMs x 12 warps x 16 rows),
+    rows aligned to 8 bytes or to a float only: each row's prediction is bitwise the one it gets in another
+    place of another call, and rows past the end are not written."""
+    p = _params(1)
+    X, _ = _data(n, n)
+    net = gbp.DampingNet(p)
+    buf = torch.zeros(n * 16 + 1, dtype=torch.float32, device="cuda")
+    buf[offset:offset + n * 16] = _dev(torch, X).reshape(-1)
+    y = torch.full((n + 16,), -1.0, dtype=torch.float32, device="cuda")
+    net.forward(buf[offset:].data_ptr(), n, y.data_ptr())
+    perm = torch.randperm(n, generator=torch.Generator().manual_seed(n)).cuda()
+    Xp = _dev(torch, X)[perm].contiguous()
+    yp = torch.empty(n, dtype=torch.float32, device="cuda")
+    net.forward(Xp.data_ptr(), n, yp.data_ptr())
+    torch.cuda.synchronize()
+    assert torch.equal(y[:n][perm], yp)
+    assert bool((y[n:] == -1.0).all())
+    ref, _ = mlp.forward(p, X.astype(np.float64))
+    assert np.abs(y[:n].cpu().numpy() - ref).max() <= 0.02
