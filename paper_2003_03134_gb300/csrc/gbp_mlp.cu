@@ -4,13 +4,13 @@
 // C ABI of the gbp_mlp object.
 //
 // One training step over a batch of B samples:
-//   mlp_grad_kernel    one block per 128 samples (4 warps x 32): forward,
-//                      backward, this block's partial gradient (warp
-//                      partials added in fixed warp order) and loss;
-//   mlp_reduce_kernel  one thread per parameter: sum of the block partials in
-//                      block order (deterministic), then optionally Adam;
-//   mlp_pack_kernel    BF16 B-operand fragments and FP32 biases from the
-//                      master weights.
+//   mlp_grad_kernel    one warp (a block) per 32 samples: forward, backward,
+//                      this warp's partial gradient and loss;
+//   mlp_reduce_kernel  the partials added in a fixed order (deterministic),
+//                      then optionally Adam and the new weights' BF16
+//                      B-operand fragments.
+// mlp_pack_kernel packs the fragments and FP32 biases from master weights set
+// by the caller.
 #include "gbp_mlp.cuh"
 #include "gbp_internal.h"
 #include "../../include/gbp.h"
@@ -30,6 +30,9 @@ static_assert(MLP_NPARAM == GBP_MLP_NPARAM && MLP_IN == GBP_MLP_NFEAT, "paramete
 
 constexpr int MLP_BLOCK = 128;               // samples per block
 constexpr int MLP_WARPS = MLP_BLOCK / 32;
+constexpr int GRAD_WAVE = 2048;              // warps of mlp_grad_kernel that run at once (14 on each of 152 SMs, rounded down)
+constexpr int MLP_PART = MLP_NPARAM + 3;     // a warp's partial gradient, its loss, pad to an even count (8-byte rows)
+static_assert(MLP_PART % 2 == 0, "float2 stores");
 
 // ------------------------------------------------------------------------
 // packing: fragment tile t, lane l holds B[2q..2q+1][g] and B[2q+8..2q+9][g]
@@ -79,6 +82,9 @@ __global__ void mlp_pack_kernel(const float* __restrict__ W, uint32_t* __restric
 // the weights to shared memory first and kept the activations there (its
 // shared-memory pipe was 94 % busy); reading the rows once takes 40 us.
 
+// relu, then a BF16 pair; a NaN becomes 0 (fmaxf)
+__device__ __forceinline__ uint32_t pack_relu(float lo, float hi) { return pack_bf16(fmaxf(lo, 0.f), fmaxf(hi, 0.f)); }
+
 // A fragment of rows [r0, r0 + 16) of X; rows past n read as zero.
 template <bool PAIRS>
 __device__ __forceinline__ void load_rows(const float* __restrict__ X, int n, int r0, int lane, float2 (&v)[4]) {
@@ -124,8 +130,8 @@ __global__ void __launch_bounds__(MLP_BLOCK, 3) mlp_forward_kernel(const uint32_
 #pragma unroll
         for (int nt = 0; nt < 8; ++nt) {
             const float2 b = *reinterpret_cast<const float2*>(bias + 8 * nt + 2 * q);
-            a[nt >> 1][(nt & 1) ? 2 : 0] = pack_bf16_relu(d[nt][0] + b.x, d[nt][1] + b.y);
-            a[nt >> 1][(nt & 1) ? 3 : 1] = pack_bf16_relu(d[nt][2] + b.x, d[nt][3] + b.y);
+            a[nt >> 1][(nt & 1) ? 2 : 0] = pack_relu(d[nt][0] + b.x, d[nt][1] + b.y);
+            a[nt >> 1][(nt & 1) ? 3 : 1] = pack_relu(d[nt][2] + b.x, d[nt][3] + b.y);
         }
         // layer 2: h2 = relu(h1 W2 + b2) -> A fragments of layer 3
 #pragma unroll
@@ -139,8 +145,8 @@ __global__ void __launch_bounds__(MLP_BLOCK, 3) mlp_forward_kernel(const uint32_
 #pragma unroll
         for (int nt = 0; nt < 8; ++nt) {
             const float2 b = *reinterpret_cast<const float2*>(bias + MLP_H + 8 * nt + 2 * q);
-            a[nt >> 1][(nt & 1) ? 2 : 0] = pack_bf16_relu(d[nt][0] + b.x, d[nt][1] + b.y);
-            a[nt >> 1][(nt & 1) ? 3 : 1] = pack_bf16_relu(d[nt][2] + b.x, d[nt][3] + b.y);
+            a[nt >> 1][(nt & 1) ? 2 : 0] = pack_relu(d[nt][0] + b.x, d[nt][1] + b.y);
+            a[nt >> 1][(nt & 1) ? 3 : 1] = pack_relu(d[nt][2] + b.x, d[nt][3] + b.y);
         }
         // layer 3: z3 = h2 W3 + b3 (column 0 of the output tile: lanes with q = 0)
         float z[4] = {0.f, 0.f, 0.f, 0.f};
@@ -157,225 +163,403 @@ __global__ void __launch_bounds__(MLP_BLOCK, 3) mlp_forward_kernel(const uint32_
 }
 
 // ------------------------------------------------------------------------
-// forward + backward of one block of samples
+// forward + backward of a minibatch: one warp per block, 32 samples
+//
+// A training minibatch is 4096 rows, so the step is a latency chain, not a
+// throughput problem: a warp per 32 rows spreads it over 128 blocks (a block
+// of 4 warps left 120 SMs idle).  Weights are read from L2 as B fragments by
+// the warp that uses them (each once: 76 loads in flight at will), with no
+// copy to shared memory; the activations and dz2 stay in registers as the A
+// fragments of the next product, and go to shared memory only for the
+// products over samples (dW2 = h1^T dz2, dW1 = x^T dz1), whose transposed
+// operands ldmatrix.trans reads 8 x 8 blocks at a time.  Each warp writes its
+// own partial gradient; mlp_reduce_kernel adds them.
+//
+// GROUPED (more rows than one wave of warps takes): a warp works the four 32s
+// of 128 samples and adds them up in its partial, in the same order, so the
+// partials take no more memory than one per 128 samples.
 
 struct GradSmem {
-    uint32_t frag[FRAG_WORDS];
-    float bias[MLP_BIAS_WORDS];
-    alignas(16) __nv_bfloat16 x[MLP_WARPS][32 * XS];
-    alignas(16) __nv_bfloat16 h1[MLP_WARPS][32 * HS];
-    alignas(16) __nv_bfloat16 h2[MLP_WARPS][32 * HS];   // h2, later dz1
-    alignas(16) __nv_bfloat16 dz[MLP_WARPS][32 * HS];   // dz2
-    float dz3[MLP_WARPS][32];
-    float gW2[MLP_H * MLP_H];
-    float gW1[MLP_IN * MLP_H];
-    float gvec[MLP_H * 3 + 1];              // b1, b2, W3, b3 partials
-    float loss;
+    alignas(16) __nv_bfloat16 x[32 * XS];
+    alignas(16) __nv_bfloat16 h1[32 * HS];
+    alignas(16) __nv_bfloat16 h2[32 * HS];   // h2, later dz1
+    alignas(16) __nv_bfloat16 dz[32 * HS];   // dz2
+    float dz3[32];
 };
 
-__global__ void __launch_bounds__(MLP_BLOCK) mlp_grad_kernel(const uint32_t* __restrict__ frag_g,
-                                                             const float* __restrict__ bias_g,
-                                                             const float* __restrict__ X, const float* __restrict__ T,
-                                                             const int32_t* __restrict__ idx, int n, float inv_batch,
-                                                             float* __restrict__ partials) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    GradSmem& S = *reinterpret_cast<GradSmem*>(smem_raw);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int g = lane >> 2, q = lane & 3;
-    for (int i = tid; i < FRAG_WORDS; i += MLP_BLOCK) S.frag[i] = frag_g[i];
-    for (int i = tid; i < MLP_BIAS_WORDS; i += MLP_BLOCK) S.bias[i] = bias_g[i];
-    for (int i = tid; i < MLP_H * MLP_H; i += MLP_BLOCK) S.gW2[i] = 0.f;
-    for (int i = tid; i < MLP_IN * MLP_H; i += MLP_BLOCK) S.gW1[i] = 0.f;
-    for (int i = tid; i < MLP_H * 3 + 1; i += MLP_BLOCK) S.gvec[i] = 0.f;
-    if (tid == 0) S.loss = 0.f;
-    const int si = blockIdx.x * MLP_BLOCK + tid;      // this lane's sample slot
+// four transposed 8 x 8 blocks; lane l gives the address of row l % 8 of block l / 8
+__device__ __forceinline__ void ldmatrix_t(const __nv_bfloat16* p, uint32_t (&r)[4]) {
+    const unsigned a = static_cast<unsigned>(__cvta_generic_to_shared(p));
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(a)
+                 : "memory");
+}
+
+__device__ __forceinline__ uint2 load_frag(const uint32_t* __restrict__ frag, int tile, int lane) {
+    return *reinterpret_cast<const uint2*>(frag + (tile * 32 + lane) * 2);
+}
+
+// a value kept where the activation it belongs to (a BF16 half) is positive
+__device__ __forceinline__ float where_pos(uint32_t h, bool upper, float v) {
+    const uint32_t b = upper ? h >> 16 : h & 0xffffu;
+    return b - 1u < 0x7f80u ? v : 0.f;   // (0, inf] by its bits
+}
+
+__device__ __forceinline__ void pdl_wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// a warp's (or group's) partial: stored by its first 32 samples, added to by
+// the others
+__device__ __forceinline__ void put2(float* o, bool first, float a, float b) {
+    if (!first) {
+        const float2 v = *reinterpret_cast<const float2*>(o);
+        a = v.x + a;
+        b = v.y + b;
+    }
+    *reinterpret_cast<float2*>(o) = make_float2(a, b);
+}
+__device__ __forceinline__ void put1(float* o, bool first, float a) { *o = first ? a : *o + a; }
+
+template <bool GROUPED>
+__global__ void __launch_bounds__(32) mlp_grad_kernel(const uint32_t* __restrict__ frag, const float* __restrict__ bias,
+                                                      const float* __restrict__ X, const float* __restrict__ T,
+                                                      const int32_t* __restrict__ idx, int n, float inv_batch,
+                                                      float* __restrict__ partials) {
+    __shared__ GradSmem S;
+    const int lane = threadIdx.x, g = lane >> 2, q = lane & 3;
+    pdl_wait_previous();
+    for (int sub = 0; sub < (GROUPED ? 4 : 1); ++sub) {
+    const int si = (GROUPED ? 4 * int(blockIdx.x) + sub : int(blockIdx.x)) * 32 + lane;   // this lane's sample slot
     const bool valid = si < n;
     const int sample = valid ? (idx ? idx[si] : si) : 0;
+    const bool first = !GROUPED || sub == 0;
+    if (GROUPED) __syncwarp();   // the tiles are rewritten
+    {
+        float x[MLP_IN];
+        const float* row = X + (size_t)sample * MLP_IN;
+        if (!valid) {
 #pragma unroll
-    for (int j = 0; j < MLP_IN; ++j)
-        S.x[warp][lane * XS + j] = __float2bfloat16_rn(valid ? X[(size_t)sample * MLP_IN + j] : 0.f);
-    __syncthreads();
+            for (int j = 0; j < MLP_IN; ++j) x[j] = 0.f;
+        } else if (reinterpret_cast<uintptr_t>(X) % 16 == 0) {
+#pragma unroll
+            for (int j = 0; j < MLP_IN / 4; ++j) {
+                const float4 v = reinterpret_cast<const float4*>(row)[j];
+                x[4 * j] = v.x; x[4 * j + 1] = v.y; x[4 * j + 2] = v.z; x[4 * j + 3] = v.w;
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < MLP_IN; ++j) x[j] = row[j];
+        }
+        uint32_t p[MLP_IN / 2];
+#pragma unroll
+        for (int j = 0; j < MLP_IN / 2; ++j) p[j] = pack_bf16(x[2 * j], x[2 * j + 1]);
+        uint4* out = reinterpret_cast<uint4*>(S.x + lane * XS);
+        out[0] = make_uint4(p[0], p[1], p[2], p[3]);
+        out[1] = make_uint4(p[4], p[5], p[6], p[7]);
+    }
+    const float target = valid ? T[sample] : 0.f;
+    __syncwarp();
 
-    // forward, keeping h1 and h2
-    const float z3 = mlp_forward_warp(S.frag, S.bias, S.x[warp], S.h2[warp], S.h1[warp], lane);
-    // the forward pass reused the input tile: restore it for dW1
+    // forward: h1, h2 as A fragments of the next layer and as rows in shared memory
+    uint32_t a1[2][4][4], a2[2][4][4];
+    {
+        uint32_t x0[4], x1[4];
+        load_a(S.x, XS, 0, 0, lane, x0[0], x0[1], x0[2], x0[3]);
+        load_a(S.x, XS, 16, 0, lane, x1[0], x1[1], x1[2], x1[3]);
 #pragma unroll
-    for (int j = 0; j < MLP_IN; ++j)
-        S.x[warp][lane * XS + j] = __float2bfloat16_rn(valid ? X[(size_t)sample * MLP_IN + j] : 0.f);
+        for (int nt = 0; nt < 8; ++nt) {
+            const uint2 w = load_frag(frag, FT_L1 + nt, lane);
+            const float b0 = bias[8 * nt + 2 * q], b1 = bias[8 * nt + 2 * q + 1];
+            float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
+            mma_bf16(d0, x0[0], x0[1], x0[2], x0[3], w.x, w.y);
+            mma_bf16(d1, x1[0], x1[1], x1[2], x1[3], w.x, w.y);
+            const int ks = nt >> 1, o = (nt & 1) * 2;
+            a1[0][ks][o] = pack_relu(d0[0] + b0, d0[1] + b1);
+            a1[0][ks][o + 1] = pack_relu(d0[2] + b0, d0[3] + b1);
+            a1[1][ks][o] = pack_relu(d1[0] + b0, d1[1] + b1);
+            a1[1][ks][o + 1] = pack_relu(d1[2] + b0, d1[3] + b1);
+        }
+    }
+#pragma unroll
+    for (int nt = 0; nt < 8; ++nt) {
+        const float b0 = bias[MLP_H + 8 * nt + 2 * q], b1 = bias[MLP_H + 8 * nt + 2 * q + 1];
+        float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks) {
+            const uint2 w = load_frag(frag, FT_L2 + ks * 8 + nt, lane);
+            mma_bf16(d0, a1[0][ks][0], a1[0][ks][1], a1[0][ks][2], a1[0][ks][3], w.x, w.y);
+            mma_bf16(d1, a1[1][ks][0], a1[1][ks][1], a1[1][ks][2], a1[1][ks][3], w.x, w.y);
+        }
+        const int ks = nt >> 1, o = (nt & 1) * 2;
+        a2[0][ks][o] = pack_relu(d0[0] + b0, d0[1] + b1);
+        a2[0][ks][o + 1] = pack_relu(d0[2] + b0, d0[3] + b1);
+        a2[1][ks][o] = pack_relu(d1[0] + b0, d1[1] + b1);
+        a2[1][ks][o + 1] = pack_relu(d1[2] + b0, d1[3] + b1);
+    }
+    float z[2][4];
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt) z[mt][0] = z[mt][1] = z[mt][2] = z[mt][3] = 0.f;
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks) {
+        const uint2 w = load_frag(frag, FT_L3 + ks, lane);
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt) mma_bf16(z[mt], a2[mt][ks][0], a2[mt][ks][1], a2[mt][ks][2], a2[mt][ks][3], w.x, w.y);
+    }
+    // row r = lane of column 0: held by lane 4 (r % 8) of m-tile r / 16
+    float z3;
+    {
+        const int src = (lane & 7) << 2;
+        const float v00 = __shfl_sync(0xffffffffu, z[0][0], src), v01 = __shfl_sync(0xffffffffu, z[0][2], src);
+        const float v10 = __shfl_sync(0xffffffffu, z[1][0], src), v11 = __shfl_sync(0xffffffffu, z[1][2], src);
+        z3 = ((lane < 16) ? ((lane & 8) ? v01 : v00) : ((lane & 8) ? v11 : v10)) + bias[2 * MLP_H];
+    }
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks)
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                const int at = (16 * mt + g + 8 * (h & 1)) * HS + 16 * ks + 2 * q + 8 * (h >> 1);
+                *reinterpret_cast<uint32_t*>(S.h1 + at) = a1[mt][ks][h];
+                *reinterpret_cast<uint32_t*>(S.h2 + at) = a2[mt][ks][h];
+            }
     const float sg = 1.0f / (1.0f + __expf(-z3));
     const float y = MLP_DMAX * sg;
-    const float r = valid ? y - T[sample] : 0.f;
+    const float r = valid ? y - target : 0.f;
     // loss = mean r^2 ; dL/dz3 = 2 r / B * 0.9 s (1 - s)
     const float dz3 = 2.0f * r * inv_batch * MLP_DMAX * sg * (1.0f - sg);
-    S.dz3[warp][lane] = dz3;
-    __syncwarp();
+    S.dz3[lane] = dz3;
     float r2 = r * r * inv_batch;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) r2 += __shfl_down_sync(0xffffffffu, r2, o);
-
-    // dz2[s][j] = dz3[s] W3[j] [h2 > 0]  (row s = this lane), as BF16
-    const float* W3 = S.bias + 2 * MLP_H + 2;
-#pragma unroll 8
-    for (int j = 0; j < MLP_H; j += 2) {
-        const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162*>(S.h2[warp] + lane * HS + j);
-        const float v0 = __bfloat162float(h.x) > 0.f ? dz3 * W3[j] : 0.f;
-        const float v1 = __bfloat162float(h.y) > 0.f ? dz3 * W3[j + 1] : 0.f;
-        *reinterpret_cast<uint32_t*>(S.dz[warp] + lane * HS + j) = pack_bf16(v0, v1);
-    }
-    __syncwarp();
-    // vector partials of this warp: dW3[j] = sum_s h2[s][j] dz3[s], db2[j] =
-    // sum_s dz2[s][j], db3 = sum_s dz3[s] (lane takes j = lane, lane + 32)
-    float pW3[2] = {0.f, 0.f}, pb2[2] = {0.f, 0.f};
-    for (int s = 0; s < 32; ++s) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int j = lane + 32 * h;
-            pW3[h] += __bfloat162float(S.h2[warp][s * HS + j]) * S.dz3[warp][s];
-            pb2[h] += __bfloat162float(S.dz[warp][s * HS + j]);
-        }
-    }
     float pb3 = dz3;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) pb3 += __shfl_down_sync(0xffffffffu, pb3, o);
+
+    // dz2[s][j] = dz3[s] W3[j] [h2 > 0] in h2's fragment positions (in place of it), as BF16
+    const float* W3 = bias + 2 * MLP_H + 2;
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt) {
+        const float r0 = __shfl_sync(0xffffffffu, dz3, 16 * mt + g), r1 = __shfl_sync(0xffffffffu, dz3, 16 * mt + g + 8);
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks)
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                const int c = 16 * ks + 2 * q + 8 * (h >> 1);
+                const float d = (h & 1) ? r1 : r0;
+                const uint32_t v = pack_bf16(where_pos(a2[mt][ks][h], false, d * W3[c]),
+                                             where_pos(a2[mt][ks][h], true, d * W3[c + 1]));
+                a2[mt][ks][h] = v;
+                *reinterpret_cast<uint32_t*>(S.dz + (16 * mt + g + 8 * (h & 1)) * HS + c) = v;
+            }
+    }
+    __syncwarp();
+    // vector partials: dW3[j] = sum_s h2[s][j] dz3[s], db2[j] = sum_s dz2[s][j],
+    // db3 = sum_s dz3[s], in sample order (lane takes j = 2 lane, 2 lane + 1)
+    float pW3[2] = {0.f, 0.f}, pb2[2] = {0.f, 0.f};
+#pragma unroll 8
+    for (int s = 0; s < 32; ++s) {
+        const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162*>(S.h2 + s * HS + 2 * lane);
+        const __nv_bfloat162 d = *reinterpret_cast<const __nv_bfloat162*>(S.dz + s * HS + 2 * lane);
+        const float ds = S.dz3[s];
+        pW3[0] = fmaf(__bfloat162float(h.x), ds, pW3[0]);
+        pW3[1] = fmaf(__bfloat162float(h.y), ds, pW3[1]);
+        pb2[0] += __bfloat162float(d.x);
+        pb2[1] += __bfloat162float(d.y);
+    }
     __syncwarp();
 
     // dh1 = dz2 W2^T ; dz1 = dh1 [h1 > 0]  -> BF16 into the h2 tile
 #pragma unroll
-    for (int mt = 0; mt < 2; ++mt) {
-        uint32_t a[4][4];
+    for (int nt = 0; nt < 8; ++nt) {
+        float d[2][4];
 #pragma unroll
-        for (int ks = 0; ks < 4; ++ks) load_a(S.dz[warp], HS, 16 * mt, 16 * ks, lane, a[ks][0], a[ks][1], a[ks][2], a[ks][3]);
+        for (int mt = 0; mt < 2; ++mt) d[mt][0] = d[mt][1] = d[mt][2] = d[mt][3] = 0.f;
 #pragma unroll
-        for (int nt = 0; nt < 8; ++nt) {
-            float d[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int ks = 0; ks < 4; ++ks) {
+            const uint2 w = load_frag(frag, FT_W2T + ks * 8 + nt, lane);
 #pragma unroll
-            for (int ks = 0; ks < 4; ++ks) {
-                uint32_t b0, b1;
-                load_b(S.frag, FT_W2T + ks * 8 + nt, lane, b0, b1);
-                mma_bf16(d, a[ks][0], a[ks][1], a[ks][2], a[ks][3], b0, b1);
-            }
-            // apply the ReLU mask of layer 1 and store dz1 as BF16
-            const __nv_bfloat16* H1 = S.h1[warp];
-            const int r0 = 16 * mt + g, c0 = 8 * nt + 2 * q;
-            const __nv_bfloat162 m0 = *reinterpret_cast<const __nv_bfloat162*>(H1 + r0 * HS + c0);
-            const __nv_bfloat162 m1 = *reinterpret_cast<const __nv_bfloat162*>(H1 + (r0 + 8) * HS + c0);
-            *reinterpret_cast<uint32_t*>(S.h2[warp] + r0 * HS + c0) =
-                pack_bf16(__bfloat162float(m0.x) > 0.f ? d[0] : 0.f, __bfloat162float(m0.y) > 0.f ? d[1] : 0.f);
-            *reinterpret_cast<uint32_t*>(S.h2[warp] + (r0 + 8) * HS + c0) =
-                pack_bf16(__bfloat162float(m1.x) > 0.f ? d[2] : 0.f, __bfloat162float(m1.y) > 0.f ? d[3] : 0.f);
+            for (int mt = 0; mt < 2; ++mt)
+                mma_bf16(d[mt], a2[mt][ks][0], a2[mt][ks][1], a2[mt][ks][2], a2[mt][ks][3], w.x, w.y);
+        }
+        // the ReLU mask of layer 1: h1 fragment (nt >> 1) holds columns 8 nt + 2q of both rows
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt) {
+            const uint32_t m0 = a1[mt][nt >> 1][(nt & 1) * 2], m1 = a1[mt][nt >> 1][(nt & 1) * 2 + 1];
+            const int at = (16 * mt + g) * HS + 8 * nt + 2 * q;
+            *reinterpret_cast<uint32_t*>(S.h2 + at) =
+                pack_bf16(where_pos(m0, false, d[mt][0]), where_pos(m0, true, d[mt][1]));
+            *reinterpret_cast<uint32_t*>(S.h2 + at + 8 * HS) =
+                pack_bf16(where_pos(m1, false, d[mt][2]), where_pos(m1, true, d[mt][3]));
         }
     }
     __syncwarp();
+    if (!GROUPED) pdl_launch_next();
     float pb1[2] = {0.f, 0.f};
+#pragma unroll 8
     for (int s = 0; s < 32; ++s) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) pb1[h] += __bfloat162float(S.h2[warp][s * HS + lane + 32 * h]);
+        const __nv_bfloat162 d = *reinterpret_cast<const __nv_bfloat162*>(S.h2 + s * HS + 2 * lane);
+        pb1[0] += __bfloat162float(d.x);
+        pb1[1] += __bfloat162float(d.y);
     }
 
-    // weight-gradient GEMMs over this warp's 32 samples (K = samples):
-    // dW2 = h1^T dz2 (64 x 64), dW1 = x^T dz1 (16 x 64)
-    float dW2[4][8][4];
+    // weight-gradient products over the 32 samples (K = samples): dW2 =
+    // h1^T dz2 (64 x 64), dW1 = x^T dz1 (16 x 64), straight to this warp's
+    // partial gradient in the flat parameter layout
+    float* out = partials + (size_t)blockIdx.x * MLP_PART;
+    const int lr = lane & 7, lb = lane >> 3;
+    {
+        uint32_t bz[2][8][2];   // B fragments of dz2: [k-step][n-tile]
 #pragma unroll
-    for (int mt = 0; mt < 4; ++mt)
+        for (int ks = 0; ks < 2; ++ks)
 #pragma unroll
-        for (int nt = 0; nt < 8; ++nt) dW2[mt][nt][0] = dW2[mt][nt][1] = dW2[mt][nt][2] = dW2[mt][nt][3] = 0.f;
-    float dW1[8][4];
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) dW1[nt][0] = dW1[nt][1] = dW1[nt][2] = dW1[nt][3] = 0.f;
-    const unsigned short* H1u = reinterpret_cast<const unsigned short*>(S.h1[warp]);
-    const unsigned short* DZu = reinterpret_cast<const unsigned short*>(S.dz[warp]);
-    const unsigned short* D1u = reinterpret_cast<const unsigned short*>(S.h2[warp]);
-    const unsigned short* Xu = reinterpret_cast<const unsigned short*>(S.x[warp]);
-#pragma unroll
-    for (int ks = 0; ks < 2; ++ks) {
-        const int s0 = 16 * ks + 2 * q;   // samples of this lane's A columns / B rows
-        uint32_t bz[8][2], b1f[8][2];
-#pragma unroll
-        for (int nt = 0; nt < 8; ++nt) {
-            const int col = 8 * nt + g;
-            bz[nt][0] = uint32_t(DZu[s0 * HS + col]) | (uint32_t(DZu[(s0 + 1) * HS + col]) << 16);
-            bz[nt][1] = uint32_t(DZu[(s0 + 8) * HS + col]) | (uint32_t(DZu[(s0 + 9) * HS + col]) << 16);
-            b1f[nt][0] = uint32_t(D1u[s0 * HS + col]) | (uint32_t(D1u[(s0 + 1) * HS + col]) << 16);
-            b1f[nt][1] = uint32_t(D1u[(s0 + 8) * HS + col]) | (uint32_t(D1u[(s0 + 9) * HS + col]) << 16);
-        }
+            for (int nt = 0; nt < 8; nt += 2) {
+                uint32_t v[4];
+                ldmatrix_t(S.dz + (16 * ks + (lb & 1) * 8 + lr) * HS + 8 * (nt + (lb >> 1)), v);
+                bz[ks][nt][0] = v[0]; bz[ks][nt][1] = v[1];
+                bz[ks][nt + 1][0] = v[2]; bz[ks][nt + 1][1] = v[3];
+            }
 #pragma unroll
         for (int mt = 0; mt < 4; ++mt) {
-            const int ra = 16 * mt + g;    // rows of A = h1 units
-            const uint32_t a0 = uint32_t(H1u[s0 * HS + ra]) | (uint32_t(H1u[(s0 + 1) * HS + ra]) << 16);
-            const uint32_t a1 = uint32_t(H1u[s0 * HS + ra + 8]) | (uint32_t(H1u[(s0 + 1) * HS + ra + 8]) << 16);
-            const uint32_t a2 = uint32_t(H1u[(s0 + 8) * HS + ra]) | (uint32_t(H1u[(s0 + 9) * HS + ra]) << 16);
-            const uint32_t a3 = uint32_t(H1u[(s0 + 8) * HS + ra + 8]) | (uint32_t(H1u[(s0 + 9) * HS + ra + 8]) << 16);
+            float d[8][4];
 #pragma unroll
-            for (int nt = 0; nt < 8; ++nt) mma_bf16(dW2[mt][nt], a0, a1, a2, a3, bz[nt][0], bz[nt][1]);
-        }
-        {
-            const int ra = g;              // rows of A = input features
-            const uint32_t a0 = uint32_t(Xu[s0 * XS + ra]) | (uint32_t(Xu[(s0 + 1) * XS + ra]) << 16);
-            const uint32_t a1 = uint32_t(Xu[s0 * XS + ra + 8]) | (uint32_t(Xu[(s0 + 1) * XS + ra + 8]) << 16);
-            const uint32_t a2 = uint32_t(Xu[(s0 + 8) * XS + ra]) | (uint32_t(Xu[(s0 + 9) * XS + ra]) << 16);
-            const uint32_t a3 = uint32_t(Xu[(s0 + 8) * XS + ra + 8]) | (uint32_t(Xu[(s0 + 9) * XS + ra + 8]) << 16);
+            for (int nt = 0; nt < 8; ++nt) d[nt][0] = d[nt][1] = d[nt][2] = d[nt][3] = 0.f;
 #pragma unroll
-            for (int nt = 0; nt < 8; ++nt) mma_bf16(dW1[nt], a0, a1, a2, a3, b1f[nt][0], b1f[nt][1]);
-        }
-    }
-    // add the warp partials into the block accumulators in warp order
-    for (int w = 0; w < MLP_WARPS; ++w) {
-        if (warp == w) {
+            for (int ks = 0; ks < 2; ++ks) {
+                uint32_t a[4];   // rows of A = h1 units
+                ldmatrix_t(S.h1 + (16 * ks + (lb >> 1) * 8 + lr) * HS + 16 * mt + (lb & 1) * 8, a);
 #pragma unroll
-            for (int mt = 0; mt < 4; ++mt)
-#pragma unroll
-                for (int nt = 0; nt < 8; ++nt) {
-                    const int r = 16 * mt + g, c = 8 * nt + 2 * q;
-                    S.gW2[r * MLP_H + c] += dW2[mt][nt][0];
-                    S.gW2[r * MLP_H + c + 1] += dW2[mt][nt][1];
-                    S.gW2[(r + 8) * MLP_H + c] += dW2[mt][nt][2];
-                    S.gW2[(r + 8) * MLP_H + c + 1] += dW2[mt][nt][3];
-                }
+                for (int nt = 0; nt < 8; ++nt) mma_bf16(d[nt], a[0], a[1], a[2], a[3], bz[ks][nt][0], bz[ks][nt][1]);
+            }
 #pragma unroll
             for (int nt = 0; nt < 8; ++nt) {
-                const int c = 8 * nt + 2 * q;
-                S.gW1[g * MLP_H + c] += dW1[nt][0];
-                S.gW1[g * MLP_H + c + 1] += dW1[nt][1];
-                S.gW1[(g + 8) * MLP_H + c] += dW1[nt][2];
-                S.gW1[(g + 8) * MLP_H + c + 1] += dW1[nt][3];
-            }
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                S.gvec[lane + 32 * h] += pb1[h];
-                S.gvec[MLP_H + lane + 32 * h] += pb2[h];
-                S.gvec[2 * MLP_H + lane + 32 * h] += pW3[h];
-            }
-            if (lane == 0) {
-                S.gvec[3 * MLP_H] += pb3;
-                S.loss += r2;
+                float* o = out + MLP_OFF_W2 + (16 * mt + g) * MLP_H + 8 * nt + 2 * q;
+                put2(o, first, d[nt][0], d[nt][1]);
+                put2(o + 8 * MLP_H, first, d[nt][2], d[nt][3]);
             }
         }
-        __syncthreads();
     }
-    // write this block's partial gradient in the flat parameter layout
-    float* out = partials + (size_t)blockIdx.x * (MLP_NPARAM + 1);
-    for (int i = tid; i < MLP_IN * MLP_H; i += MLP_BLOCK) out[MLP_OFF_W1 + i] = S.gW1[i];
-    for (int i = tid; i < MLP_H * MLP_H; i += MLP_BLOCK) out[MLP_OFF_W2 + i] = S.gW2[i];
-    for (int i = tid; i < MLP_H; i += MLP_BLOCK) {
-        out[MLP_OFF_B1 + i] = S.gvec[i];
-        out[MLP_OFF_B2 + i] = S.gvec[MLP_H + i];
-        out[MLP_OFF_W3 + i] = S.gvec[2 * MLP_H + i];
+    {
+        float d[8][4];
+#pragma unroll
+        for (int nt = 0; nt < 8; ++nt) d[nt][0] = d[nt][1] = d[nt][2] = d[nt][3] = 0.f;
+#pragma unroll
+        for (int ks = 0; ks < 2; ++ks) {
+            uint32_t a[4];       // rows of A = input features
+            ldmatrix_t(S.x + (16 * ks + (lb >> 1) * 8 + lr) * XS + (lb & 1) * 8, a);
+#pragma unroll
+            for (int nt = 0; nt < 8; nt += 2) {
+                uint32_t v[4];
+                ldmatrix_t(S.h2 + (16 * ks + (lb & 1) * 8 + lr) * HS + 8 * (nt + (lb >> 1)), v);
+                mma_bf16(d[nt], a[0], a[1], a[2], a[3], v[0], v[1]);
+                mma_bf16(d[nt + 1], a[0], a[1], a[2], a[3], v[2], v[3]);
+            }
+        }
+#pragma unroll
+        for (int nt = 0; nt < 8; ++nt) {
+            float* o = out + MLP_OFF_W1 + g * MLP_H + 8 * nt + 2 * q;
+            put2(o, first, d[nt][0], d[nt][1]);
+            put2(o + 8 * MLP_H, first, d[nt][2], d[nt][3]);
+        }
     }
-    if (tid == 0) {
-        out[MLP_OFF_B3] = S.gvec[3 * MLP_H];
-        out[MLP_NPARAM] = S.loss;
+    put2(out + MLP_OFF_B1 + 2 * lane, first, pb1[0], pb1[1]);
+    put2(out + MLP_OFF_B2 + 2 * lane, first, pb2[0], pb2[1]);
+    put2(out + MLP_OFF_W3 + 2 * lane, first, pW3[0], pW3[1]);
+    if (lane == 0) {
+        put1(out + MLP_OFF_B3, first, pb3);
+        put1(out + MLP_NPARAM, first, r2);
+    }
     }
 }
 
-// Sum of the block partials in block order; optionally an Adam step
-// (step >= 1).  grad_out (nullable) receives the gradient, loss_out the loss.
-__global__ void mlp_reduce_kernel(const float* __restrict__ partials, int n_blocks, float* __restrict__ W,
-                                  float* __restrict__ m, float* __restrict__ v, int step, float lr,
-                                  float* __restrict__ grad_out, float* __restrict__ loss_out) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p > MLP_NPARAM) return;
+// The updated parameter's places in the packed fragments and the side buffer
+// (what mlp_pack_kernel writes for it).
+__device__ __forceinline__ void pack_param(int p, float w, uint32_t* __restrict__ frag, float* __restrict__ bias) {
+    auto put = [&](int tile, int k, int n) {   // element [k][n] of a 16 x 8 B tile
+        const int word = (tile * 32 + n * 4 + ((k & 7) >> 1)) * 2 + (k >> 3);
+        reinterpret_cast<__nv_bfloat16*>(frag)[2 * word + (k & 1)] = __float2bfloat16_rn(w);
+    };
+    if (p < MLP_OFF_B1) {
+        const int k = p / MLP_H, n = p % MLP_H;
+        put(FT_L1 + n / 8, k, n % 8);
+    } else if (p < MLP_OFF_W2) {
+        bias[p - MLP_OFF_B1] = w;
+    } else if (p < MLP_OFF_B2) {
+        const int k = (p - MLP_OFF_W2) / MLP_H, n = (p - MLP_OFF_W2) % MLP_H;
+        put(FT_L2 + (k / 16) * 8 + n / 8, k % 16, n % 8);
+        put(FT_W2T + (n / 16) * 8 + k / 8, n % 16, k % 8);
+    } else if (p < MLP_OFF_W3) {
+        bias[MLP_H + p - MLP_OFF_B2] = w;
+    } else if (p < MLP_OFF_B3) {
+        const int k = p - MLP_OFF_W3;
+        put(FT_L3 + k / 16, k % 16, 0);
+        bias[2 * MLP_H + 2 + k] = w;
+    } else {
+        bias[2 * MLP_H] = w;
+    }
+}
+
+// Sum of the partials in a fixed order -- the four warps of each 128 samples
+// first (PER = 4; PER = 1: the partials are these groups' already), then
+// those sums in order -- and optionally an Adam step
+// (step >= 1) with the packing of the new weights.  A block takes 32
+// parameters; its 8 warps load RED_GROUPS groups of 128 samples at a time
+// (16 loads of a lane in flight), one warp adds them up.  grad_out (nullable)
+// receives the gradient, loss_out the loss.
+constexpr int RED_WARPS = 8, RED_PER_WARP = 4, RED_GROUPS = RED_WARPS * RED_PER_WARP;
+
+template <int PER>
+__global__ void __launch_bounds__(RED_WARPS * 32) mlp_reduce_kernel(const float* __restrict__ partials, int n_part,
+                                                                    float* __restrict__ W, float* __restrict__ m,
+                                                                    float* __restrict__ v, int step, float lr,
+                                                                    float* __restrict__ grad_out,
+                                                                    float* __restrict__ loss_out,
+                                                                    uint32_t* __restrict__ frag,
+                                                                    float* __restrict__ bias) {
+    __shared__ float part[2][RED_GROUPS][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int p = blockIdx.x * 32 + lane;
+    const bool mine = p <= MLP_NPARAM;
+    const int n_groups = (n_part + PER - 1) / PER;
+    pdl_wait_previous();
+    // the optimiser's state is needed only after the sum: in flight with the partials
+    float w0 = 0.f, m0 = 0.f, v0 = 0.f;
+    if (warp == 0 && step > 0 && p < MLP_NPARAM) {
+        w0 = W[p];
+        m0 = m[p];
+        v0 = v[p];
+    }
     float gsum = 0.f;
-    for (int b = 0; b < n_blocks; ++b) gsum += partials[(size_t)b * (MLP_NPARAM + 1) + p];
+    for (int g0 = 0, buf = 0; g0 < n_groups; g0 += RED_GROUPS, buf ^= 1) {
+        float u[RED_PER_WARP][PER];
+#pragma unroll
+        for (int i = 0; i < RED_PER_WARP; ++i) {
+            const int gr = g0 + warp + RED_WARPS * i;
+#pragma unroll
+            for (int j = 0; j < PER; ++j)
+                u[i][j] = mine && PER * gr + j < n_part ? __ldcg(partials + (size_t)(PER * gr + j) * MLP_PART + p) : 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < RED_PER_WARP; ++i) {
+            float sum = 0.f;
+#pragma unroll
+            for (int j = 0; j < PER; ++j) sum += u[i][j];
+            part[buf][warp + RED_WARPS * i][lane] = sum;
+        }
+        __syncthreads();   // the other buffer is free once every warp has passed here
+        if (warp == 0) {
+            const int k = min(RED_GROUPS, n_groups - g0);
+            if (k == RED_GROUPS) {
+#pragma unroll
+                for (int i = 0; i < RED_GROUPS; ++i) gsum += part[buf][i][lane];
+            } else {
+                for (int i = 0; i < k; ++i) gsum += part[buf][i][lane];
+            }
+        }
+    }
+    pdl_launch_next();
+    if (warp != 0 || !mine) return;
     if (p == MLP_NPARAM) {
         if (loss_out) *loss_out = gsum;
         return;
@@ -383,13 +567,15 @@ __global__ void mlp_reduce_kernel(const float* __restrict__ partials, int n_bloc
     if (grad_out) grad_out[p] = gsum;
     if (step > 0) {
         const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-        const float mm = b1 * m[p] + (1.f - b1) * gsum;
-        const float vv = b2 * v[p] + (1.f - b2) * gsum * gsum;
+        const float mm = b1 * m0 + (1.f - b1) * gsum;
+        const float vv = b2 * v0 + (1.f - b2) * gsum * gsum;
         m[p] = mm;
         v[p] = vv;
         const float mh = mm / (1.f - powf(b1, float(step)));
         const float vh = vv / (1.f - powf(b2, float(step)));
-        W[p] -= lr * mh / (sqrtf(vh) + eps);
+        const float w = w0 - lr * mh / (sqrtf(vh) + eps);
+        W[p] = w;
+        pack_param(p, w, frag, bias);
     }
 }
 
@@ -408,7 +594,7 @@ struct gbp_mlp {
     uint32_t* frag = nullptr;   // packed BF16 fragments
     float* bias = nullptr;      // b1, b2, b3, pad, W3 (FP32)
     float* partials = nullptr;
-    int cap_blocks = 0;
+    int cap_warps = 0;
     float* d_loss = nullptr;
     float* d_grad = nullptr;
     int step = 0;
@@ -424,23 +610,38 @@ gbp_status mlp_pack(gbp_mlp* n) {
 gbp_status mlp_grad(gbp_mlp* n, const float* X, const float* T, const int32_t* idx, int count, int step, float lr,
                     float* grad_out) {
     if (count <= 0) return GBP_EINVAL;
-    const int nb = (count + MLP_BLOCK - 1) / MLP_BLOCK;
-    if (nb > n->cap_blocks) {
+    // a warp per 32 rows while one wave of warps takes them (142 registers
+    // and 15.5 KB a warp: 14 per SM), else a warp per 128
+    const int warps = (count + 31) / 32;
+    const bool grouped = warps > GRAD_WAVE;
+    const int nw = grouped ? (count + 127) / 128 : warps;   // partials; a block each
+    if (nw > n->cap_warps) {
         if (n->partials) cudaFree(n->partials);
         n->partials = nullptr;
-        if (cudaMalloc(reinterpret_cast<void**>(&n->partials), sizeof(float) * (size_t)nb * (MLP_NPARAM + 1)) != cudaSuccess)
+        n->cap_warps = 0;
+        if (cudaMalloc(reinterpret_cast<void**>(&n->partials), sizeof(float) * (size_t)nw * MLP_PART) != cudaSuccess)
             return GBP_ENOMEM;
-        n->cap_blocks = nb;
+        n->cap_warps = nw;
     }
-    const size_t smem = sizeof(GradSmem);
-    if (cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return GBP_ECUDA;
-    mlp_grad_kernel<<<nb, MLP_BLOCK, smem, n->stream>>>(n->frag, n->bias, X, T, idx, count, 1.0f / count, n->partials);
-    mlp_reduce_kernel<<<(MLP_NPARAM + 1 + 255) / 256, 256, 0, n->stream>>>(n->partials, nb, n->W, n->m, n->v, step, lr,
-                                                                           grad_out, n->d_loss);
-    if (cudaGetLastError() != cudaSuccess) return GBP_ECUDA;
-    if (step > 0) return mlp_pack(n);
-    return GBP_OK;
+    // programmatic dependent launch: each kernel's launch overlaps the end of
+    // the one before it, whose results it waits for before it reads anything
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.stream = n->stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cfg.gridDim = dim3(nw);
+    cfg.blockDim = dim3(32);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, grouped ? mlp_grad_kernel<true> : mlp_grad_kernel<false>, (const uint32_t*)n->frag, (const float*)n->bias, X, T, idx,
+                                       count, 1.0f / count, n->partials);
+    cfg.gridDim = dim3((MLP_NPARAM + 1 + 31) / 32);
+    cfg.blockDim = dim3(RED_WARPS * 32);
+    if (e == cudaSuccess)
+        e = cudaLaunchKernelEx(&cfg, grouped ? mlp_reduce_kernel<1> : mlp_reduce_kernel<4>, (const float*)n->partials, nw, n->W, n->m, n->v, step, lr,
+                               grad_out, n->d_loss, n->frag, n->bias);
+    return e == cudaSuccess ? GBP_OK : GBP_ECUDA;
 }
 
 }  // namespace

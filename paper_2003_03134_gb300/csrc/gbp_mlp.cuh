@@ -69,95 +69,11 @@ __device__ __forceinline__ void load_a(const __nv_bfloat16* T, int stride, int r
     a3 = *reinterpret_cast<const uint32_t*>(T + (r0 + g + 8) * stride + c0 + 2 * q + 8);
 }
 
-// Store a 16 x 8 D fragment (after f) as BF16 pairs into a row-major tile.
-template <typename F>
-__device__ __forceinline__ void store_d_bf16(__nv_bfloat16* T, int stride, int r0, int c0, int lane,
-                                             const float (&d)[4], F f) {
-    const int g = lane >> 2, q = lane & 3;
-    *reinterpret_cast<uint32_t*>(T + (r0 + g) * stride + c0 + 2 * q) = pack_bf16(f(d[0], c0 + 2 * q), f(d[1], c0 + 2 * q + 1));
-    *reinterpret_cast<uint32_t*>(T + (r0 + g + 8) * stride + c0 + 2 * q) =
-        pack_bf16(f(d[2], c0 + 2 * q), f(d[3], c0 + 2 * q + 1));
-}
-
 // B fragment of tile `tile` for this lane.
 __device__ __forceinline__ void load_b(const uint32_t* frag, int tile, int lane, uint32_t& b0, uint32_t& b1) {
     const uint2 v = *reinterpret_cast<const uint2*>(frag + (tile * 32 + lane) * 2);
     b0 = v.x;
     b1 = v.y;
-}
-
-// Forward pass of one warp over 32 rows.  X: the 32 x 16 input tile (BF16,
-// stride XS); H: a 32 x 64 scratch tile (stride HS; on return it holds h2).
-// When H1 is given, h1 is also kept there (training).  Returns the output
-// pre-activation z3 of row `lane`.  frag/bias in shared memory; bias =
-// b1 (64), b2 (64), b3 (1).
-__device__ __forceinline__ float mlp_forward_warp(const uint32_t* frag, const float* bias, __nv_bfloat16* X,
-                                                  __nv_bfloat16* H, __nv_bfloat16* H1, int lane) {
-    const int g = lane >> 2, q = lane & 3;
-    (void)g;
-    __nv_bfloat16* L1out = H1 ? H1 : H;
-    // layer 1: h1 = relu(X W1 + b1)
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt) {
-        uint32_t a0, a1, a2, a3;
-        load_a(X, XS, 16 * mt, 0, lane, a0, a1, a2, a3);
-#pragma unroll
-        for (int nt = 0; nt < 8; ++nt) {
-            float d[4] = {0.f, 0.f, 0.f, 0.f};
-            uint32_t b0, b1;
-            load_b(frag, FT_L1 + nt, lane, b0, b1);
-            mma_bf16(d, a0, a1, a2, a3, b0, b1);
-            store_d_bf16(L1out, HS, 16 * mt, 8 * nt, lane, d, [&](float v, int c) { return fmaxf(v + bias[c], 0.f); });
-        }
-    }
-    __syncwarp();
-    // layer 2: h2 = relu(h1 W2 + b2), one 16-row block at a time so that it
-    // can overwrite h1 in place when no separate h1 tile is kept
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt) {
-        uint32_t a[4][4];
-#pragma unroll
-        for (int ks = 0; ks < 4; ++ks) load_a(L1out, HS, 16 * mt, 16 * ks, lane, a[ks][0], a[ks][1], a[ks][2], a[ks][3]);
-        float d[8][4];
-#pragma unroll
-        for (int nt = 0; nt < 8; ++nt) {
-            d[nt][0] = d[nt][1] = d[nt][2] = d[nt][3] = 0.f;
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks) {
-                uint32_t b0, b1;
-                load_b(frag, FT_L2 + ks * 8 + nt, lane, b0, b1);
-                mma_bf16(d[nt], a[ks][0], a[ks][1], a[ks][2], a[ks][3], b0, b1);
-            }
-        }
-        __syncwarp();
-#pragma unroll
-        for (int nt = 0; nt < 8; ++nt)
-            store_d_bf16(H, HS, 16 * mt, 8 * nt, lane, d[nt],
-                         [&](float v, int c) { return fmaxf(v + bias[MLP_H + c], 0.f); });
-    }
-    __syncwarp();
-    // layer 3: z3 = h2 W3 + b3 (W3 in output column 0 of the tile)
-    float* out = reinterpret_cast<float*>(X);   // the input tile is free now
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt) {
-        float d[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int ks = 0; ks < 4; ++ks) {
-            uint32_t a0, a1, a2, a3, b0, b1;
-            load_a(H, HS, 16 * mt, 16 * ks, lane, a0, a1, a2, a3);
-            load_b(frag, FT_L3 + ks, lane, b0, b1);
-            mma_bf16(d, a0, a1, a2, a3, b0, b1);
-        }
-        __syncwarp();
-        if (q == 0) {
-            out[16 * mt + (lane >> 2)] = d[0];
-            out[16 * mt + (lane >> 2) + 8] = d[2];
-        }
-    }
-    __syncwarp();
-    const float z3 = out[lane] + bias[2 * MLP_H];
-    __syncwarp();
-    return z3;
 }
 
 __device__ __forceinline__ float mlp_output(float z3) { return MLP_DMAX / (1.0f + __expf(-z3)); }
@@ -166,9 +82,9 @@ __device__ __forceinline__ float mlp_output(float z3) { return MLP_DMAX / (1.0f 
 // layer (16 x 8 tiles, FP32) are exactly the A fragments of the next layer
 // (16 x 16, BF16 pairs) once packed -- tile 2j supplies columns 0-7 and tile
 // 2j+1 columns 8-15 of k-step j -- so activations never leave registers.
-// Bitwise equal to mlp_forward_warp (same roundings, same mma order).
 // X: the warp's 32 x 16 input tile (BF16, stride XS) in shared memory;
-// frag/bias as for mlp_forward_warp.  Returns z3 of row `lane`.
+// frag/bias (b1 (64), b2 (64), b3 (1)) in shared memory.  Returns the output
+// pre-activation z3 of row `lane`.
 __device__ __forceinline__ float mlp_forward_regs(const uint32_t* frag, const float* bias, const __nv_bfloat16* X,
                                                   int lane) {
     const int g = lane >> 2, q = lane & 3;
