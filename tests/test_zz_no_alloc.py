@@ -106,3 +106,54 @@ def test_noalloc_empty_input(torch):
     p.obs_kf, p.obs_lm, p.obs_uv = p.obs_kf[:0], p.obs_lm[:0], p.obs_uv[:0]
     out = _DeviceInputs(torch, p, p.kf_Rt_init, p.lm_init).call(torch, torch.cuda.current_stream().cuda_stream)
     np.testing.assert_array_equal(out, [0.0, 0.0])
+
+
+@pytest.mark.parametrize("n", [1, 31, 255, 257, 1216 * 256 - 1, 1216 * 256 + 3, gbp.GBP_NOALLOC_MAX_OBS])
+@pytest.mark.parametrize("scale", [1.0, 1e-70, 1e140])
+def test_noalloc_matches_numpy(torch, n, scale):
+    """Sizes around a block and around one pass of all blocks; scenes scaled so that the squared quantities leave the
+    exponent range (the division path) and exact zero residuals among the rest.  Each error carries a handful of
+    roundings of relative size 2^-53, some amplified by |uv| / |residual| (typical ratio below 1e3 here, averaged over
+    n): 1e-11 relative."""
+    rng = np.random.default_rng(n)
+    n_kf, n_lm = 7, 50
+    R = np.stack([np.linalg.qr(rng.normal(size=(3, 3)))[0] for _ in range(n_kf)])
+    t = rng.normal(size=(n_kf, 3)) + [0, 0, 6.0]
+    X = rng.uniform(-1, 1, (n_lm, 3))
+    kf = np.concatenate([R.reshape(-1, 9), scale * t], 1)
+    lm = scale * X
+    ok, ol = rng.integers(0, n_kf, n).astype(np.int32), rng.integers(0, n_lm, n).astype(np.int32)
+    p = np.einsum("nij,nj->ni", R[ok], lm[ol]) + scale * t[ok]
+    h = np.stack([500 * p[:, 0] / p[:, 2] + 320, 500 * p[:, 1] / p[:, 2] + 240], 1)
+    uv = h + rng.normal(0, 3, (n, 2))
+    lm[0], ol[::5] = 0.0, 0            # projects to (500 tx/tz + 320, ...) exactly the same way for every view
+    p = np.einsum("nij,nj->ni", R[ok], lm[ol]) + scale * t[ok]
+    err = np.linalg.norm(uv - np.stack([500 * p[:, 0] / p[:, 2] + 320, 500 * p[:, 1] / p[:, 2] + 240], 1), axis=1)
+    dev = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (kf, lm, ok, ol, uv)]
+    out = torch.full((2,), -1.0, dtype=torch.float64, device="cuda")
+    gbp.gbp_reprojection_error_noalloc((500.0, 500.0, 320.0, 240.0, 640, 480), scale, n_kf, dev[0].data_ptr(), n_lm,
+                                       dev[1].data_ptr(), n, dev[2].data_ptr(), dev[3].data_ptr(), dev[4].data_ptr(),
+                                       out.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    are, count = out.cpu().numpy()
+    assert count == n
+    assert abs(are - err.mean()) <= 1e-11 * err.mean(), (are, err.mean())
+
+
+def test_noalloc_infinite_and_exact_observations(torch):
+    """A zero residual counts as 0; an infinite pixel makes the average infinite; a NaN depth is left out."""
+    kf = torch.tensor([[1, 0, 0, 0, 1, 0, 0, 0, 1, 0, 0, 0.0]], dtype=torch.float64, device="cuda")
+    lm = torch.tensor([[0, 0, 2.0], [1, 1, float("nan")]], dtype=torch.float64, device="cuda")
+    idx = torch.zeros(2, dtype=torch.int32, device="cuda")
+    uv = torch.tensor([[320.0, 240.0], [320.0, 240.0]], dtype=torch.float64, device="cuda")
+    out = torch.zeros(2, dtype=torch.float64, device="cuda")
+
+    def call(ol):
+        gbp.gbp_reprojection_error_noalloc((500.0, 500.0, 320.0, 240.0, 640, 480), 0.05, 1, kf.data_ptr(), 2,
+                                           lm.data_ptr(), 2, idx.data_ptr(), ol.data_ptr(), uv.data_ptr(),
+                                           out.data_ptr(), torch.cuda.current_stream().cuda_stream)
+        return out.cpu().tolist()
+
+    assert call(idx) == [0.0, 2.0]
+    assert call(torch.tensor([0, 1], dtype=torch.int32, device="cuda")) == [0.0, 1.0]
+    uv[1, 0] = float("inf")
+    assert call(idx) == [float("inf"), 2.0]
