@@ -2226,78 +2226,98 @@ __global__ void prior_reduce_kernel(DevGraph<R> g, const R* tmp_k, const R* tmp_
 // metrics: average reprojection error (Sec. 9.1) at the current means, its
 // distance to reference projections, Huber-regime count.  Two-pass fixed
 // order reduction through per-block partials.
+//
+// Bound: the FP64 pipe (a warp instruction per 16 cycles and SM).  The
+// references come rounded to R from the host (kf_Rr, f_dlc: the same roundings
+// as rounding them here), counts are integers, and what is left in FP64 per
+// factor is the square root of |r|^2 and the sum.  900k factors: 61 -> 34 us
+// (metrics_kernel), and 192 -> 5 us for the final sum by a block instead of
+// one thread.
+
+// |z - h(mu)|^2 of factor f at the current means; false where the point is
+// closer than z_min to its camera.
+template <typename R>
+__device__ __forceinline__ bool error2_at_means(const DevGraph<R>& g, const KParams<R>& P, int f, R zu, R zv, R& r2) {
+    const size_t n_f = g.n_f;
+    const int k = g.fk[f], m = g.fm[f];
+    const R* kb = g.kf_bel + (size_t)k * KBEL;
+    const R* lb = g.lm_bel + (size_t)m * LBEL;
+    const R x[9] = {kb[KB_MU], kb[KB_MU + 1], kb[KB_MU + 2], kb[KB_MU + 3], kb[KB_MU + 4], kb[KB_MU + 5],
+                    lb[9], lb[10], lb[11]};
+    KParams<R> Q = P;
+    Q.huber_n = R(0);
+    Lin<R> L;
+    const R dlc[3] = {g.f_dlc[f], g.f_dlc[n_f + f], g.f_dlc[2 * n_f + f]};
+    R Rr[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) Rr[i] = g.kf_Rr[(size_t)k * 9 + i];
+    linearise_ref<R>(Q, Rr, dlc, x, zu, zv, L);
+    r2 = L.r2;
+    return L.W > R(0);
+}
+
+// Sums of a block: one double (tree over the threads) and up to three counts.
+template <int NC>
+__device__ __forceinline__ double block_metrics(double v, int (&n)[NC]) {
+    __shared__ double red[METRIC_BLOCK];
+    __shared__ int cnt[NC];
+    const int tid = threadIdx.x;
+    red[tid] = v;
+    if (tid < NC) cnt[tid] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < NC; ++j) {
+        n[j] = __reduce_add_sync(0xffffffffu, n[j]);
+        if ((tid & 31) == 0 && n[j]) atomicAdd(&cnt[j], n[j]);
+    }
+    for (int st = METRIC_BLOCK / 2; st > 0; st >>= 1) {
+        if (tid < st) red[tid] += red[tid + st];
+        __syncthreads();
+    }
+#pragma unroll
+    for (int j = 0; j < NC; ++j) n[j] = cnt[j];
+    return red[0];
+}
 
 template <typename R>
 __global__ void __launch_bounds__(METRIC_BLOCK) metrics_kernel(DevGraph<R> g, KParams<R> P, double* partials) {
-    __shared__ double red[4][METRIC_BLOCK];
-    const int tid = threadIdx.x;
-    double v[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int f = blockIdx.x * METRIC_BLOCK + tid; f < g.n_f; f += gridDim.x * METRIC_BLOCK) {
-        const int k = g.fk[f], m = g.fm[f];
-        const R* kb = g.kf_bel + (size_t)k * KBEL;
-        const R* lb = g.lm_bel + (size_t)m * LBEL;
-        R x[9] = {kb[KB_MU], kb[KB_MU + 1], kb[KB_MU + 2], kb[KB_MU + 3], kb[KB_MU + 4], kb[KB_MU + 5],
-                   lb[9], lb[10], lb[11]};
-        KParams<R> Q = P;
-        Q.huber_n = R(0);
-        Lin<R> L;
-        linearise<R>(Q, g.kf_R + (size_t)k * 9, g.kf_c + (size_t)k * 3, g.lm_ref + (size_t)m * 3, x,
-                     g.z[2 * (size_t)f], g.z[2 * (size_t)f + 1], L);
-        if (L.W > R(0)) {
-            double e = sqrt(double(L.r2));
-            v[0] += e;
-            v[2] += 1.0;
-            if (P.huber_n > R(0) && e * double(P.inv_sigma) > double(P.huber_n)) v[3] += 1.0;
+    double v = 0.0;
+    int n[2] = {0, 0};   // counted, in the Huber regime
+    for (int f = blockIdx.x * METRIC_BLOCK + threadIdx.x; f < g.n_f; f += gridDim.x * METRIC_BLOCK) {
+        R r2;
+        if (error2_at_means<R>(g, P, f, g.z[2 * (size_t)f], g.z[2 * (size_t)f + 1], r2)) {
+            const double e = sqrt(double(r2));
+            v += e;
+            ++n[0];
+            if (P.huber_n > R(0) && e * double(P.inv_sigma) > double(P.huber_n)) ++n[1];
         }
     }
-    for (int j = 0; j < 4; ++j) red[j][tid] = v[j];
-    __syncthreads();
-    for (int st = METRIC_BLOCK / 2; st > 0; st >>= 1) {
-        if (tid < st)
-            for (int j = 0; j < 4; ++j) red[j][tid] += red[j][tid + st];
-        __syncthreads();
+    const double s = block_metrics<2>(v, n);
+    if (threadIdx.x == 0) {
+        partials[blockIdx.x] = s;
+        partials[2 * (size_t)gridDim.x + blockIdx.x] = double(n[0]);
+        partials[3 * (size_t)gridDim.x + blockIdx.x] = double(n[1]);
     }
-    if (tid == 0)
-        for (int j = 0; j < 4; ++j) partials[(size_t)j * gridDim.x + blockIdx.x] = red[j][0];
 }
 
 // reference-projection distance needs the residual vector, not only |r|:
-// recompute h(mu) per factor
+// recompute h(mu) per factor (with z = reference pixel the residual is ref - h(mu))
 template <typename R>
 __global__ void __launch_bounds__(METRIC_BLOCK) metrics_ref_kernel(DevGraph<R> g, KParams<R> P, double* partials) {
-    __shared__ double red[2][METRIC_BLOCK];
-    const int tid = threadIdx.x;
-    double acc = 0.0, cnt = 0.0;
-    for (int f = blockIdx.x * METRIC_BLOCK + tid; f < g.n_f; f += gridDim.x * METRIC_BLOCK) {
-        const int k = g.fk[f], m = g.fm[f];
-        const R* kb = g.kf_bel + (size_t)k * KBEL;
-        const R* lb = g.lm_bel + (size_t)m * LBEL;
-        R x[9] = {kb[KB_MU], kb[KB_MU + 1], kb[KB_MU + 2], kb[KB_MU + 3], kb[KB_MU + 4], kb[KB_MU + 5],
-                   lb[9], lb[10], lb[11]};
-        KParams<R> Q = P;
-        Q.huber_n = R(0);
-        Lin<R> L;
-        // with z = reference pixel the residual is ref - h(mu)
-        R ru = g.uv_ref[2 * (size_t)f], rv = g.uv_ref[2 * (size_t)f + 1];
-        linearise<R>(Q, g.kf_R + (size_t)k * 9, g.kf_c + (size_t)k * 3, g.lm_ref + (size_t)m * 3, x, ru, rv, L);
-        if (L.W > R(0) && isfinite(ru)) {
-            acc += sqrt(double(L.r2));
-            cnt += 1.0;
+    double v = 0.0;
+    int n[1] = {0};
+    for (int f = blockIdx.x * METRIC_BLOCK + threadIdx.x; f < g.n_f; f += gridDim.x * METRIC_BLOCK) {
+        const R ru = g.uv_ref[2 * (size_t)f], rv = g.uv_ref[2 * (size_t)f + 1];
+        R r2;
+        if (error2_at_means<R>(g, P, f, ru, rv, r2) && isfinite(ru)) {
+            v += sqrt(double(r2));
+            ++n[0];
         }
     }
-    red[0][tid] = acc;
-    red[1][tid] = cnt;
-    __syncthreads();
-    for (int st = METRIC_BLOCK / 2; st > 0; st >>= 1) {
-        if (tid < st) {
-            red[0][tid] += red[0][tid + st];
-            red[1][tid] += red[1][tid + st];
-        }
-        __syncthreads();
-    }
-    if (tid == 0) {
-        partials[(size_t)4 * gridDim.x + blockIdx.x] = red[0][0];
-        partials[(size_t)5 * gridDim.x + blockIdx.x] = red[1][0];
+    const double s = block_metrics<1>(v, n);
+    if (threadIdx.x == 0) {
+        partials[4 * (size_t)gridDim.x + blockIdx.x] = s;
+        partials[5 * (size_t)gridDim.x + blockIdx.x] = double(n[0]);
     }
 }
 
@@ -2307,36 +2327,24 @@ __global__ void __launch_bounds__(METRIC_BLOCK) metrics_ref_kernel(DevGraph<R> g
 template <typename R>
 __global__ void __launch_bounds__(METRIC_BLOCK) problem_metrics_kernel(DevGraph<R> g, KParams<R> P,
                                                                        const int32_t* prob_f0, double* out) {
-    __shared__ double red[3][METRIC_BLOCK];
-    const int tid = threadIdx.x, p = blockIdx.x;
-    double v[3] = {0.0, 0.0, 0.0};
-    for (int f = prob_f0[p] + tid; f < prob_f0[p + 1]; f += METRIC_BLOCK) {
-        const int k = g.fk[f], m = g.fm[f];
-        const R* kb = g.kf_bel + (size_t)k * KBEL;
-        const R* lb = g.lm_bel + (size_t)m * LBEL;
-        R x[9] = {kb[KB_MU], kb[KB_MU + 1], kb[KB_MU + 2], kb[KB_MU + 3], kb[KB_MU + 4], kb[KB_MU + 5],
-                   lb[9], lb[10], lb[11]};
-        KParams<R> Q = P;
-        Q.huber_n = R(0);
-        Lin<R> L;
-        linearise<R>(Q, g.kf_R + (size_t)k * 9, g.kf_c + (size_t)k * 3, g.lm_ref + (size_t)m * 3, x,
-                     g.z[2 * (size_t)f], g.z[2 * (size_t)f + 1], L);
-        if (L.W > R(0)) {
-            double e = sqrt(double(L.r2));
-            v[0] += e;
-            v[1] += 1.0;
-            if (P.huber_n > R(0) && e * double(P.inv_sigma) > double(P.huber_n)) v[2] += 1.0;
+    const int p = blockIdx.x;
+    double v = 0.0;
+    int n[2] = {0, 0};
+    for (int f = prob_f0[p] + threadIdx.x; f < prob_f0[p + 1]; f += METRIC_BLOCK) {
+        R r2;
+        if (error2_at_means<R>(g, P, f, g.z[2 * (size_t)f], g.z[2 * (size_t)f + 1], r2)) {
+            const double e = sqrt(double(r2));
+            v += e;
+            ++n[0];
+            if (P.huber_n > R(0) && e * double(P.inv_sigma) > double(P.huber_n)) ++n[1];
         }
     }
-    for (int j = 0; j < 3; ++j) red[j][tid] = v[j];
-    __syncthreads();
-    for (int st = METRIC_BLOCK / 2; st > 0; st >>= 1) {
-        if (tid < st)
-            for (int j = 0; j < 3; ++j) red[j][tid] += red[j][tid + st];
-        __syncthreads();
+    const double s = block_metrics<2>(v, n);
+    if (threadIdx.x == 0) {
+        out[3 * (size_t)p] = s;
+        out[3 * (size_t)p + 1] = double(n[0]);
+        out[3 * (size_t)p + 2] = double(n[1]);
     }
-    if (tid == 0)
-        for (int j = 0; j < 3; ++j) out[3 * (size_t)p + j] = red[j][0];
 }
 
 // Per-factor reprojection error |z - h(mu)| at the current means (Sec. 9.1),
@@ -2345,30 +2353,34 @@ template <typename R>
 __global__ void __launch_bounds__(METRIC_BLOCK) residual_kernel(DevGraph<R> g, KParams<R> P, double* out) {
     const int f = blockIdx.x * METRIC_BLOCK + threadIdx.x;
     if (f >= g.n_f) return;
-    const int k = g.fk[f], m = g.fm[f];
-    const R* kb = g.kf_bel + (size_t)k * KBEL;
-    const R* lb = g.lm_bel + (size_t)m * LBEL;
-    R x[9] = {kb[KB_MU], kb[KB_MU + 1], kb[KB_MU + 2], kb[KB_MU + 3], kb[KB_MU + 4], kb[KB_MU + 5],
-              lb[9], lb[10], lb[11]};
-    KParams<R> Q = P;
-    Q.huber_n = R(0);
-    Lin<R> L;
-    linearise<R>(Q, g.kf_R + (size_t)k * 9, g.kf_c + (size_t)k * 3, g.lm_ref + (size_t)m * 3, x,
-                 g.z[2 * (size_t)f], g.z[2 * (size_t)f + 1], L);
-    out[f] = L.W > R(0) ? sqrt(double(L.r2)) : -1.0;
+    R r2;
+    const bool ok = error2_at_means<R>(g, P, f, g.z[2 * (size_t)f], g.z[2 * (size_t)f + 1], r2);
+    out[f] = ok ? sqrt(double(r2)) : -1.0;
 }
 
-__global__ void metrics_finish_kernel(const double* partials, int nb, int with_ref, double* out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double s[6] = {0, 0, 0, 0, 0, 0};
-    for (int j = 0; j < 6; ++j) {
-        if (j >= 4 && !with_ref) break;
-        for (int b = 0; b < nb; ++b) s[j] += partials[(size_t)j * nb + b];
+// The blocks' partials added up by one block, in a fixed order (a thread's
+// own in block order, then a tree).
+__global__ void __launch_bounds__(METRIC_BLOCK) metrics_finish_kernel(const double* partials, int nb, int with_ref,
+                                                                      double* out) {
+    __shared__ double red[6][METRIC_BLOCK];
+    const int tid = threadIdx.x, rows = with_ref ? 6 : 4;   // rows: error, -, counted, Huber, ref error, ref counted
+    for (int j = 0; j < rows; ++j) {
+        double s = 0.0;
+        if (j != 1)
+            for (int b = tid; b < nb; b += METRIC_BLOCK) s += partials[(size_t)j * nb + b];
+        red[j][tid] = s;
     }
-    out[MET_N_ARE] = s[2];
-    out[MET_ARE] = s[2] > 0 ? s[0] / s[2] : 0.0;
-    out[MET_HUBER] = s[3];
-    out[MET_ARE_REF] = with_ref ? (s[5] > 0 ? s[4] / s[5] : 0.0) : -1.0;
+    __syncthreads();
+    for (int st = METRIC_BLOCK / 2; st > 0; st >>= 1) {
+        if (tid < st)
+            for (int j = 0; j < rows; ++j) red[j][tid] += red[j][tid + st];
+        __syncthreads();
+    }
+    if (tid != 0) return;
+    out[MET_N_ARE] = red[2][0];
+    out[MET_ARE] = red[2][0] > 0 ? red[0][0] / red[2][0] : 0.0;
+    out[MET_HUBER] = red[3][0];
+    out[MET_ARE_REF] = with_ref ? (red[5][0] > 0 ? red[4][0] / red[5][0] : 0.0) : -1.0;
 }
 
 // ------------------------------------------------------------------------
@@ -2527,7 +2539,7 @@ cudaError_t launch_metrics(const DevGraph<R>& g, const KParams<R>& p, double* pa
                            cudaStream_t s) {
     metrics_kernel<R><<<nb, METRIC_BLOCK, 0, s>>>(g, p, partials);
     if (g.uv_ref) metrics_ref_kernel<R><<<nb, METRIC_BLOCK, 0, s>>>(g, p, partials);
-    metrics_finish_kernel<<<1, 32, 0, s>>>(partials, nb, g.uv_ref != nullptr, out);
+    metrics_finish_kernel<<<1, METRIC_BLOCK, 0, s>>>(partials, nb, g.uv_ref != nullptr, out);
     return cudaGetLastError();
 }
 
