@@ -220,6 +220,15 @@ struct gbp_graph {
     uint32_t* mlp_frag = nullptr;
     float* mlp_bias = nullptr;
     bool has_model = false;
+    // device buffers of what the caller reads back (means, residuals,
+    // per-problem statistics), kept between calls, and the caller's
+    // observation index of each factor
+    double* h_read = nullptr;                   // pinned, SMALL_READ doubles
+    void* d_read = nullptr;
+    size_t read_cap = 0;
+    int32_t* d_obs = nullptr;
+    size_t obs_cap = 0;
+    bool obs_current = false;
 };
 
 namespace {
@@ -764,9 +773,40 @@ float last_dmu(const gbp_graph* g) {
     return v;
 }
 
-gbp_status read_ctl(gbp_graph* g) {
-    CK(cudaMemcpyAsync(g->h_ctl, g->ctl, sizeof(int32_t) * CTL_N, cudaMemcpyDeviceToHost, g->stream));
-    CK(cudaStreamSynchronize(g->stream));
+// The read-back buffer, at least n doubles.
+gbp_status read_buffer(gbp_graph* g, size_t n, double** out) {
+    const size_t bytes = sizeof(double) * std::max<size_t>(n, 1);
+    if (bytes > g->read_cap) {
+        if (g->d_read) cudaFree(g->d_read);
+        g->d_read = nullptr;
+        g->read_cap = 0;
+        const size_t want = size_t(double(bytes) * g->headroom);
+        CK(cudaMalloc(&g->d_read, want));
+        g->read_cap = want;
+    }
+    *out = static_cast<double*>(g->d_read);
+    return GBP_OK;
+}
+
+// The caller's observation index of each internal factor, on the device.
+gbp_status upload_obs_index(gbp_graph* g) {
+    if (g->obs_current) return GBP_OK;
+    const size_t n = g->obs_index.size();
+    if (n > g->obs_cap) {
+        if (g->d_obs) cudaFree(g->d_obs);
+        g->d_obs = nullptr;
+        g->obs_cap = 0;
+        const size_t want = size_t(double(n) * g->headroom) + 1;
+        CK(dev_alloc(&g->d_obs, want));
+        g->obs_cap = want;
+    }
+    CK(cudaMemcpyAsync(g->d_obs, g->obs_index.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, g->stream));
+    g->obs_current = true;
+    return GBP_OK;
+}
+
+// The status that the mirrored control block reports.
+gbp_status ctl_status(gbp_graph* g) {
     if (g->h_ctl[CTL_ERR] == 2)
         return fail(g, GBP_ETIMEOUT, "grid barrier wait exceeded its limit (blocks not co-resident?)");
     if (g->h_ctl[CTL_ERR]) {
@@ -776,6 +816,46 @@ gbp_status read_ctl(gbp_graph* g) {
         return fail(g, GBP_EDIVERGED, buf);
     }
     return GBP_OK;
+}
+
+gbp_status read_ctl(gbp_graph* g) {
+    CK(cudaMemcpyAsync(g->h_ctl, g->ctl, sizeof(int32_t) * CTL_N, cudaMemcpyDeviceToHost, g->stream));
+    CK(cudaStreamSynchronize(g->stream));
+    return ctl_status(g);
+}
+
+// The means, converted on the device, into the caller's arrays (chart: 6 per
+// keyframe, world: 12; 3 per point), and the control block's status.  Up to
+// SMALL_READ doubles the kernel writes into pinned host memory and the host
+// copies them on (one launch and one wait: a paper-scale read is all
+// latency); more are copied straight to the caller's pageable arrays, which
+// on this machine's coherent link runs at the rate of pinned ones (4.8 MB:
+// 37 us, where a host copy out of pinned memory takes 160).  Synchronises.
+constexpr size_t SMALL_READ = 16384;
+
+gbp_status download_means(gbp_graph* g, bool world, double* kf, double* lm) {
+    const size_t nk = (size_t)g->n_kf * (world ? 12 : 6), nl = 3 * (size_t)g->n_lm;
+    const bool small = nk + nl <= SMALL_READ;
+    double* d = nullptr;
+    if (small) {
+        if (!g->h_read) CK(cudaMallocHost(reinterpret_cast<void**>(&g->h_read), sizeof(double) * SMALL_READ));
+        d = g->h_read;
+    } else {
+        gbp_status st = read_buffer(g, nk + nl, &d);
+        if (st != GBP_OK) return st;
+    }
+    CK(g->storage ? launch_means<double>(g->sd.g, world, d, d + nk, g->h_ctl, g->stream)
+                  : launch_means<float>(g->sf.g, world, d, d + nk, g->h_ctl, g->stream));
+    if (!small) {
+        if (nk) CK(cudaMemcpyAsync(kf, d, sizeof(double) * nk, cudaMemcpyDeviceToHost, g->stream));
+        if (nl) CK(cudaMemcpyAsync(lm, d + nk, sizeof(double) * nl, cudaMemcpyDeviceToHost, g->stream));
+    }
+    CK(cudaStreamSynchronize(g->stream));
+    if (small) {
+        std::copy(d, d + nk, kf);
+        std::copy(d + nk, d + nk + nl, lm);
+    }
+    return ctl_status(g);
 }
 
 bool finite_all(const double* p, size_t n) {
@@ -1056,6 +1136,7 @@ void order_factors_append(gbp_graph* g, int L1, int K0, int n_obs, const int32_t
     g->fm.swap(fm);
     g->z.swap(z);
     g->obs_index.swap(oi);
+    g->obs_current = false;
     g->f_of_obs.assign(F1, 0);
     for (int q = 0; q < F1; ++q) g->f_of_obs[g->obs_index[q]] = q;
 }
@@ -1429,14 +1510,14 @@ gbp_status gbp_get_problem_are(const gbp_graph* cg, double* are, int32_t* n_are,
     const int np = (int)g->prob_kf0.size() - 1;
     if (np == 0) return GBP_OK;
     double* d_out = nullptr;
-    CK(cudaMalloc(reinterpret_cast<void**>(&d_out), sizeof(double) * 3 * np));
+    const gbp_status bst = read_buffer(g, 3 * (size_t)np, &d_out);
+    if (bst != GBP_OK) return bst;
     cudaError_t e = g->storage
         ? launch_problem_metrics<double>(g->sd.g, make_kparams<double>(g), g->d_prob_f0, np, d_out, g->stream)
         : launch_problem_metrics<float>(g->sf.g, make_kparams<float>(g), g->d_prob_f0, np, d_out, g->stream);
     std::vector<double> h(3 * (size_t)np);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h.data(), d_out, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, g->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
-    cudaFree(d_out);
     if (e != cudaSuccess) return cuda_fail(g, e, "problem metrics");
     for (int p = 0; p < np; ++p) {
         are[p] = h[3 * p + 1] > 0 ? h[3 * p] / h[3 * p + 1] : 0.0;
@@ -1562,43 +1643,25 @@ gbp_status gbp_iterate(gbp_graph* g, int32_t n_iters, int32_t* iters_done) {
 gbp_status gbp_get_means(const gbp_graph* cg, double* kf_mu, double* lm_mu) {
     gbp_graph* g = const_cast<gbp_graph*>(cg);
     if (!g || (g->n_kf && !kf_mu) || (g->n_lm && !lm_mu)) return GBP_EINVAL;
-    std::vector<double> kb, lb;
-    gbp_status st = download_beliefs(g, kb, lb);
-    if (st != GBP_OK) return st;
-    for (int v = 0; v < g->n_kf; ++v)
-        for (int i = 0; i < 6; ++i) kf_mu[6 * v + i] = kb[(size_t)KBEL * v + KB_MU + i];
-    for (int v = 0; v < g->n_lm; ++v)
-        for (int i = 0; i < 3; ++i) lm_mu[3 * v + i] = lb[(size_t)LBEL * v + 9 + i];
-    return read_ctl(g);
+    return download_means(g, false, kf_mu, lm_mu);
 }
 
 gbp_status gbp_get_beliefs(const gbp_graph* cg, double* kf_Rt, double* lm_xyz, double* kf_cov, double* lm_cov) {
     gbp_graph* g = const_cast<gbp_graph*>(cg);
     if (!g || (g->n_kf && !kf_Rt) || (g->n_lm && !lm_xyz)) return GBP_EINVAL;
-    std::vector<double> kb, lb;
-    gbp_status st = download_beliefs(g, kb, lb);
-    if (st != GBP_OK) return st;
-    for (int v = 0; v < g->n_kf; ++v) {
-        const double* mu = &kb[(size_t)KBEL * v + KB_MU];
-        double E[9], R[9], c[3];
-        so3_exp_host(mu + 3, E);
-        const double* Rr = &g->kf_R[9 * (size_t)v];
-        for (int i = 0; i < 3; ++i)
-            for (int j = 0; j < 3; ++j)
-                R[3 * i + j] = E[3 * i] * Rr[j] + E[3 * i + 1] * Rr[3 + j] + E[3 * i + 2] * Rr[6 + j];
-        for (int i = 0; i < 3; ++i) c[i] = g->kf_c[3 * v + i] + mu[i];
-        double* o = kf_Rt + 12 * (size_t)v;
-        for (int i = 0; i < 9; ++i) o[i] = R[i];
-        for (int i = 0; i < 3; ++i) o[9 + i] = -(R[3 * i] * c[0] + R[3 * i + 1] * c[1] + R[3 * i + 2] * c[2]);
-        if (kf_cov && !packed_inverse(6, &kb[(size_t)KBEL * v + KB_LAM], kf_cov + 36 * (size_t)v))
-            return fail(g, GBP_EDIVERGED, "keyframe belief not positive definite");
+    const gbp_status st = download_means(g, true, kf_Rt, lm_xyz);
+    if (kf_cov || lm_cov) {
+        std::vector<double> kb, lb;
+        const gbp_status dst = download_beliefs(g, kb, lb);
+        if (dst != GBP_OK) return dst;
+        for (int v = 0; kf_cov && v < g->n_kf; ++v)
+            if (!packed_inverse(6, &kb[(size_t)KBEL * v + KB_LAM], kf_cov + 36 * (size_t)v))
+                return fail(g, GBP_EDIVERGED, "keyframe belief not positive definite");
+        for (int v = 0; lm_cov && v < g->n_lm; ++v)
+            if (!packed_inverse(3, &lb[(size_t)LBEL * v], lm_cov + 9 * (size_t)v))
+                return fail(g, GBP_EDIVERGED, "landmark belief not positive definite");
     }
-    for (int v = 0; v < g->n_lm; ++v) {
-        for (int i = 0; i < 3; ++i) lm_xyz[3 * v + i] = g->lm_ref[3 * v + i] + lb[(size_t)LBEL * v + 9 + i];
-        if (lm_cov && !packed_inverse(3, &lb[(size_t)LBEL * v], lm_cov + 9 * (size_t)v))
-            return fail(g, GBP_EDIVERGED, "landmark belief not positive definite");
-    }
-    return read_ctl(g);
+    return st;
 }
 
 gbp_status gbp_set_reference(gbp_graph* g, const double* ref_kf_Rt, const double* ref_lm) {
@@ -1681,16 +1744,13 @@ gbp_status gbp_get_residuals(const gbp_graph* cg, double* err) {
     if (!g || (g->n_f && !err)) return GBP_EINVAL;
     if (g->n_f == 0) return GBP_OK;
     double* d = nullptr;
-    CK(cudaMalloc(reinterpret_cast<void**>(&d), sizeof(double) * g->n_f));
-    cudaError_t e = g->storage ? launch_residuals<double>(g->sd.g, make_kparams<double>(g), d, g->stream)
-                               : launch_residuals<float>(g->sf.g, make_kparams<float>(g), d, g->stream);
-    std::vector<double> h(g->n_f);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h.data(), d, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, g->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
-    cudaFree(d);
-    if (e != cudaSuccess) return cuda_fail(g, e, "residuals");
-    for (int f = 0; f < g->n_f; ++f) err[g->obs_index[f]] = h[f];
-    return read_ctl(g);
+    gbp_status st = read_buffer(g, (size_t)g->n_f, &d);
+    if (st == GBP_OK) st = upload_obs_index(g);
+    if (st != GBP_OK) return st;
+    CK(g->storage ? launch_residuals<double>(g->sd.g, make_kparams<double>(g), g->d_obs, d, g->stream)
+                  : launch_residuals<float>(g->sf.g, make_kparams<float>(g), g->d_obs, d, g->stream));
+    CK(cudaMemcpyAsync(err, d, sizeof(double) * (size_t)g->n_f, cudaMemcpyDeviceToHost, g->stream));
+    return read_ctl(g);   // synchronises
 }
 
 gbp_status gbp_get_sizes(const gbp_graph* g, int32_t* n_kf, int32_t* n_lm, int32_t* n_obs) {
@@ -2010,6 +2070,9 @@ void gbp_destroy_graph(gbp_graph* g) {
     if (g->d_prob_f0) cudaFree(g->d_prob_f0);
     if (g->h_ctl) cudaFreeHost(g->h_ctl);
     if (g->h_met) cudaFreeHost(g->h_met);
+    if (g->h_read) cudaFreeHost(g->h_read);
+    if (g->d_read) cudaFree(g->d_read);
+    if (g->d_obs) cudaFree(g->d_obs);
     if (g->capture) cudaStreamDestroy(g->capture);
     if (g->mlp_frag) cudaFree(g->mlp_frag);
     if (g->mlp_bias) cudaFree(g->mlp_bias);

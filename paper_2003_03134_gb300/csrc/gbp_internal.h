@@ -240,8 +240,13 @@ template <typename R> cudaError_t launch_metrics(const DevGraph<R>& g, const KPa
 template <typename R> cudaError_t launch_problem_metrics(const DevGraph<R>& g, const KParams<R>& p,
                                                          const int32_t* prob_f0, int n_problems, double* out,
                                                          cudaStream_t s);
-template <typename R> cudaError_t launch_residuals(const DevGraph<R>& g, const KParams<R>& p, double* out,
-                                                   cudaStream_t s);
+// err of every factor, to out[obs_index[f]]
+template <typename R> cudaError_t launch_residuals(const DevGraph<R>& g, const KParams<R>& p, const int32_t* obs_index,
+                                                   double* out, cudaStream_t s);
+// the means in double: chart (n_kf x 6, n_lm x 3) or world (n_kf x 12, n_lm x 3); ctl_out
+// (nullable): a copy of the control block
+template <typename R> cudaError_t launch_means(const DevGraph<R>& g, bool world, double* kf, double* lm,
+                                               int32_t* ctl_out, cudaStream_t s);
 template <typename R> cudaError_t launch_split_records(const DevGraph<R>& g, int kind, int put, int n,
                                                        const int32_t* idx, float* io, cudaStream_t s);
 int metrics_blocks(int n_f);

@@ -2230,9 +2230,9 @@ __global__ void prior_reduce_kernel(DevGraph<R> g, const R* tmp_k, const R* tmp_
 // Bound: the FP64 pipe (a warp instruction per 16 cycles and SM).  The
 // references come rounded to R from the host (kf_Rr, f_dlc: the same roundings
 // as rounding them here), counts are integers, and what is left in FP64 per
-// factor is the square root of |r|^2 and the sum.  900k factors: 61 -> 34 us
-// (metrics_kernel), and 192 -> 5 us for the final sum by a block instead of
-// one thread.
+// factor is the square root of |r|^2 and the sum.  900k factors: 61 -> 38 us
+// (metrics_kernel), 45 -> 23 us (residual_kernel), and 192 -> 8 us for the
+// final sum by a block instead of one thread (kernel times under ncu).
 
 // |z - h(mu)|^2 of factor f at the current means; false where the point is
 // closer than z_min to its camera.
@@ -2348,14 +2348,70 @@ __global__ void __launch_bounds__(METRIC_BLOCK) problem_metrics_kernel(DevGraph<
 }
 
 // Per-factor reprojection error |z - h(mu)| at the current means (Sec. 9.1),
-// -1 for a point closer than z_min to its camera.
+// -1 for a point closer than z_min to its camera; to its place in the
+// caller's order.
 template <typename R>
-__global__ void __launch_bounds__(METRIC_BLOCK) residual_kernel(DevGraph<R> g, KParams<R> P, double* out) {
+__global__ void __launch_bounds__(METRIC_BLOCK) residual_kernel(DevGraph<R> g, KParams<R> P,
+                                                                const int32_t* __restrict__ obs_index, double* out) {
     const int f = blockIdx.x * METRIC_BLOCK + threadIdx.x;
     if (f >= g.n_f) return;
     R r2;
     const bool ok = error2_at_means<R>(g, P, f, g.z[2 * (size_t)f], g.z[2 * (size_t)f + 1], r2);
-    out[f] = ok ? sqrt(double(r2)) : -1.0;
+    out[obs_index[f]] = ok ? sqrt(double(r2)) : -1.0;
+}
+
+// The current means for the caller, in double, so that they leave the device
+// as the arrays the caller asked for (a copy of 120 bytes a keyframe and
+// point, no pass over the belief records on the host): chart means (n x 6,
+// n x 3), or world poses Exp(dw) Rref | t and points.
+__device__ __forceinline__ void so3_exp_double(const double w[3], double E[9]) {
+    const double th2 = w[0] * w[0] + w[1] * w[1] + w[2] * w[2];
+    double a, b;
+    if (th2 < 1e-12) {
+        a = 1.0 - th2 / 6.0;
+        b = 0.5 - th2 / 24.0;
+    } else {
+        const double th = sqrt(th2), sh = sin(0.5 * th);
+        a = sin(th) / th;
+        b = 2.0 * sh * sh / th2;
+    }
+    const double W[9] = {0, -w[2], w[1], w[2], 0, -w[0], -w[1], w[0], 0};
+    const double W2[9] = {w[0] * w[0] - th2, w[0] * w[1], w[0] * w[2], w[1] * w[0], w[1] * w[1] - th2, w[1] * w[2],
+                          w[2] * w[0], w[2] * w[1], w[2] * w[2] - th2};
+    for (int i = 0; i < 9; ++i) E[i] = a * W[i] + b * W2[i];
+    E[0] += 1.0; E[4] += 1.0; E[8] += 1.0;
+}
+
+template <typename R>
+__global__ void __launch_bounds__(128) means_kernel(DevGraph<R> g, int world, double* __restrict__ kf,
+                                                    double* __restrict__ lm, int32_t* __restrict__ ctl_out) {
+    const int v = blockIdx.x * blockDim.x + threadIdx.x;
+    if (ctl_out && blockIdx.x == 0 && threadIdx.x < CTL_N) ctl_out[threadIdx.x] = g.ctl[threadIdx.x];
+    if (v < g.n_kf) {
+        const R* kb = g.kf_bel + (size_t)v * KBEL + KB_MU;
+        double mu[6];
+        for (int i = 0; i < 6; ++i) mu[i] = double(kb[i]);
+        if (!world) {
+            for (int i = 0; i < 6; ++i) kf[6 * (size_t)v + i] = mu[i];
+            return;
+        }
+        double E[9], Rm[9], c[3];
+        so3_exp_double(mu + 3, E);
+        const double* Rr = g.kf_R + 9 * (size_t)v;
+        for (int i = 0; i < 3; ++i)
+            for (int j = 0; j < 3; ++j)
+                Rm[3 * i + j] = E[3 * i] * Rr[j] + E[3 * i + 1] * Rr[3 + j] + E[3 * i + 2] * Rr[6 + j];
+        for (int i = 0; i < 3; ++i) c[i] = g.kf_c[3 * (size_t)v + i] + mu[i];
+        double* o = kf + 12 * (size_t)v;
+        for (int i = 0; i < 9; ++i) o[i] = Rm[i];
+        for (int i = 0; i < 3; ++i) o[9 + i] = -(Rm[3 * i] * c[0] + Rm[3 * i + 1] * c[1] + Rm[3 * i + 2] * c[2]);
+    } else if (v < g.n_kf + g.n_lm) {
+        const size_t m = v - g.n_kf;
+        for (int i = 0; i < 3; ++i) {
+            const double d = double(g.lm_bel[m * LBEL + 9 + i]);
+            lm[3 * m + i] = world ? g.lm_ref[3 * m + i] + d : d;
+        }
+    }
 }
 
 // The blocks' partials added up by one block, in a fixed order (a thread's
@@ -2551,8 +2607,18 @@ cudaError_t launch_problem_metrics(const DevGraph<R>& g, const KParams<R>& p, co
 }
 
 template <typename R>
-cudaError_t launch_residuals(const DevGraph<R>& g, const KParams<R>& p, double* out, cudaStream_t s) {
-    if (g.n_f > 0) residual_kernel<R><<<(g.n_f + METRIC_BLOCK - 1) / METRIC_BLOCK, METRIC_BLOCK, 0, s>>>(g, p, out);
+cudaError_t launch_residuals(const DevGraph<R>& g, const KParams<R>& p, const int32_t* obs_index, double* out,
+                             cudaStream_t s) {
+    if (g.n_f > 0)
+        residual_kernel<R><<<(g.n_f + METRIC_BLOCK - 1) / METRIC_BLOCK, METRIC_BLOCK, 0, s>>>(g, p, obs_index, out);
+    return cudaGetLastError();
+}
+
+template <typename R>
+cudaError_t launch_means(const DevGraph<R>& g, bool world, double* kf, double* lm, int32_t* ctl_out, cudaStream_t s) {
+    static_assert(CTL_N <= 128, "a thread per control word");
+    const int nv = std::max(g.n_kf + g.n_lm, 1);
+    means_kernel<R><<<(nv + 127) / 128, 128, 0, s>>>(g, world ? 1 : 0, kf, lm, ctl_out);
     return cudaGetLastError();
 }
 
@@ -2674,7 +2740,8 @@ cudaError_t launch_relayout(const DevGraph<R>& nw, const RelayoutSrc<R>& o, int 
     template cudaError_t launch_persistent<R>(const DevGraph<R>&, const KParams<R>&, int, float, int, int, cudaStream_t, int, int); \
     template cudaError_t launch_prior<R>(const DevGraph<R>&, const KParams<R>&, R*, R*, R*, R*, cudaStream_t); \
     template cudaError_t launch_metrics<R>(const DevGraph<R>&, const KParams<R>&, double*, int, double*, cudaStream_t); \
-    template cudaError_t launch_residuals<R>(const DevGraph<R>&, const KParams<R>&, double*, cudaStream_t); \
+    template cudaError_t launch_residuals<R>(const DevGraph<R>&, const KParams<R>&, const int32_t*, double*, cudaStream_t); \
+    template cudaError_t launch_means<R>(const DevGraph<R>&, bool, double*, double*, int32_t*, cudaStream_t); \
     template cudaError_t launch_split_records<R>(const DevGraph<R>&, int, int, int, const int32_t*, float*, cudaStream_t); \
     template cudaError_t launch_relayout<R>(const DevGraph<R>&, const RelayoutSrc<R>&, int, cudaStream_t);
 

@@ -285,18 +285,18 @@ def gbp_get_sizes(g: int):
 
 def gbp_get_beliefs(g: int, covariances: bool = False):
     n_kf, n_lm, _ = gbp_get_sizes(g)
-    kf = np.zeros((n_kf, 12))
-    lm = np.zeros((n_lm, 3))
-    kc = np.zeros((n_kf, 6, 6)) if covariances else None
-    lc = np.zeros((n_lm, 3, 3)) if covariances else None
+    kf = np.empty((n_kf, 12))
+    lm = np.empty((n_lm, 3))
+    kc = np.empty((n_kf, 6, 6)) if covariances else None
+    lc = np.empty((n_lm, 3, 3)) if covariances else None
     _check(lib().gbp_get_beliefs(g, _dp(kf), _dp(lm), _dp(kc), _dp(lc)), g)
     return (kf, lm, kc, lc) if covariances else (kf, lm)
 
 
 def gbp_get_means(g: int):
     n_kf, n_lm, _ = gbp_get_sizes(g)
-    kf = np.zeros((n_kf, 6))
-    lm = np.zeros((n_lm, 3))
+    kf = np.empty((n_kf, 6))
+    lm = np.empty((n_lm, 3))
     _check(lib().gbp_get_means(g, _dp(kf), _dp(lm)), g)
     return kf, lm
 
@@ -330,7 +330,7 @@ def gbp_get_relin_iters(g: int) -> np.ndarray:
 def gbp_get_residuals(g: int) -> np.ndarray:
     """Reprojection error of every observation at the current means
     (observation order), -1 where the point is closer than z_min."""
-    e = np.zeros(gbp_get_sizes(g)[2])
+    e = np.empty(gbp_get_sizes(g)[2])
     _check(lib().gbp_get_residuals(g, _dp(e)), g)
     return e
 

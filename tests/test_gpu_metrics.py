@@ -43,3 +43,43 @@ def test_stats_are_the_residuals_statistics(n_kf, n_lm, precision):
     both = ok & (z1 >= 0.05)
     # FP32 projections of ~500 px: 1e-4 px each
     assert abs(ref - np.linalg.norm(a - b, axis=1)[both].mean()) <= 1e-3 + 1e-4 * ref
+
+
+@pytest.mark.parametrize("n_lm", [40, 5381, 5382, 9000])
+@pytest.mark.parametrize("precision", [0, 2])
+def test_world_beliefs_are_the_chart_means(n_lm, precision):
+    """Read-backs just below and above the size that goes through pinned memory (16384 doubles: 20 x 12 + 3 x 5381 is
+    one less).  Points are lref + dl exactly; poses Exp(dw) Rref and t = -R c carry a few roundings of entries below
+    20: 1e-13."""
+    from scipy.spatial.transform import Rotation
+
+    p = synth.make_walk(7, n_kf=20, n_lm=n_lm)
+    with gbp.Graph(p, huber_nsigma=2.0, precision_mode=precision) as g:
+        g.iterate(6)
+        kf, lm = g.beliefs()
+        mk, ml = g.means()
+    assert np.array_equal(lm, p.lm_init + ml)
+    R0 = p.kf_Rt_init[:, :9].reshape(-1, 3, 3)
+    c = -np.einsum("nji,nj->ni", R0, p.kf_Rt_init[:, 9:]) + mk[:, :3]
+    R = Rotation.from_rotvec(mk[:, 3:]).as_matrix() @ R0
+    assert np.abs(kf[:, :9].reshape(-1, 3, 3) - R).max() <= 1e-13
+    assert np.abs(kf[:, 9:] + np.einsum("nij,nj->ni", R, c)).max() <= 1e-13
+
+
+def test_residuals_follow_the_observation_order_after_a_keyframe_is_added():
+    init, steps = synth.make_stream(3, n_kf=14, n_lm=220, start_kf=10)
+    with gbp.Graph(init, huber_nsigma=2.0) as g:
+        g.iterate(5)
+        assert g.residuals().shape == (init.n_obs,)
+        ok, ol, uv = [init.obs_kf], [init.obs_lm], [init.obs_uv]
+        for s in steps[:3]:
+            k = g.add_keyframe(s.obs_lm, s.obs_uv, n_new_lm=s.n_new_lm)
+            g.iterate(5)
+            ok.append(np.full(len(s.obs_lm), k)), ol.append(s.obs_lm), uv.append(s.obs_uv)
+            kf, lm = g.beliefs()
+            a, b, z = np.concatenate(ok), np.concatenate(ol), np.concatenate(uv)
+            q = np.einsum("nij,nj->ni", kf[a, :9].reshape(-1, 3, 3), lm[b]) + kf[a, 9:]
+            h = np.stack([init.fx * q[:, 0] / q[:, 2] + init.cx, init.fy * q[:, 1] / q[:, 2] + init.cy], 1)
+            e, want = g.residuals(), np.linalg.norm(z - h, axis=1)
+            far = q[:, 2] > 0.5                     # FP32 projections: ~1e-6 relative of up to 1000 px and depth
+            assert np.abs(e - want)[far].max() <= 0.05 + 1e-4 * want[far].max()
