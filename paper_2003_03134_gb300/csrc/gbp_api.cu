@@ -99,6 +99,7 @@ struct DevState {
     int32_t* kpos = nullptr;
     int32_t* lm_off = nullptr;
     int32_t* tile_start = nullptr;
+    int4* tidx = nullptr;
     int32_t* big_lm = nullptr;
     int32_t* deferred = nullptr;
     int32_t* orphan = nullptr;
@@ -125,7 +126,7 @@ struct DevState {
 
     // every buffer freed, or (pool given) handed back to the pool
     void release(BufPool* pool = nullptr) {
-        void* ptrs[] = {z, fk, fm, kf_R, kf_c, lm_ref, kf_Rr, f_dlc, kf_off, kf_list, kpos, lm_off, tile_start, big_lm, deferred, orphan, kf_birth, lm_birth, kf_D, kf_A, lm_D,
+        void* ptrs[] = {z, fk, fm, kf_R, kf_c, lm_ref, kf_Rr, f_dlc, kf_off, kf_list, kpos, lm_off, tile_start, tidx, big_lm, deferred, orphan, kf_birth, lm_birth, kf_D, kf_A, lm_D,
                         uv_ref, x0, tlin, mk, mk2, kj, kjs, lin, ml, mlx, kf_bel, lm_bel, prior_s, hist, eta_inf};
         for (void* p : ptrs)
             if (p) {
@@ -437,6 +438,7 @@ gbp_status build_device(gbp_graph* g, const std::vector<R>* x0_init = nullptr, c
     CK(g->pool.alloc(&s.kpos, nf, g->headroom));
     CK(g->pool.alloc(&s.lm_off, nl + 1, g->headroom));
     CK(g->pool.alloc(&s.tile_start, tiles.size(), g->headroom));
+    CK(g->pool.alloc(&s.tidx, 32 * (size_t)n_tiles, g->headroom));
     CK(g->pool.alloc(&s.big_lm, big.size(), g->headroom));
     CK(g->pool.alloc(&s.deferred, (size_t)n_tiles, g->headroom));
     CK(g->pool.alloc(&s.orphan, orphan.size(), g->headroom));
@@ -500,6 +502,7 @@ gbp_status build_device(gbp_graph* g, const std::vector<R>* x0_init = nullptr, c
     d.kpos = s.kpos;
     d.lm_off = s.lm_off;
     d.tile_start = s.tile_start;
+    d.tidx = s.tidx;
     d.big_lm = s.big_lm;
     d.deferred = s.deferred;
     d.orphan = s.orphan;
@@ -569,6 +572,7 @@ gbp_status build_device(gbp_graph* g, const std::vector<R>* x0_init = nullptr, c
     d.rec_X = nullptr;
     d.rec_T = nullptr;
     d.ctl = g->ctl;
+    CK(launch_tile_index<R>(d, n_tiles, s.tidx, st));
     if (rs && nf) CK(launch_relayout<R>(d, *rs, 0, st));
 
     // priors: per-factor diagonal information at the reference (temporary

@@ -68,6 +68,7 @@ constexpr int KB_LAM = 28; // Lambda, packed lower (21)
 constexpr int KB_ETA = 49; // eta (6)
 constexpr int KBEL = 56;
 constexpr int LBEL = 12;   // landmark belief record
+constexpr int TIDX_WHOLE = 1 << 16;
 
 // Solver parameters as the kernels see them, in the kernel's own precision
 // (no double-to-float conversions in the hot loop).
@@ -123,6 +124,9 @@ struct DevGraph {
     const int32_t* kpos;      // n_f: slot of factor f's keyframe message = its position in kf_list
     const int32_t* lm_off;    // n_lm + 1
     const int32_t* tile_start;// n_tiles + 1: warp tiles of whole landmarks (<= 32 factors each)
+    const int4* tidx;         // n_tiles x 32, a tile's lanes: keyframe (-1: no factor), slot, landmark, and
+                              // the lanes of the landmark's factors in the tile (first, last << 8, TIDX_WHOLE
+                              // if they are all of its factors; else the lane itself)
     const int32_t* big_lm;    // landmarks split across tiles (more than 32 factors)
     int32_t* deferred;        // n_tiles: tiles left to factor_deferred_kernel in this iteration
     const int32_t* orphan;    // variables without factors: keyframe v, or n_kf + landmark
@@ -225,6 +229,7 @@ struct RelayoutSrc {
 };
 template <typename R> cudaError_t launch_relayout(const DevGraph<R>& nw, const RelayoutSrc<R>& o, int phase,
                                                   cudaStream_t s);
+template <typename R> cudaError_t launch_tile_index(const DevGraph<R>& g, int n_tiles, int4* tidx, cudaStream_t s);
 template <typename R> cudaError_t launch_init(const DevGraph<R>& g, const KParams<R>& p, cudaStream_t s);
 template <typename R> cudaError_t launch_belief(const DevGraph<R>& g, const KParams<R>& p, cudaStream_t s,
                                                 bool pdl = false);

@@ -362,6 +362,16 @@ __device__ __forceinline__ void load_rec_cg(const R* src, R* dst) {
     }
 }
 
+// Records that the belief phase and the factor phase exchange: through L2 in
+// the persistent kernel (COH), through L1 in the per-phase kernels, where the
+// kernel boundary makes them visible -- the 16-byte pieces of a record then
+// share their 32-byte sectors instead of fetching each from L2 twice.
+template <bool COH, typename R, int N>
+__device__ __forceinline__ void load_shared_rec(const R* src, R* dst) {
+    if constexpr (COH) load_rec_cg<R, N>(src, dst);
+    else load_rec<R, N>(src, dst);
+}
+
 // An iteration index kept in a Real slot of a record, by its bits.
 template <typename R>
 __device__ __forceinline__ R int_bits(int v) {
@@ -1190,11 +1200,11 @@ __device__ __forceinline__ void mlp_load_wait() {
 
 // One factor's messages once both incoming precisions are known (Lm, im:
 // the landmark side's FP32 Cholesky factor; ks: the keyframe side): the
-// FP64 redo where FP32 cannot take an incoming precision (FP64 = true),
+// FP64 redo where FP32 cannot take an incoming precision,
 // the kept messages, the relinearisation test and the linearisation at the
 // new point, and both new messages in compact form (ck to the keyframe, cl
 // to the landmark), in the basis of L.
-template <typename R, bool FP64>
+template <typename R>
 __device__ __forceinline__ void form_messages(const DevGraph<R>& g, const KParams<R>& P, int f, int k, int slot, int t,
                                               int& tl, bool due, bool active, const R* kbp, Lin<R>& L,
                                               const KfSide<R>& ks, const R* mo, const R* cml, const R* kmu,
@@ -1206,7 +1216,7 @@ __device__ __forceinline__ void form_messages(const DevGraph<R>& g, const KParam
     // relinearisation test)
     bool m64 = false, k64 = false;
     double kc[KC64];   // the keyframe's FP64 incoming precision, formed once for both uses
-    if (FP64 && sizeof(R) == 4 && P.fallback && active) {
+    if (sizeof(R) == 4 && P.fallback && active) {
         if (!ok_m) {
             Arr9<R> pq;
 #pragma unroll
@@ -1365,24 +1375,25 @@ __device__ __forceinline__ void damp_store_fixed(const DevGraph<R>& g, const KPa
 // evaluates the network for the warp's 32 factors at once on the tensor
 // cores, between forming the messages and damping them.
 
-// DEFER (fixed FP32 schedule): a tile with a factor whose incoming
-// precision FP32 cannot take is not worked here -- it stores nothing and is
-// listed for factor_deferred_kernel, which works it with the FP64 redo --
-// so that this kernel carries no state for the FP64 path.
-template <typename R, int MODE, bool DEFER = false>
+template <typename R, int MODE, bool COH>
 __device__ __forceinline__ float tile_work(const DevGraph<R>& g, const KParams<R>& P, int tile, int t, int lane,
                                            MlpSmem<MODE>& S, bool weights_pending = false) {
     const int n_f = g.n_f;
-    const int ts = g.tile_start[tile], te = g.tile_start[tile + 1];
-    const int f = ts + lane;
-    const bool active = f < te;
     constexpr bool FEAT = MODE != DAMP_FIXED;
 
     // Every load of the common path is issued in two waves before anything
-    // is stored: the factor's own entries (wave 1), then what they index
-    // (wave 2).  A store in between (the first linearisation writes the
-    // lin record and the keyframe block) would keep later loads behind it.
-    int m = -1, lo = 0, hi = 0, k = 0, slot = 0, tl = 0, lbirth = 0;
+    // is stored: the lane's tile entry and the tile's first factor (wave 1),
+    // then the factor's own entries and what the tile entry indexes (wave 2).
+    // A store in between (the first linearisation writes the lin record and
+    // the keyframe block) would keep later loads behind it.
+    const int4 te = g.tidx[(size_t)tile * 32 + lane];
+    const int ts = g.tile_start[tile];
+    const bool active = te.x >= 0;
+    const int f = ts + lane;
+    const int m = te.z, k = active ? te.x : 0, slot = te.y;
+    const bool whole = (te.w & TIDX_WHOLE) != 0;
+    const int seg0 = te.w & 31, seg1 = (te.w >> 8) & 31;
+    int lo = 0, hi = 0, tl = 0, lbirth = 0;
     R cml[NML];          // this factor's previous message to the landmark (compact)
     R lin4[NLIN];        // y0, y1, W, |r|^2 of its stored linearisation
 #pragma unroll
@@ -1390,9 +1401,6 @@ __device__ __forceinline__ float tile_work(const DevGraph<R>& g, const KParams<R
 #pragma unroll
     for (int i = 0; i < NLIN; ++i) lin4[i] = R(0);
     if (active) {
-        m = g.fm[f];
-        k = g.fk[f];
-        slot = g.kpos[f];
         tl = g.tlin[f];
 #pragma unroll
         for (int i = 0; i < NML; ++i) cml[i] = g.ml[(size_t)i * n_f + f];
@@ -1400,9 +1408,10 @@ __device__ __forceinline__ float tile_work(const DevGraph<R>& g, const KParams<R
         for (int i = 0; i < NLIN; ++i) lin4[i] = g.lin[(size_t)i * n_f + f];
     }
     // the linearisation point is needed for a factor's first linearisation
-    // and for the relinearisation test once the interval allows one
-    const bool fresh = active && tl == t;
-    const bool due = active && !P.linear && t - tl >= P.relin_interval;
+    // and for the relinearisation test once the interval allows one; from
+    // then on most factors are due in most iterations, so it joins wave 2
+    // without waiting for t_lin
+    const bool may_due = !P.linear && t >= P.relin_interval;
     const R* kbp = g.kf_bel + (size_t)k * KBEL;
     R x0[9];
     R jr[KJ];            // the stored keyframe block of the factor's messages
@@ -1411,13 +1420,15 @@ __device__ __forceinline__ float tile_work(const DevGraph<R>& g, const KParams<R
     R lb_mu[3];          // the landmark's mean mu^t
     R lD[3];             // the landmark's prior diagonal
     if (active) {
-        lo = g.lm_off[m];
-        hi = g.lm_off[m + 1];
+        if constexpr (FEAT) {
+            lo = g.lm_off[m];
+            hi = g.lm_off[m + 1];
+        }
         lbirth = g.lm_birth[m];
         // the keyframe block is moved into kj by the belief phase, on another
         // SM within one persistent launch: read through L2, as the beliefs
-        load_rec_cg<R, KJ>(g.kj + (size_t)slot * KJ, jr);
-        load_rec_cg<R, KB_A>(kbp, kb);
+        load_shared_rec<COH, R, KJ>(g.kj + (size_t)slot * KJ, jr);
+        load_shared_rec<COH, R, KB_A>(kbp, kb);
         load_rec<R, KREC>(mk_read(g, t) + (size_t)slot * KREC, mo);
         const R* lbp = g.lm_bel + (size_t)m * LBEL;
 #pragma unroll
@@ -1438,7 +1449,12 @@ __device__ __forceinline__ float tile_work(const DevGraph<R>& g, const KParams<R
         for (int i = 0; i < 3; ++i) { lb_mu[i] = R(0); lD[i] = R(0); }
     }
 #pragma unroll
-    for (int i = 0; i < 9; ++i) x0[i] = (fresh || due) ? g.x0[(size_t)i * n_f + f] : R(0);
+    for (int i = 0; i < 9; ++i) x0[i] = R(0);
+    const bool fresh = active && tl == t;
+    const bool due = active && may_due && t - tl >= P.relin_interval;
+    if (fresh || due)
+#pragma unroll
+        for (int i = 0; i < 9; ++i) x0[i] = g.x0[(size_t)i * n_f + f];
     // The learned schedule reads a factor's features only where it damps
     // (t - t_lin >= damp_hold), and those read the history written in the
     // two iterations before; earlier in the hold the features are neither
@@ -1464,9 +1480,6 @@ __device__ __forceinline__ float tile_work(const DevGraph<R>& g, const KParams<R
             for (int j = 0; j < HIST; ++j) h[j] = 0.0f;
         }
     }
-    const bool whole = active && lo >= ts && hi <= te;
-    const int seg0 = whole ? lo - ts : lane;
-    const int seg1 = whole ? hi - ts - 1 : lane;
     // the scans below need steps d < the longest landmark segment of the
     // tile; the steps they skip would add nothing
     const int seg_max = __reduce_max_sync(0xffffffffu, unsigned(seg1 - seg0 + 1));
@@ -1591,29 +1604,8 @@ __device__ __forceinline__ float tile_work(const DevGraph<R>& g, const KParams<R
     // 3, 4 and 5
     R ck[NML], cl[NML];  // the new messages: to the keyframe, to the landmark
     R sum[9];            // the new landmark message, expanded
-    if constexpr (DEFER) {
-        static_assert(MODE == DAMP_FIXED && sizeof(R) == 4, "deferral: fixed FP32 schedule");
-        // a tile with a factor that needs the FP64 redo is left to
-        // factor_deferred_kernel: nothing of it is stored here (a first
-        // linearisation above stores what the deferred run stores again)
-        const bool needs64 = P.fallback && active && (!ok_m || !(ks.det >= P.cav_ratio));
-        if (__any_sync(0xffffffffu, needs64)) {
-            if (lane == 0) {
-                const int i = atomicAdd(&g.ctl[CTL_DEFER_N0 + (t & 1)], 1);
-                if (i < g.n_tiles) g.deferred[i] = tile;
-            }
-            return 0.0f;
-        }
-        if (active) {
-            form_messages<R, false>(g, P, f, k, slot, t, tl, due, active, kbp, L, ks, mo, cml, kmu, lb_mu, x0, Pm, qm,
-                                    Lm, im, ok_m, ok_k, ck, cl);
-            damp_store_fixed<R>(g, P, f, slot, t, tl, whole, ok_m, ok_k, ck, cl, mo, cml, L, sum);
-        } else {
-#pragma unroll
-            for (int i = 0; i < 9; ++i) sum[i] = R(0);
-        }
-    } else {
-        form_messages<R, true>(g, P, f, k, slot, t, tl, due, active, kbp, L, ks, mo, cml, kmu, lb_mu, x0, Pm, qm, Lm,
+    {
+        form_messages<R>(g, P, f, k, slot, t, tl, due, active, kbp, L, ks, mo, cml, kmu, lb_mu, x0, Pm, qm, Lm,
                                im, ok_m, ok_k, ck, cl);
         // features of the learned schedule and targets of the record schedule
         float feat[N_FEAT];
@@ -1759,13 +1751,247 @@ __device__ __forceinline__ float tile_work(const DevGraph<R>& g, const KParams<R
         }
     }
     float dmu = 0.0f;
-    if (whole && lane == hi - ts - 1) {
+    if (whole && lane == seg1) {
         dmu = finish_landmark<R>(g, P, m, prior_scale(P, t + 1 - lbirth), sum, lb_mu, g.lm_bel_out);
     }
     return dmu;
 }
 
+// ------------------------------------------------------------------------
+// Phase A, FP32 fixed schedule, deferring: a tile with a factor whose
+// incoming precision FP32 cannot take is not worked here -- it stores nothing
+// (a first linearisation stores what the deferred run stores again) and is
+// listed for factor_deferred_kernel, which works it with the FP64 redo -- so
+// that this kernel carries no state for the FP64 path.
+//
+// The same arithmetic as tile_work, in an order that lets values go early:
+// the message to the landmark as soon as the keyframe side stands (a
+// relinearisation forms it again), then the relinearisation test (it frees
+// the keyframe's mean and the linearisation point).  127 registers, 4 blocks
+// per SM.  What bounds it is the load/store unit (it carries ~130 shuffles
+// and ~45 loads a tile besides the stores), not latency or occupancy: 5
+// blocks per SM (96 registers, 130 bytes spilled) take 7 % longer, bringing
+// later tiles into L2 ahead of their warps 5 % longer, and one dependent load
+// less (the tile entry holds what tile_start led to) is worth 2 %.  Reading
+// the gathered records through L1, so that a record's 16-byte pieces share
+// their 32-byte sectors, took 11 %; the early messages 6 %.  2M factors, a
+// steady iteration: 222 -> 196 us (with a relinearisation test due: 233 ->
+// 214); 690k factors in 32 problems: 95 -> 80 us.
 
+__device__ __forceinline__ float tile_work_deferring(const DevGraph<float>& g, const KParams<float>& P, int tile, int t,
+                                                     int lane) {
+    typedef float R;
+    const int n_f = g.n_f;
+    const int4 te = g.tidx[(size_t)tile * 32 + lane];
+    const int ts = g.tile_start[tile];
+    const bool active = te.x >= 0;
+    const int f = ts + lane;
+    const int m = te.z, k = active ? te.x : 0, slot = te.y;
+    const bool whole = (te.w & TIDX_WHOLE) != 0;
+    const int seg0 = te.w & 31, seg1 = (te.w >> 8) & 31;
+
+    int tl = 0, lbirth = 0;
+    R cml[NML], lin4[NLIN], jr[KJ], kb[KB_A], mo[KREC], lb_mu[3], lD[3];
+    if (active) {
+        tl = g.tlin[f];
+#pragma unroll
+        for (int i = 0; i < NML; ++i) cml[i] = g.ml[(size_t)i * n_f + f];
+#pragma unroll
+        for (int i = 0; i < NLIN; ++i) lin4[i] = g.lin[(size_t)i * n_f + f];
+        lbirth = g.lm_birth[m];
+        load_rec<R, KJ>(g.kj + (size_t)slot * KJ, jr);
+        load_rec<R, KB_A>(g.kf_bel + (size_t)k * KBEL, kb);
+        load_rec<R, KREC>(mk_read(g, t) + (size_t)slot * KREC, mo);
+        R lb[4];
+        load_rec<R, 4>(g.lm_bel + (size_t)m * LBEL + 8, lb);   // eta_2, mu
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            lb_mu[i] = lb[1 + i];
+            lD[i] = g.lm_D[m * 3 + i];
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < NML; ++i) cml[i] = R(0);
+#pragma unroll
+        for (int i = 0; i < NLIN; ++i) lin4[i] = R(0);
+#pragma unroll
+        for (int i = 0; i < KJ; ++i) jr[i] = R(0);
+#pragma unroll
+        for (int i = 0; i < KB_A; ++i) kb[i] = R(0);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) kb[pk(i, i)] = R(1);
+#pragma unroll
+        for (int i = 0; i < KREC; ++i) mo[i] = R(0);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) { lb_mu[i] = R(0); lD[i] = R(0); }
+    }
+    const bool fresh = active && tl == t;
+    // the relinearisation test's other operand, in flight over the keyframe side
+    const bool due = active && !P.linear && t - tl >= P.relin_interval;
+    R x0[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) x0[i] = due ? g.x0[(size_t)i * n_f + f] : R(0);
+    const int seg_max = __reduce_max_sync(0xffffffffu, unsigned(seg1 - seg0 + 1));
+
+    // the factor's linearisation (Sec. 4), the basis of its stored messages
+    Lin<R> L;
+    if (fresh) {
+        Arr9<R> xv;
+#pragma unroll
+        for (int i = 0; i < 9; ++i) xv.v[i] = g.x0[(size_t)i * n_f + f];
+        L = linearise_at<R>(xv, lin_args<R>(P, g, k, f));
+        store_lin<R>(g, f, L);
+        store_jac<R>(g.kjs + (size_t)slot * KJ, L.Jk);
+        if (!kf_in_part(g, k)) store_jac<R>(g.kj + (size_t)slot * KJ, L.Jk);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+            L.Jk[0][j] = jr[j];
+            L.Jk[1][j] = jr[6 + j];
+        }
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            L.Jl[0][j] = -jr[j];
+            L.Jl[1][j] = -jr[6 + j];
+        }
+        L.y[0] = lin4[0];
+        L.y[1] = lin4[1];
+        L.W = lin4[2];
+        L.r2 = lin4[3];
+    }
+
+    // keyframe side and, at once, the message to the landmark it gives
+    KfSide<R> ks;   // a relinearisation needs its a and K again
+    kf_side<R>(kb, kb + KB_MU, L.Jk, mo, ks);
+    const bool ok_k = ks.pd, low = !(ks.det >= P.cav_ratio);
+    R cl[NML];
+#pragma unroll
+    for (int i = 0; i < NML; ++i) cl[i] = cml[i];   // kept unless formed
+    if (ok_k) message_to_landmark<R>(ks, L.y, L.W, cl);
+
+    // the relinearisation test (Sec. 5, Sec. 8), from iteration-t state
+    bool relin = false;
+    if (due) {
+        R d2 = R(0);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) d2 += (kb[KB_MU + i] - x0[i]) * (kb[KB_MU + i] - x0[i]);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) d2 += (lb_mu[i] - x0[6 + i]) * (lb_mu[i] - x0[6 + i]);
+        relin = d2 > P.relin_beta * P.relin_beta;
+    }
+
+    // landmark incoming precision (tile_work, step 2b)
+    R Pm[6], qm[3];
+    {
+        R mlo[9];
+        expand_msg<R, 3>(L.Jl, cml[0], cml[1], cml[2], cml[3], cml[4], mlo, mlo + 6);
+        R fw[9], bw[9];
+#pragma unroll
+        for (int j = 0; j < 9; ++j) { fw[j] = mlo[j]; bw[j] = mlo[j]; }
+        for (int d = 1; d < seg_max; d <<= 1) {
+#pragma unroll
+            for (int j = 0; j < 9; ++j) {
+                R o = __shfl_up_sync(0xffffffffu, fw[j], d);
+                if (lane - d >= seg0) fw[j] += o;
+                R u = __shfl_down_sync(0xffffffffu, bw[j], d);
+                if (lane + d <= seg1) bw[j] += u;
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 9; ++j) {
+            R pre = __shfl_up_sync(0xffffffffu, fw[j], 1);
+            R suf = __shfl_down_sync(0xffffffffu, bw[j], 1);
+            const R cv = (lane - 1 >= seg0 ? pre : R(0)) + (lane + 1 <= seg1 ? suf : R(0));
+            if (j < 6) Pm[j] = cv;
+            else qm[j - 6] = cv;
+        }
+        if (active) {
+            if (whole) {
+                const R sp = prior_scale(P, t - lbirth) * P.inv_sigma2;
+#pragma unroll
+                for (int i = 0; i < 3; ++i) Pm[pk(i, i)] += sp * lD[i];
+            } else {
+                // a landmark split across tiles: its belief divided by this message
+                const R* lbp = g.lm_bel + (size_t)m * LBEL;
+                R lb[9];
+#pragma unroll
+                for (int i = 0; i < 9; ++i) lb[i] = __ldcg(lbp + i);
+#pragma unroll
+                for (int i = 0; i < 6; ++i) Pm[i] = lb[i] - mlo[i];
+#pragma unroll
+                for (int i = 0; i < 3; ++i) qm[i] = lb[6 + i] - mlo[6 + i];
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 6; ++i) Pm[i] = R(0);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) { Pm[pk(i, i)] = R(1); qm[i] = R(0); }
+        }
+    }
+    R im[3], rm;
+    const bool ok_m = chol_packed<R, 3>(Pm, im, rm);   // Pm: its Cholesky factor from here on
+
+    if (__any_sync(0xffffffffu, P.fallback && active && (!ok_m || low))) {
+        if (lane == 0) {
+            const int i = atomicAdd(&g.ctl[CTL_DEFER_N0 + (t & 1)], 1);
+            if (i < g.n_tiles) g.deferred[i] = tile;
+        }
+        return 0.0f;
+    }
+    R sum[9];
+    if (active) {
+        if (!ok_m) atomicAdd(&g.ctl[CTL_HELD], 1);
+        if (!ok_k) atomicAdd(&g.ctl[CTL_HELD], 1);
+        if (relin && ok_m && ok_k) {
+            const R* kbp = g.kf_bel + (size_t)k * KBEL;
+            Arr9<R> xn;
+            Arr12<R> Jo;
+#pragma unroll
+            for (int i = 0; i < 6; ++i) {
+                xn.v[i] = __ldcg(kbp + KB_MU + i);
+                Jo.v[i] = L.Jk[0][i];
+                Jo.v[6 + i] = L.Jk[1][i];
+            }
+#pragma unroll
+            for (int i = 0; i < 3; ++i) xn.v[6 + i] = lb_mu[i];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) g.x0[(size_t)i * n_f + f] = xn.v[i];
+            tl = t;
+            g.tlin[f] = t;
+            atomicAdd(&g.ctl[CTL_RELINS], 1);
+            const Rebased<R> rb = rebase<R>(kbp, Jo, mo[3], mo[4], ks.a0, ks.a1, ks.K00, ks.K01, ks.K11, true, xn,
+                                            lin_args<R>(P, g, k, f));
+            L = rb.L;
+            store_lin<R>(g, f, L);
+            store_jac<R>(g.kjs + (size_t)slot * KJ, L.Jk);
+            if (!kf_in_part(g, k)) store_jac<R>(g.kj + (size_t)slot * KJ, L.Jk);
+#pragma unroll
+            for (int i = 0; i < NML; ++i) cl[i] = rb.cl[i];
+        }
+        R ck[NML];
+        if (ok_m) {
+            message_chol<R, 3>(Pm, im, qm, L.Jl, L.y, L.W, ck);
+        } else {
+#pragma unroll
+            for (int i = 0; i < NML; ++i) ck[i] = mo[i];
+        }
+        damp_store_fixed<R>(g, P, f, slot, t, tl, whole, ok_m, ok_k, ck, cl, mo, cml, L, sum);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) sum[i] = R(0);
+    }
+    for (int d = 1; d < seg_max; d <<= 1) {
+#pragma unroll
+        for (int j = 0; j < 9; ++j) {
+            R o = __shfl_up_sync(0xffffffffu, sum[j], d);
+            if (lane - d >= seg0) sum[j] += o;
+        }
+    }
+    float dmu = 0.0f;
+    if (whole && lane == seg1)
+        dmu = finish_landmark<R>(g, P, m, prior_scale(P, t + 1 - lbirth), sum, lb_mu, g.lm_bel_out);
+    return dmu;
+}
 
 // ------------------------------------------------------------------------
 // Phase B: one group of threads per work item -- one warp, or the whole
@@ -1827,7 +2053,7 @@ __device__ __forceinline__ void group_total(R (&v)[NV], R (&out)[NVAL]) {
 }
 
 // W: warps per item (g.b_warps)
-template <typename R, int W>
+template <typename R, int W, bool COH>
 __device__ __forceinline__ float phase_b_item(const DevGraph<R>& g, const KParams<R>& P, int item, int t) {
     const int gsize = 32 * W;
     const int tg = threadIdx.x & (gsize - 1);   // thread within the group
@@ -1862,8 +2088,8 @@ __device__ __forceinline__ float phase_b_item(const DevGraph<R>& g, const KParam
             for (int u = 0; u < BU; ++u) {
                 const int i = i0 + u * gsize;
                 if (i < b1) {
-                    load_rec_cg<R, KREC>(msgs + (size_t)i * KREC, rec[u]);
-                    load_rec_cg<R, KJ>(g.kj + (size_t)i * KJ, jr[u]);
+                    load_shared_rec<COH, R, KREC>(msgs + (size_t)i * KREC, rec[u]);
+                    load_shared_rec<COH, R, KJ>(g.kj + (size_t)i * KJ, jr[u]);
                 }
             }
 #pragma unroll
@@ -1969,7 +2195,8 @@ __device__ __forceinline__ void factor_body(const DevGraph<R>& g, const KParams<
     const int t = g.ctl[CTL_ITER];
     float dmu = 0.0f;
     if (tile < g.n_tiles)   // uniform per warp
-        dmu = tile_work<R, MODE, DEFER>(g, P, g.tile_off + tile, t, lane, S, MODE == DAMP_LEARNED);
+        if constexpr (DEFER) dmu = tile_work_deferring(g, P, g.tile_off + tile, t, lane);
+        else dmu = tile_work<R, MODE, false>(g, P, g.tile_off + tile, t, lane, S, MODE == DAMP_LEARNED);
     else if constexpr (MODE == DAMP_LEARNED) mlp_load_wait();   // the block's barrier, for warps without a tile
     pdl_allow_next();
     dmu = warp_max(dmu);
@@ -2033,7 +2260,7 @@ __global__ void __launch_bounds__(FACTOR_BLOCK) belief_kernel(DevGraph<R> g, KPa
     }
     float dmu = 0.0f;
     const int item = phase_b_item_of(BW, blockIdx.x);
-    if (item < phase_b_items(g)) dmu = phase_b_item<R, BW>(g, P, item, t);   // uniform per group
+    if (item < phase_b_items(g)) dmu = phase_b_item<R, BW, false>(g, P, item, t);   // uniform per group
     pdl_allow_next();
     // max is order independent: the atomic on non-negative float bits is deterministic
     if (dmu > 0.0f) dmu_atomic_max_slot(g.ctl, dmu_slot(t), dmu);
@@ -2104,7 +2331,7 @@ __global__ void __launch_bounds__(FACTOR_BLOCK, MINB)
         // phase A: factors and landmarks wholly inside a tile
         float dmu = 0.0f;
         for (int tile = gwarp; tile < g.n_tiles; tile += nwarps)
-            dmu = fmaxf(dmu, tile_work<R, MODE>(g, P, g.tile_off + tile, t, lane, S));
+            dmu = fmaxf(dmu, tile_work<R, MODE, true>(g, P, g.tile_off + tile, t, lane, S));
         dmu = warp_max(dmu);
         if (lane == 0 && dmu > 0.0f) dmu_atomic_max_slot(g.ctl, dmu_slot(t), dmu);
         if (!grid_barrier(g.ctl, nb, &flag_sh)) break;
@@ -2115,7 +2342,7 @@ __global__ void __launch_bounds__(FACTOR_BLOCK, MINB)
         constexpr bool per_block = BW == WPB;
         const int stride = per_block ? nb : nwarps;
         for (int item = per_block ? int(blockIdx.x) : gwarp; item < items; item += stride)
-            d2 = fmaxf(d2, phase_b_item<R, BW>(g, P, item, t));
+            d2 = fmaxf(d2, phase_b_item<R, BW, true>(g, P, item, t));
         if (d2 > 0.0f) dmu_atomic_max_slot(g.ctl, dmu_slot(t), d2);   // groups' first threads
         if (!grid_barrier(g.ctl, nb, &flag_sh)) break;
         done = it + 1;
@@ -2127,6 +2354,23 @@ __global__ void __launch_bounds__(FACTOR_BLOCK, MINB)
         g.ctl[CTL_DMU_LAST] = __float_as_int(last);
         g.ctl[CTL_ITERS_RUN] = done;
     }
+}
+
+// The tile entries (gbp_internal.h) from the factor arrays: a warp per tile.
+template <typename R>
+__global__ void __launch_bounds__(128) tile_index_kernel(DevGraph<R> g, int n_tiles, int4* __restrict__ tidx) {
+    const int tile = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (tile >= n_tiles) return;
+    const int ts = g.tile_start[tile], te = g.tile_start[tile + 1], f = ts + lane;
+    int4 e = make_int4(-1, 0, -1, lane | (lane << 8));
+    if (f < te) {
+        e.x = g.fk[f];
+        e.y = g.kpos[f];
+        e.z = g.fm[f];
+        const int lo = g.lm_off[e.z], hi = g.lm_off[e.z + 1];
+        if (lo >= ts && hi <= te) e.w = (lo - ts) | ((hi - ts - 1) << 8) | TIDX_WHOLE;
+    }
+    tidx[(size_t)tile * 32 + lane] = e;
 }
 
 // Beliefs of iteration 0: b^0 = prior(0) (+ anchor), mean 0.
@@ -2575,6 +2819,12 @@ cudaError_t launch_capture_messages(const DevGraph<R>& g, int t, R* eta_inf, cud
 }
 
 template <typename R>
+cudaError_t launch_tile_index(const DevGraph<R>& g, int n_tiles, int4* tidx, cudaStream_t s) {
+    if (n_tiles > 0) tile_index_kernel<R><<<(n_tiles + 3) / 4, 128, 0, s>>>(g, n_tiles, tidx);
+    return cudaGetLastError();
+}
+
+template <typename R>
 cudaError_t launch_init(const DevGraph<R>& g, const KParams<R>& p, cudaStream_t s) {
     int nv = g.n_kf + g.n_lm;
     if (nv > 0) init_beliefs_kernel<R><<<(nv + 127) / 128, 128, 0, s>>>(g, p);
@@ -2733,6 +2983,7 @@ cudaError_t launch_relayout(const DevGraph<R>& nw, const RelayoutSrc<R>& o, int 
 #define GBP_INSTANTIATE(R)                                                                                 \
     template cudaError_t launch_factor<R>(const DevGraph<R>&, const KParams<R>&, cudaStream_t, int, bool, int); \
     template cudaError_t launch_capture_messages<R>(const DevGraph<R>&, int, R*, cudaStream_t);            \
+    template cudaError_t launch_tile_index<R>(const DevGraph<R>&, int, int4*, cudaStream_t);               \
     template cudaError_t launch_init<R>(const DevGraph<R>&, const KParams<R>&, cudaStream_t);              \
     template cudaError_t launch_belief<R>(const DevGraph<R>&, const KParams<R>&, cudaStream_t, bool);      \
     template cudaError_t launch_problem_metrics<R>(const DevGraph<R>&, const KParams<R>&, const int32_t*, int, double*, cudaStream_t); \

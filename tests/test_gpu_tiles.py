@@ -1,0 +1,44 @@
+"""The deferring factor kernel against the general factor phase at the edges of its tiles: landmarks with 31, 32, 33 and
+more factors (split across tiles), tiles of one factor, landmarks without factors, relinearisations in every iteration
+(beta = 0, interval 1) and none (linear)."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+from paper_2003_03134_gb300 import build, gbp, synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    build.build()
+    gbp.lib()
+
+
+def _problem(counts):
+    """A walk of 64 keyframes whose i-th landmark keeps counts[i] of its observations (0: none)."""
+    p = synth.make_walk(11, n_kf=64, n_lm=len(counts), obs_range=(max(counts), 64))
+    rank = np.arange(p.n_obs) - np.searchsorted(p.obs_lm, p.obs_lm)
+    keep = rank < np.asarray(counts)[p.obs_lm]
+    return dataclasses.replace(p, obs_kf=p.obs_kf[keep], obs_lm=p.obs_lm[keep], obs_uv=p.obs_uv[keep],
+                               obs_outlier=p.obs_outlier[keep])
+
+
+@pytest.mark.parametrize("counts", [[31, 32, 33, 0, 1, 32, 40, 2, 3, 0], [1] * 70, [32] * 9, [4, 5, 6, 7, 8, 9, 10] * 12])
+@pytest.mark.parametrize("params", [{}, {"linear": 1}, {"relin_beta": 0.0, "relin_interval": 3}])
+def test_deferring_kernel_gives_the_general_phase_bits(counts, params):
+    p = _problem(counts)
+    got = []
+    for mode, shape in ((2, 0), (2, 4), (2, 5), (1, 0)):
+        with gbp.Graph(p, huber_nsigma=2.0, launch_mode=mode, factor_shape=shape, **params) as g:
+            for n in (1, 9, 2, 13):
+                g.iterate(n)
+            got.append([*g.means(), g.relin_iters()])
+    for other in got[1:]:
+        for a, b in zip(got[0], other):
+            assert np.array_equal(a, b)
