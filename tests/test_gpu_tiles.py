@@ -21,8 +21,8 @@ def _lib():
 
 
 def _problem(counts):
-    """A walk of 64 keyframes whose i-th landmark keeps counts[i] of its observations (0: none)."""
-    p = synth.make_walk(11, n_kf=64, n_lm=len(counts), obs_range=(max(counts), 64))
+    """A ring of 64 keyframes whose i-th landmark keeps counts[i] of its observations (0: none)."""
+    p = synth.make_circle(11, n_kf=64, n_lm=len(counts), obs_range=(max(counts), max(counts)))
     rank = np.arange(p.n_obs) - np.searchsorted(p.obs_lm, p.obs_lm)
     keep = rank < np.asarray(counts)[p.obs_lm]
     return dataclasses.replace(p, obs_kf=p.obs_kf[keep], obs_lm=p.obs_lm[keep], obs_uv=p.obs_uv[keep],
