@@ -372,6 +372,52 @@ __device__ __forceinline__ void load_shared_rec(const R* src, R* dst) {
     else load_rec<R, N>(src, dst);
 }
 
+// 32-byte loads and stores of FP32 records that start on 32-byte boundaries
+// (message records, 8 floats; belief records, 56 floats): one access a
+// sector, half the load/store instructions.
+template <bool COH>
+__device__ __forceinline__ void load8(const float* p, float* v) {
+    if constexpr (COH)
+        asm volatile("ld.global.cg.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                     : "l"(p)
+                     : "memory");
+    else
+        asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                     : "l"(p)
+                     : "memory");
+}
+__device__ __forceinline__ void store8(float* p, const float* v) {
+    asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]),
+                 "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+                 : "memory");
+}
+
+// A message record, and the part of a belief record the factor phase reads.
+template <bool COH, typename R>
+__device__ __forceinline__ void load_msg(const R* src, R* dst) {
+    if constexpr (sizeof(R) == 4) load8<COH>(src, dst);
+    else load_shared_rec<COH, R, KREC>(src, dst);
+}
+template <typename R>
+__device__ __forceinline__ void store_msg(R* dst, const R* src) {
+    if constexpr (sizeof(R) == 4) store8(dst, src);
+    else store_rec<R, KREC>(dst, src);
+}
+template <bool COH, typename R>
+__device__ __forceinline__ void load_kf(const R* src, R* dst) {
+    if constexpr (sizeof(R) == 4) {
+        load8<COH>(src, dst);
+        load8<COH>(src + 8, dst + 8);
+        load8<COH>(src + 16, dst + 16);
+        load_shared_rec<COH, R, KB_A - 24>(src + 24, dst + 24);
+    } else {
+        load_shared_rec<COH, R, KB_A>(src, dst);
+    }
+}
+static_assert(KREC == 8 && KBEL % 8 == 0 && KB_A > 24, "32-byte records");
+
 // An iteration index kept in a Real slot of a record, by its bits.
 template <typename R>
 __device__ __forceinline__ R int_bits(int v) {
@@ -1345,7 +1391,7 @@ __device__ __forceinline__ void damp_store_fixed(const DevGraph<R>& g, const KPa
     rec[KREC_TL] = int_bits<R>(tl);
     rec[6] = R(0);
     rec[7] = R(0);
-    store_rec<R, KREC>(mk_write(g, t) + (size_t)slot * KREC, rec);
+    store_msg<R>(mk_write(g, t) + (size_t)slot * KREC, rec);
 #pragma unroll
     for (int i = 0; i < NML; ++i) g.ml_out[(size_t)i * n_f + f] = cl[i];
     expand_msg<R, 3>(L.Jl, cl[0], cl[1], cl[2], cl[3], cl[4], sum, sum + 6);
@@ -1428,8 +1474,8 @@ __device__ __forceinline__ float tile_work(const DevGraph<R>& g, const KParams<R
         // the keyframe block is moved into kj by the belief phase, on another
         // SM within one persistent launch: read through L2, as the beliefs
         load_shared_rec<COH, R, KJ>(g.kj + (size_t)slot * KJ, jr);
-        load_shared_rec<COH, R, KB_A>(kbp, kb);
-        load_rec<R, KREC>(mk_read(g, t) + (size_t)slot * KREC, mo);
+        load_kf<COH, R>(kbp, kb);
+        load_msg<false, R>(mk_read(g, t) + (size_t)slot * KREC, mo);
         const R* lbp = g.lm_bel + (size_t)m * LBEL;
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
@@ -1728,7 +1774,7 @@ __device__ __forceinline__ float tile_work(const DevGraph<R>& g, const KParams<R
             rec[KREC_TL] = int_bits<R>(tl);
             rec[6] = R(0);
             rec[7] = R(0);
-            store_rec<R, KREC>(mk_write(g, t) + (size_t)slot * KREC, rec);
+            store_msg<R>(mk_write(g, t) + (size_t)slot * KREC, rec);
 #pragma unroll
             for (int i = 0; i < NML; ++i) g.ml_out[(size_t)i * n_f + f] = cl[i];
             expand_msg<R, 3>(L.Jl, cl[0], cl[1], cl[2], cl[3], cl[4], sum, sum + 6);
@@ -1774,9 +1820,10 @@ __device__ __forceinline__ float tile_work(const DevGraph<R>& g, const KParams<R
 // later tiles into L2 ahead of their warps 5 % longer, and one dependent load
 // less (the tile entry holds what tile_start led to) is worth 2 %.  Reading
 // the gathered records through L1, so that a record's 16-byte pieces share
-// their 32-byte sectors, took 11 %; the early messages 6 %.  2M factors, a
-// steady iteration: 222 -> 196 us (with a relinearisation test due: 233 ->
-// 214); 690k factors in 32 problems: 95 -> 80 us.
+// their 32-byte sectors, took 11 % off, the early messages 6 %, 32-byte loads
+// and stores of the records 5 %.  2M factors, a steady iteration (all
+// kernels): 222 -> 186 us (with a relinearisation test due: 233 -> 205); 690k
+// factors in 32 problems: 95 -> 78 us.
 
 __device__ __forceinline__ float tile_work_deferring(const DevGraph<float>& g, const KParams<float>& P, int tile, int t,
                                                      int lane) {
@@ -1800,8 +1847,8 @@ __device__ __forceinline__ float tile_work_deferring(const DevGraph<float>& g, c
         for (int i = 0; i < NLIN; ++i) lin4[i] = g.lin[(size_t)i * n_f + f];
         lbirth = g.lm_birth[m];
         load_rec<R, KJ>(g.kj + (size_t)slot * KJ, jr);
-        load_rec<R, KB_A>(g.kf_bel + (size_t)k * KBEL, kb);
-        load_rec<R, KREC>(mk_read(g, t) + (size_t)slot * KREC, mo);
+        load_kf<false, R>(g.kf_bel + (size_t)k * KBEL, kb);
+        load_msg<false, R>(mk_read(g, t) + (size_t)slot * KREC, mo);
         R lb[4];
         load_rec<R, 4>(g.lm_bel + (size_t)m * LBEL + 8, lb);   // eta_2, mu
 #pragma unroll
@@ -2088,7 +2135,7 @@ __device__ __forceinline__ float phase_b_item(const DevGraph<R>& g, const KParam
             for (int u = 0; u < BU; ++u) {
                 const int i = i0 + u * gsize;
                 if (i < b1) {
-                    load_shared_rec<COH, R, KREC>(msgs + (size_t)i * KREC, rec[u]);
+                    load_msg<COH, R>(msgs + (size_t)i * KREC, rec[u]);
                     load_shared_rec<COH, R, KJ>(g.kj + (size_t)i * KJ, jr[u]);
                 }
             }
