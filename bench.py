@@ -80,7 +80,7 @@ def peaks():
 
 def kernel_source_hash():
     h = hashlib.sha256()
-    for name in ("gbp_kernels.cu", "gbp_internal.h"):
+    for name in ("gbp_device.cuh", "gbp_kernels.cu", "gbp_resident.cu", "gbp_internal.h"):
         with open(os.path.join(ROOT, "paper_2003_03134_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]

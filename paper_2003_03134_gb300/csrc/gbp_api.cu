@@ -1053,9 +1053,13 @@ gbp_status iterate_phases(gbp_graph* g, int n, float conv_tol, int* done_out) {
 gbp_status iterate_persistent(gbp_graph* g, int n, float conv_tol, int* done_out) {
     const int dm = g->prm.damping_mode;
     const int ps = persistent_shape(g);
-    const int grid = g->storage ? persistent_grid<double>(g->sd.g, dm, ps) : persistent_grid<float>(g->sf.g, dm, ps);
+    int na = 0;
+    const bool resident = !g->storage && dm == 0 && resident_grid(g->sf.g, &na) > 0;
+    const int grid = resident ? 1 : g->storage ? persistent_grid<double>(g->sd.g, dm, ps) : persistent_grid<float>(g->sf.g, dm, ps);
     if (grid <= 0) return fail(g, GBP_ECUDA, "persistent launch: occupancy query failed");
-    cudaError_t e = g->storage
+    cudaError_t e = resident
+        ? launch_resident(g->sf.g, make_kparams<float>(g), n, conv_tol, g->prm.check_every, g->stream)
+        : g->storage
         ? launch_persistent<double>(g->sd.g, make_kparams<double>(g), n, conv_tol, g->prm.check_every, grid, g->stream,
                                     dm, ps)
         : launch_persistent<float>(g->sf.g, make_kparams<float>(g), n, conv_tol, g->prm.check_every, grid, g->stream,

@@ -188,7 +188,12 @@ enum Ctl : int {
     CTL_DEFER_N1 = 15,     // in odd iterations
     CTL_DEFER_DONE = 16,   // blocks of factor_deferred_kernel done (its last block clears the list)
     CTL_RESUMS = 17,       // keyframe incoming precisions summed again exactly from their parts (FP64)
-    CTL_N = 20
+    // 18, 19: the device convergence loop's state (gbp_api.cu)
+    CTL_RES_BASE1 = 20,    // resident kernel: its arrival counts at the end of the last launch
+    CTL_RES_BASE2 = 21,
+    CTL_RES_CNT1 = 64,     // messages stored: arrivals (a cache line of their own, polled)
+    CTL_RES_CNT2 = 96,     // end of iteration: arrivals
+    CTL_N = 128
 };
 
 // metrics reduction output (double slots)
@@ -237,6 +242,10 @@ template <typename R> int persistent_grid(const DevGraph<R>& g, int mode, int sh
 template <typename R> cudaError_t launch_persistent(const DevGraph<R>& g, const KParams<R>& p, int n_iters,
                                                     float conv_tol, int check_every, int grid, cudaStream_t s,
                                                     int mode, int shape);
+// resident kernel (gbp_resident.cu): blocks (0 = not for this graph), factor warps per block in *na
+int resident_grid(const DevGraph<float>& g, int* na);
+cudaError_t launch_resident(const DevGraph<float>& g, const KParams<float>& p, int n_iters, float conv_tol,
+                            int check_every, cudaStream_t s);
 template <typename R> cudaError_t launch_capture_messages(const DevGraph<R>& g, int t, R* eta_inf, cudaStream_t s);
 template <typename R> cudaError_t launch_prior(const DevGraph<R>& g, const KParams<R>& p, R* tmp_k, R* tmp_l,
                                                R* kf_D, R* lm_D, cudaStream_t s);

@@ -42,3 +42,22 @@ def test_deferring_kernel_gives_the_general_phase_bits(counts, params):
     for other in got[1:]:
         for a, b in zip(got[0], other):
             assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("n_problems", [1, 15, 16, 34, 36, 60])
+@pytest.mark.parametrize("params", [{}, {"fp64_pivot_ratio": 1.0}, {"conv_tol": 1e-3, "check_every": 3}])
+def test_persistent_launch_gives_the_per_phase_bits(n_problems, params):
+    """Rings of 10 keyframes and ~17 tiles each as one graph: fewer and more keyframes than blocks (152), one and two
+    tiles per factor warp's SM share (608 tiles), up to the size that the resident kernel takes; several calls, so that
+    each starts from the state the last one left."""
+    problems = [synth.make_circle(s) for s in range(n_problems)]
+    got = []
+    for mode in (1, 2):
+        with gbp.Graph(problems, huber_nsigma=2.0, launch_mode=mode, **params) as g:
+            done = [g.iterate(n) for n in (1, 2, 9, 20)]
+            st = g.stats()
+            got.append([np.array(done), *g.means(), g.relin_iters(),
+                        np.array([st[k] for k in ("iterations", "max_dmu", "fp64_fallbacks", "relinearisations",
+                                                  "held_messages", "fp64_resums")])])
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
