@@ -30,6 +30,7 @@ static_assert(GBP_SPLIT_KF_FLOATS == KBEL, "split keyframe record");
 namespace {
 
 constexpr int GRAPH_CHUNK = 8;   // iterations per captured CUDA graph
+constexpr size_t STAGE_MAX = 4 << 20;   // host arrays of a grown layout up to this many bytes go up in one pinned copy
 
 template <typename T>
 cudaError_t dev_alloc(T** p, size_t n) {
@@ -85,7 +86,9 @@ struct BufPool {
 template <typename R>
 struct DevState {
     DevGraph<R> g{};
-    // owned device pointers (non-const views of g)
+    // one device allocation holds every array of the layout; the pointers
+    // below (non-const views of g) lie in it, except the last group
+    unsigned char* arena = nullptr;
     R* z = nullptr;
     int32_t* fk = nullptr;
     int32_t* fm = nullptr;
@@ -108,7 +111,6 @@ struct DevState {
     R* kf_D = nullptr;
     R* kf_A = nullptr;
     R* lm_D = nullptr;
-    R* uv_ref = nullptr;
     R* x0 = nullptr;
     int32_t* tlin = nullptr;
     R* mk = nullptr;
@@ -120,14 +122,17 @@ struct DevState {
     R* mlx = nullptr;
     R* kf_bel = nullptr;
     R* lm_bel = nullptr;
-    R* prior_s = nullptr;      // prior scale table, prior_anneal_iters + 1 entries
+    R* anc = nullptr;          // 6 x n_kf: 1 on anchored keyframes, else 0
+    int32_t* src_f = nullptr;  // the previous layout's factor of each factor (a keyframe was added)
     float* hist = nullptr;     // learned damping: HIST x n_f message-change history
+    // allocated by themselves
+    R* uv_ref = nullptr;
+    R* prior_s = nullptr;      // prior scale table, prior_anneal_iters + 1 entries
     R* eta_inf = nullptr;      // record schedule: 9 x n_f reference messages (gbp_capture_messages)
 
-    // every buffer freed, or (pool given) handed back to the pool
+    // every allocation freed, or (pool given) handed back to the pool
     void release(BufPool* pool = nullptr) {
-        void* ptrs[] = {z, fk, fm, kf_R, kf_c, lm_ref, kf_Rr, f_dlc, kf_off, kf_list, kpos, lm_off, tile_start, tidx, big_lm, deferred, orphan, kf_birth, lm_birth, kf_D, kf_A, lm_D,
-                        uv_ref, x0, tlin, mk, mk2, kj, kjs, lin, ml, mlx, kf_bel, lm_bel, prior_s, hist, eta_inf};
+        void* ptrs[] = {arena, uv_ref, prior_s, eta_inf};
         for (void* p : ptrs)
             if (p) {
                 if (pool) pool->put(p);
@@ -155,20 +160,6 @@ void so3_exp_host(const double w[3], double E[9]) {
                     w[2] * w[0], w[2] * w[1], w[2] * w[2] - th2};
     for (int i = 0; i < 9; ++i) E[i] = a * W[i] + b * W2[i];
     E[0] += 1.0; E[4] += 1.0; E[8] += 1.0;
-}
-
-// The keyframe belief record of a prior-only belief (diagonal p): its
-// Cholesky factor (1/sqrt(p_i) on the diagonal), mean 0, trace, Lambda.
-template <typename R>
-void kf_prior_record_host(const R* p, R* out) {
-    std::fill(out, out + KBEL, R(0));
-    R tr = R(0);
-    for (int i = 0; i < 6; ++i) {
-        out[KB_L + i * (i + 1) / 2 + i] = R(1.0 / std::sqrt(double(p[i])));
-        out[KB_LAM + i * (i + 1) / 2 + i] = p[i];
-        tr += p[i];
-    }
-    out[KB_TR] = tr;
 }
 
 }  // namespace
@@ -227,6 +218,8 @@ struct gbp_graph {
     double* h_read = nullptr;                   // pinned, SMALL_READ doubles
     void* d_read = nullptr;
     size_t read_cap = 0;
+    unsigned char* h_stage = nullptr;           // pinned, STAGE_MAX bytes: a layout's arrays on their way to the device
+    bool stage_busy = false;                    // its last copy may still be in flight
     int32_t* d_obs = nullptr;
     size_t obs_cap = 0;
     bool obs_current = false;
@@ -341,11 +334,17 @@ gbp_status upload_prior_table(gbp_graph* g) {
 // Upload the problem into freshly allocated device buffers of type R and
 // generate the priors; leaves the dynamic state uninitialised.
 template <typename R>
-// x0_init: linearisation points for the prior pass (host), or rs: gathered
-// on the device from a previous layout (a keyframe was added), else zero.
-gbp_status build_device(gbp_graph* g, const std::vector<R>* x0_init = nullptr, const RelayoutSrc<R>* rs = nullptr) {
+// rs, src_f: the linearisation points are gathered on the device from a
+// previous layout (a keyframe was added; rs->src_f is set to src_f's device
+// copy), else they are zero.
+gbp_status build_device(gbp_graph* g, RelayoutSrc<R>* rs = nullptr, const std::vector<int32_t>* src_f = nullptr) {
     DevState<R>& s = state<R>(g);
-    s.release(&g->pool);
+    {
+        R* const table = s.prior_s;   // depends on the parameters alone: kept
+        s.prior_s = nullptr;
+        s.release(&g->pool);
+        s.prior_s = table;
+    }
     const int nk = g->n_kf, nl = g->n_lm, nf = g->n_f;
     // CSR lists
     std::vector<int32_t> kf_off(nk + 1, 0), lm_off(nl + 1, 0), kf_list(nf);
@@ -423,66 +422,82 @@ gbp_status build_device(gbp_graph* g, const std::vector<R>* x0_init = nullptr, c
             dlc[(size_t)j * nf + f] = R(g->lm_ref[3 * (size_t)g->fm[f] + j] - g->kf_c[3 * (size_t)g->fk[f] + j]);
     for (int v = 0; v < nk; ++v)
         if (g->anchored[v])
-            for (int i = 0; i < 6; ++i) anc[6 * v + i] = R(1);   // scaled by D after the prior pass
+            for (int i = 0; i < 6; ++i) anc[6 * v + i] = R(1);   // the prior pass scales it by D
 
-    CK(g->pool.alloc(&s.z, 2 * (size_t)nf, g->headroom));
-    CK(g->pool.alloc(&s.fk, nf, g->headroom));
-    CK(g->pool.alloc(&s.fm, nf, g->headroom));
-    CK(g->pool.alloc(&s.kf_R, 9 * (size_t)nk, g->headroom));
-    CK(g->pool.alloc(&s.kf_c, 3 * (size_t)nk, g->headroom));
-    CK(g->pool.alloc(&s.lm_ref, 3 * (size_t)nl, g->headroom));
-    CK(g->pool.alloc(&s.kf_Rr, 9 * (size_t)nk, g->headroom));
-    CK(g->pool.alloc(&s.f_dlc, 3 * (size_t)nf, g->headroom));
-    CK(g->pool.alloc(&s.kf_off, nk + 1, g->headroom));
-    CK(g->pool.alloc(&s.kf_list, nf, g->headroom));
-    CK(g->pool.alloc(&s.kpos, nf, g->headroom));
-    CK(g->pool.alloc(&s.lm_off, nl + 1, g->headroom));
-    CK(g->pool.alloc(&s.tile_start, tiles.size(), g->headroom));
-    CK(g->pool.alloc(&s.tidx, 32 * (size_t)n_tiles, g->headroom));
-    CK(g->pool.alloc(&s.big_lm, big.size(), g->headroom));
-    CK(g->pool.alloc(&s.deferred, (size_t)n_tiles, g->headroom));
-    CK(g->pool.alloc(&s.orphan, orphan.size(), g->headroom));
-    CK(g->pool.alloc(&s.kf_birth, nk, g->headroom));
-    CK(g->pool.alloc(&s.lm_birth, nl, g->headroom));
-    CK(g->pool.alloc(&s.kf_D, 6 * (size_t)nk, g->headroom));
-    CK(g->pool.alloc(&s.kf_A, 6 * (size_t)nk, g->headroom));
-    CK(g->pool.alloc(&s.lm_D, 3 * (size_t)nl, g->headroom));
-    CK(g->pool.alloc(&s.x0, 9 * (size_t)nf, g->headroom));
-    CK(g->pool.alloc(&s.tlin, nf, g->headroom));
-    CK(g->pool.alloc(&s.mk, (size_t)KREC * nf, g->headroom));
-    CK(g->pool.alloc(&s.mk2, (size_t)KREC * nf, g->headroom));
-    CK(g->pool.alloc(&s.kj, (size_t)KJ * nf, g->headroom));
-    CK(g->pool.alloc(&s.kjs, (size_t)KJ * nf, g->headroom));
-    CK(g->pool.alloc(&s.lin, (size_t)NLIN * nf, g->headroom));
-    CK(g->pool.alloc(&s.ml, (size_t)NML * nf, g->headroom));
-    CK(g->pool.alloc(&s.mlx, 9 * (size_t)nf, g->headroom));
-    CK(g->pool.alloc(&s.kf_bel, (size_t)KBEL * nk, g->headroom));
-    CK(g->pool.alloc(&s.lm_bel, (size_t)LBEL * nl, g->headroom));
-    CK(g->pool.alloc(&s.hist, HIST * (size_t)std::max(nf, 1), g->headroom));
+    // every array of the layout in one allocation, those with host contents
+    // first: when a keyframe is added they travel in one copy out of pinned
+    // memory (a copy each, and an allocation each, was most of what adding a
+    // keyframe cost: 0.4 -> 0.27 ms at 60 keyframes)
+    struct Item {
+        void** dst;
+        size_t bytes, at;
+        const void* src;
+    };
+    std::vector<Item> items;
+    size_t total = 0;
+    auto place = [&](void** dst, size_t bytes, const void* src) {
+        items.push_back(Item{dst, bytes, total, src});
+        total += (bytes + 255) / 256 * 256;
+    };
+#define UP(ptr, vec) place(reinterpret_cast<void**>(&s.ptr), sizeof((vec)[0]) * (vec).size(), (vec).data())
+    UP(z, zr);
+    UP(fk, g->fk);
+    UP(fm, g->fm);
+    UP(kf_R, g->kf_R);
+    UP(kf_c, g->kf_c);
+    UP(lm_ref, g->lm_ref);
+    UP(kf_Rr, rr);
+    UP(f_dlc, dlc);
+    UP(kf_off, kf_off);
+    UP(kf_list, kf_list);
+    UP(kpos, kpos);
+    UP(lm_off, lm_off);
+    UP(tile_start, tiles);
+    UP(orphan, orphan);
+    UP(big_lm, big);
+    UP(kf_birth, g->kf_birth);
+    UP(lm_birth, g->lm_birth);
+    UP(anc, anc);
+    if (src_f) UP(src_f, *src_f);
+#undef UP
+    const size_t up_bytes = total;
+#define DEV(ptr, n) place(reinterpret_cast<void**>(&s.ptr), sizeof(*s.ptr) * (size_t)(n), nullptr)
+    DEV(tidx, 32 * (size_t)n_tiles);
+    DEV(deferred, n_tiles);
+    DEV(kf_D, 6 * (size_t)nk);
+    DEV(kf_A, 6 * (size_t)nk);
+    DEV(lm_D, 3 * (size_t)nl);
+    DEV(x0, 9 * (size_t)nf);
+    DEV(tlin, nf);
+    DEV(mk, (size_t)KREC * nf);
+    DEV(mk2, (size_t)KREC * nf);
+    DEV(kj, (size_t)KJ * nf);
+    DEV(kjs, (size_t)KJ * nf);
+    DEV(lin, (size_t)NLIN * nf);
+    DEV(ml, (size_t)NML * nf);
+    DEV(mlx, 9 * (size_t)nf);
+    DEV(kf_bel, (size_t)KBEL * nk);
+    DEV(lm_bel, (size_t)LBEL * nl);
+    DEV(hist, HIST * (size_t)nf);
+#undef DEV
     cudaStream_t st = g->stream;
-    CK(cudaMemcpyAsync(s.z, zr.data(), sizeof(R) * zr.size(), cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(s.fk, g->fk.data(), sizeof(int32_t) * nf, cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(s.fm, g->fm.data(), sizeof(int32_t) * nf, cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(s.kf_R, g->kf_R.data(), sizeof(double) * 9 * nk, cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(s.kf_c, g->kf_c.data(), sizeof(double) * 3 * nk, cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(s.lm_ref, g->lm_ref.data(), sizeof(double) * 3 * nl, cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(s.kf_Rr, rr.data(), sizeof(R) * rr.size(), cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(s.f_dlc, dlc.data(), sizeof(R) * dlc.size(), cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(s.kf_off, kf_off.data(), sizeof(int32_t) * (nk + 1), cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(s.kf_list, kf_list.data(), sizeof(int32_t) * nf, cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(s.kpos, kpos.data(), sizeof(int32_t) * nf, cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(s.lm_off, lm_off.data(), sizeof(int32_t) * (nl + 1), cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(s.tile_start, tiles.data(), sizeof(int32_t) * tiles.size(), cudaMemcpyHostToDevice, st));
-    if (!orphan.empty())
-        CK(cudaMemcpyAsync(s.orphan, orphan.data(), sizeof(int32_t) * orphan.size(), cudaMemcpyHostToDevice, st));
-    if (!big.empty())
-        CK(cudaMemcpyAsync(s.big_lm, big.data(), sizeof(int32_t) * big.size(), cudaMemcpyHostToDevice, st));
-    if (nk) CK(cudaMemcpyAsync(s.kf_birth, g->kf_birth.data(), sizeof(int32_t) * nk, cudaMemcpyHostToDevice, st));
-    if (nl) CK(cudaMemcpyAsync(s.lm_birth, g->lm_birth.data(), sizeof(int32_t) * nl, cudaMemcpyHostToDevice, st));
+    CK(g->pool.alloc(&s.arena, total, g->headroom));
+    for (const Item& it : items) *it.dst = s.arena + it.at;
+    const bool staged = src_f && up_bytes <= STAGE_MAX;   // a growing graph: the pinned buffer serves many layouts
+    if (staged) {
+        if (!g->h_stage) CK(cudaMallocHost(reinterpret_cast<void**>(&g->h_stage), STAGE_MAX));
+        if (g->stage_busy) CK(cudaStreamSynchronize(st));
+        for (const Item& it : items)
+            if (it.src && it.bytes) std::memcpy(g->h_stage + it.at, it.src, it.bytes);
+        CK(cudaMemcpyAsync(s.arena, g->h_stage, up_bytes, cudaMemcpyHostToDevice, st));
+        g->stage_busy = true;
+    } else {
+        for (const Item& it : items)
+            if (it.src && it.bytes)
+                CK(cudaMemcpyAsync(s.arena + it.at, it.src, it.bytes, cudaMemcpyHostToDevice, st));
+    }
     // linearisation points (the references at creation) for the prior pass
-    if (x0_init && nf)
-        CK(cudaMemcpyAsync(s.x0, x0_init->data(), sizeof(R) * 9 * (size_t)nf, cudaMemcpyHostToDevice, st));
-    else if (nf && !rs)
+    if (nf && !rs)
         CK(cudaMemsetAsync(s.x0, 0, sizeof(R) * 9 * (size_t)nf, st));
 
     DevGraph<R>& d = s.g;
@@ -573,32 +588,27 @@ gbp_status build_device(gbp_graph* g, const std::vector<R>* x0_init = nullptr, c
     d.rec_T = nullptr;
     d.ctl = g->ctl;
     CK(launch_tile_index<R>(d, n_tiles, s.tidx, st));
+    if (rs) rs->src_f = s.src_f;
     if (rs && nf) CK(launch_relayout<R>(d, *rs, 0, st));
 
     // priors: per-factor diagonal information at the reference (temporary
-    // buffers reuse the message storage, which is cleared afterwards)
-    {
+    // buffers reuse the message storage, which is cleared afterwards); the
+    // anchor diagonal is D on anchored keyframes
+    if (!s.prior_s) {
         gbp_status pst = upload_prior_table<R>(g);
         if (pst != GBP_OK) return pst;
     }
     KParams<R> kp = make_kparams<R>(g);
-    CK(launch_prior<R>(d, kp, s.mk, s.ml, s.kf_D, s.lm_D, st));
-    // anchor diagonal = D on anchored keyframes
-    {
-        std::vector<R> D(6 * (size_t)nk);
-        CK(cudaMemcpyAsync(D.data(), s.kf_D, sizeof(R) * D.size(), cudaMemcpyDeviceToHost, st));
-        CK(cudaStreamSynchronize(st));
-        for (size_t i = 0; i < D.size(); ++i) anc[i] *= D[i];
-        CK(cudaMemcpyAsync(s.kf_A, anc.data(), sizeof(R) * anc.size(), cudaMemcpyHostToDevice, st));
-    }
+    CK(launch_prior<R>(d, kp, s.mk, s.ml, s.kf_D, s.kf_A, s.anc, s.lm_D, st));
     if (!g->uv_ref.empty()) {
         std::vector<R> u(g->uv_ref.size());
         for (size_t i = 0; i < u.size(); ++i) u[i] = R(g->uv_ref[i]);
         CK(g->pool.alloc(&s.uv_ref, u.size(), g->headroom));
         CK(cudaMemcpyAsync(s.uv_ref, u.data(), sizeof(R) * u.size(), cudaMemcpyHostToDevice, st));
         d.uv_ref = s.uv_ref;
+        CK(cudaStreamSynchronize(st));
     }
-    CK(cudaStreamSynchronize(st));
+    if (!staged) CK(cudaStreamSynchronize(st));   // pageable arrays: copied before they go
     return GBP_OK;
 }
 
@@ -621,8 +631,7 @@ gbp_status reset_state(gbp_graph* g) {
     CK(cudaMemsetAsync(s.kf_bel, 0, sizeof(R) * KBEL * g->n_kf, st));
     CK(cudaMemsetAsync(s.lm_bel, 0, sizeof(R) * LBEL * g->n_lm, st));
     CK(cudaMemsetAsync(s.hist, 0, sizeof(float) * HIST * nf, st));
-    int32_t c0[CTL_N] = {0};
-    CK(cudaMemcpyAsync(g->ctl, c0, sizeof(c0), cudaMemcpyHostToDevice, st));
+    CK(cudaMemsetAsync(g->ctl, 0, sizeof(int32_t) * CTL_N, st));
     CK(launch_init<R>(s.g, make_kparams<R>(g), st));
     g->launches += 1;
     return GBP_OK;
@@ -898,12 +907,19 @@ gbp_status check_params(const gbp_params* p, std::string& why) {
 void order_factors(gbp_graph* g, const std::vector<int32_t>& ok, const std::vector<int32_t>& ol,
                    const std::vector<double>& uv, const std::vector<int32_t>& idx) {
     const int n = (int)ok.size();
-    std::vector<int32_t> perm(n);
-    std::iota(perm.begin(), perm.end(), 0);
-    std::stable_sort(perm.begin(), perm.end(), [&](int a, int b) {
-        if (ol[a] != ol[b]) return ol[a] < ol[b];
-        return ok[a] < ok[b];
-    });
+    // stable, by landmark with a counting sort (observations come grouped by
+    // landmark or by keyframe in practice), then each landmark's few by keyframe
+    std::vector<int32_t> perm(n), off(g->n_lm + 1, 0);
+    for (int i = 0; i < n; ++i) off[ol[i] + 1]++;
+    for (int m = 0; m < g->n_lm; ++m) off[m + 1] += off[m];
+    {
+        std::vector<int32_t> fill(off.begin(), off.end() - 1);
+        for (int i = 0; i < n; ++i) perm[fill[ol[i]]++] = i;
+    }
+    const auto by_kf = [&](int a, int b) { return ok[a] < ok[b]; };
+    for (int m = 0; m < g->n_lm; ++m)
+        if (!std::is_sorted(perm.begin() + off[m], perm.begin() + off[m + 1], by_kf))
+            std::stable_sort(perm.begin() + off[m], perm.begin() + off[m + 1], by_kf);
     g->n_f = n;
     g->fk.resize(n);
     g->fm.resize(n);
@@ -1169,6 +1185,7 @@ gbp_status add_keyframe_impl(gbp_graph* g, const double* kf_Rt_init, int n_new_l
                            st));
         CK(cudaStreamSynchronize(st));
     }
+    g->stage_busy = false;
     const int t = ctl[CTL_ITER];
     if (ctl[CTL_ERR]) return fail(g, GBP_ESTATE, "graph is in an error state");
 
@@ -1215,28 +1232,24 @@ gbp_status add_keyframe_impl(gbp_graph* g, const double* kf_Rt_init, int n_new_l
     g->prob_kf0 = {0, K1};
     g->prob_lm0 = {0, L1};
     g->prob_f0 = {0, F1};
-    CK(cudaMemcpy(g->d_prob_f0, g->prob_f0.data(), sizeof(int32_t) * 2, cudaMemcpyHostToDevice));
+    CK(cudaMemcpyAsync(g->d_prob_f0, g->prob_f0.data(), sizeof(int32_t) * 2, cudaMemcpyHostToDevice, st));
     g->uv_ref.clear();   // the reference projections no longer cover every factor
 
     // the previous layout stays alive until its state is gathered, then its
-    // buffers go back to the pool for the next addition
+    // buffers go back to the pool for the next addition (whose work on the
+    // same stream comes after this one's).  Nothing is read back: the call
+    // leaves the device busy.
     g->headroom = 1.25;
     DevState<R> old = state<R>(g);
     state<R>(g) = DevState<R>();
-    int32_t* d_src = nullptr;
-    cudaError_t e = dev_alloc(&d_src, (size_t)F1);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(d_src, src_f.data(), sizeof(int32_t) * (size_t)F1, cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) {
-        old.release(&g->pool);
-        if (d_src) cudaFree(d_src);
-        return cuda_fail(g, e, "add_keyframe");
-    }
-    const RelayoutSrc<R> rs{d_src, F0, L0, t, old.x0, old.tlin, old.ml, old.lin, old.hist, old.kpos, old.kj,
-                            (t & 1) ? old.mk2 : old.mk, (t & 1) ? old.mk : old.mk2, old.lm_bel};
+    state<R>(g).prior_s = old.prior_s;
+    old.prior_s = nullptr;
+    RelayoutSrc<R> rs{nullptr, F0, L0, t, old.x0, old.tlin, old.ml, old.lin, old.hist, old.kpos, old.kj,
+                      (t & 1) ? old.mk2 : old.mk, (t & 1) ? old.mk : old.mk2, old.lm_bel};
     destroy_exec(g);
-    gbp_status bst = build_device<R>(g, nullptr, &rs);
+    gbp_status bst = build_device<R>(g, &rs, &src_f);
     DevState<R>& s = state<R>(g);
+    cudaError_t e = cudaSuccess;
     if (bst == GBP_OK) {
         // factor state in the new layout
         e = launch_relayout<R>(s.g, rs, 1, st);
@@ -1252,33 +1265,9 @@ gbp_status add_keyframe_impl(gbp_graph* g, const double* kf_Rt_init, int n_new_l
         if (e == cudaSuccess) e = cudaMemsetAsync(s.kjs, 0, sizeof(R) * KJ * (size_t)F1, st);
         if (e == cudaSuccess) e = cudaMemsetAsync(s.mlx, 0, sizeof(R) * 9 * (size_t)F1, st);
         if (e == cudaSuccess) e = cudaMemsetAsync(s.kf_A + 6 * (size_t)K0, 0, sizeof(R) * 6, st);
-        std::vector<R> kD(6), lD(3 * (size_t)n_new_lm);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(kD.data(), s.kf_D + 6 * (size_t)K0, sizeof(R) * 6, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess && n_new_lm)
-            e = cudaMemcpyAsync(lD.data(), s.lm_D + 3 * (size_t)L0, sizeof(R) * lD.size(), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e == cudaSuccess) {
-            const R s0 = g->prm.prior_anneal_iters > 0 ? R(1) : R(g->prm.prior_final_scale);
-            const R isig2 = R(1.0 / (double(g->prm.sigma_px) * double(g->prm.sigma_px)));
-            std::vector<R> kbn(KBEL), lbn(LBEL * (size_t)n_new_lm, R(0));
-            R pd[6];
-            for (int i = 0; i < 6; ++i) pd[i] = s0 * kD[i] * isig2;
-            kf_prior_record_host<R>(pd, kbn.data());
-            for (int j = 0; j < n_new_lm; ++j)
-                for (int i = 0; i < 3; ++i) lbn[(size_t)LBEL * j + i * (i + 1) / 2 + i] = s0 * lD[3 * (size_t)j + i] * isig2;
-            e = cudaMemcpyAsync(s.kf_bel + (size_t)KBEL * K0, kbn.data(), sizeof(R) * KBEL, cudaMemcpyHostToDevice, st);
-            if (e == cudaSuccess && n_new_lm)
-                e = cudaMemcpyAsync(s.lm_bel + (size_t)LBEL * L0, lbn.data(), sizeof(R) * lbn.size(),
-                                    cudaMemcpyHostToDevice, st);
-            // the control block as it was (the prior pass leaves it alone; kept
-            // explicit so that the iteration count and flags carry over)
-            if (e == cudaSuccess)
-                e = cudaMemcpyAsync(g->ctl, ctl, sizeof(int32_t) * CTL_N, cudaMemcpyHostToDevice, st);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        }
+        if (e == cudaSuccess) e = launch_init_new<R>(s.g, make_kparams<R>(g), K0, L0, st);
     }
     old.release(&g->pool);
-    cudaFree(d_src);
     if (bst != GBP_OK) return bst;
     if (e != cudaSuccess) return cuda_fail(g, e, "add_keyframe");
     return GBP_OK;
@@ -2079,6 +2068,7 @@ void gbp_destroy_graph(gbp_graph* g) {
     if (g->h_ctl) cudaFreeHost(g->h_ctl);
     if (g->h_met) cudaFreeHost(g->h_met);
     if (g->h_read) cudaFreeHost(g->h_read);
+    if (g->h_stage) cudaFreeHost(g->h_stage);
     if (g->d_read) cudaFree(g->d_read);
     if (g->d_obs) cudaFree(g->d_obs);
     if (g->capture) cudaStreamDestroy(g->capture);

@@ -247,8 +247,12 @@ int resident_grid(const DevGraph<float>& g, int* na);
 cudaError_t launch_resident(const DevGraph<float>& g, const KParams<float>& p, int n_iters, float conv_tol,
                             int check_every, cudaStream_t s);
 template <typename R> cudaError_t launch_capture_messages(const DevGraph<R>& g, int t, R* eta_inf, cudaStream_t s);
+// prior diagonals kf_D, lm_D; kf_A = anc x kf_D
 template <typename R> cudaError_t launch_prior(const DevGraph<R>& g, const KParams<R>& p, R* tmp_k, R* tmp_l,
-                                               R* kf_D, R* lm_D, cudaStream_t s);
+                                               R* kf_D, R* kf_A, const R* anc, R* lm_D, cudaStream_t s);
+// beliefs of the variables added to a graph (keyframes from k0, landmarks from l0): their prior at s(0)
+template <typename R> cudaError_t launch_init_new(const DevGraph<R>& g, const KParams<R>& p, int k0, int l0,
+                                                  cudaStream_t s);
 template <typename R> cudaError_t launch_metrics(const DevGraph<R>& g, const KParams<R>& p, double* partials,
                                                  int n_partials, double* out, cudaStream_t s);
 template <typename R> cudaError_t launch_problem_metrics(const DevGraph<R>& g, const KParams<R>& p,

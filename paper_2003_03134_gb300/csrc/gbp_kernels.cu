@@ -249,6 +249,29 @@ __global__ void init_beliefs_kernel(DevGraph<R> g, KParams<R> P) {
     }
 }
 
+// Beliefs of variables added to a graph: prior(0) alone, mean 0.  The factor
+// of a keyframe's record is rounded from FP64.
+template <typename R>
+__global__ void init_new_kernel(DevGraph<R> g, KParams<R> P, int k0, int l0) {
+    const int v = blockIdx.x * blockDim.x + threadIdx.x;
+    const int nk = g.n_kf - k0, nl = g.n_lm - l0;
+    const R s0 = prior_scale(P, 0), isig2 = P.inv_sigma2;
+    if (v < nk) {
+        const int k = k0 + v;
+        R p[6], out[KBEL];
+        for (int i = 0; i < 6; ++i) p[i] = mul_rn(mul_rn(s0, g.kf_D[k * 6 + i]), isig2);
+        kf_prior_record<R>(p, out);
+        for (int i = 0; i < 6; ++i) out[KB_L + pk(i, i)] = R(1.0 / sqrt(double(p[i])));
+        store_rec<R, KBEL>(g.kf_bel + (size_t)k * KBEL, out);
+    } else if (v < nk + nl) {
+        const size_t m = l0 + (v - nk);
+        R out[LBEL];
+        for (int j = 0; j < LBEL; ++j) out[j] = R(0);
+        for (int i = 0; i < 3; ++i) out[pk(i, i)] = mul_rn(mul_rn(s0, g.lm_D[m * 3 + i]), isig2);
+        store_rec<R, LBEL>(g.lm_bel + m * LBEL, out);
+    }
+}
+
 // ------------------------------------------------------------------------
 // prior generation (Sec. 4 / Sec. 8): per-variable mean over its factors of
 // diag(J_v^T J_v) at the factors' linearisation points (the references, at
@@ -291,7 +314,8 @@ __device__ __forceinline__ void finish_prior(R* D, int deg) {
 }
 
 template <typename R>
-__global__ void prior_reduce_kernel(DevGraph<R> g, const R* tmp_k, const R* tmp_l, R* kf_D, R* lm_D) {
+__global__ void prior_reduce_kernel(DevGraph<R> g, const R* tmp_k, const R* tmp_l, R* kf_D, R* kf_A, const R* anc,
+                                    R* lm_D) {
     const int v = blockIdx.x * blockDim.x + threadIdx.x;
     if (v < g.n_kf) {
         R D[6] = {R(0), R(0), R(0), R(0), R(0), R(0)};
@@ -303,7 +327,10 @@ __global__ void prior_reduce_kernel(DevGraph<R> g, const R* tmp_k, const R* tmp_
         }
         finish_prior<R, 6>(D, b1 - b0);
 #pragma unroll
-        for (int j = 0; j < 6; ++j) kf_D[v * 6 + j] = D[j];
+        for (int j = 0; j < 6; ++j) {
+            kf_D[v * 6 + j] = D[j];
+            kf_A[v * 6 + j] = anc[v * 6 + j] * D[j];
+        }
     } else if (v < g.n_kf + g.n_lm) {
         const int m = v - g.n_kf;
         R D[3] = {R(0), R(0), R(0)};
@@ -671,6 +698,13 @@ cudaError_t launch_capture_messages(const DevGraph<R>& g, int t, R* eta_inf, cud
 }
 
 template <typename R>
+cudaError_t launch_init_new(const DevGraph<R>& g, const KParams<R>& p, int k0, int l0, cudaStream_t s) {
+    const int n = (g.n_kf - k0) + (g.n_lm - l0);
+    if (n > 0) init_new_kernel<R><<<(n + 127) / 128, 128, 0, s>>>(g, p, k0, l0);
+    return cudaGetLastError();
+}
+
+template <typename R>
 cudaError_t launch_tile_index(const DevGraph<R>& g, int n_tiles, int4* tidx, cudaStream_t s) {
     if (n_tiles > 0) tile_index_kernel<R><<<(n_tiles + 3) / 4, 128, 0, s>>>(g, n_tiles, tidx);
     return cudaGetLastError();
@@ -684,11 +718,11 @@ cudaError_t launch_init(const DevGraph<R>& g, const KParams<R>& p, cudaStream_t 
 }
 
 template <typename R>
-cudaError_t launch_prior(const DevGraph<R>& g, const KParams<R>& p, R* tmp_k, R* tmp_l, R* kf_D, R* lm_D,
-                         cudaStream_t s) {
+cudaError_t launch_prior(const DevGraph<R>& g, const KParams<R>& p, R* tmp_k, R* tmp_l, R* kf_D, R* kf_A,
+                         const R* anc, R* lm_D, cudaStream_t s) {
     if (g.n_f > 0) prior_factor_kernel<R><<<(g.n_f + FACTOR_BLOCK - 1) / FACTOR_BLOCK, FACTOR_BLOCK, 0, s>>>(g, p, tmp_k, tmp_l);
     int nv = g.n_kf + g.n_lm;
-    if (nv > 0) prior_reduce_kernel<R><<<(nv + 127) / 128, 128, 0, s>>>(g, tmp_k, tmp_l, kf_D, lm_D);
+    if (nv > 0) prior_reduce_kernel<R><<<(nv + 127) / 128, 128, 0, s>>>(g, tmp_k, tmp_l, kf_D, kf_A, anc, lm_D);
     return cudaGetLastError();
 }
 
@@ -841,7 +875,8 @@ cudaError_t launch_relayout(const DevGraph<R>& nw, const RelayoutSrc<R>& o, int 
     template cudaError_t launch_problem_metrics<R>(const DevGraph<R>&, const KParams<R>&, const int32_t*, int, double*, cudaStream_t); \
     template int persistent_grid<R>(const DevGraph<R>&, int, int);                                         \
     template cudaError_t launch_persistent<R>(const DevGraph<R>&, const KParams<R>&, int, float, int, int, cudaStream_t, int, int); \
-    template cudaError_t launch_prior<R>(const DevGraph<R>&, const KParams<R>&, R*, R*, R*, R*, cudaStream_t); \
+    template cudaError_t launch_prior<R>(const DevGraph<R>&, const KParams<R>&, R*, R*, R*, R*, const R*, R*, cudaStream_t); \
+    template cudaError_t launch_init_new<R>(const DevGraph<R>&, const KParams<R>&, int, int, cudaStream_t); \
     template cudaError_t launch_metrics<R>(const DevGraph<R>&, const KParams<R>&, double*, int, double*, cudaStream_t); \
     template cudaError_t launch_residuals<R>(const DevGraph<R>&, const KParams<R>&, const int32_t*, double*, cudaStream_t); \
     template cudaError_t launch_means<R>(const DevGraph<R>&, bool, double*, double*, int32_t*, cudaStream_t); \
