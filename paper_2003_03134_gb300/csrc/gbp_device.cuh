@@ -40,7 +40,9 @@ __device__ __forceinline__ R rcp(R x) {
 }
 
 // (sqrt(s), 1/sqrt(s)) for s > 0.  FP32: hardware reciprocal square root
-// refined by one Newton-Raphson step y <- y (3 - s y^2) / 2; FP64: exact.
+// refined by one Newton-Raphson step y <- y (3 - s y^2) / 2; FP64: the
+// library's reciprocal square root (1 ulp, as the quotient of a rounded root:
+// one dependent sequence instead of a square root's and a division's).
 template <typename R>
 __device__ __forceinline__ void sqrt_pair(R s, R& d, R& id) {
     if constexpr (sizeof(R) == 4) {
@@ -49,8 +51,8 @@ __device__ __forceinline__ void sqrt_pair(R s, R& d, R& id) {
         id = y;
         d = s * y;
     } else {
-        d = sqrt(fmax(s, R(0)));
-        id = R(1) / d;
+        id = rsqrt(fmax(s, R(0)));
+        d = s * id;
     }
 }
 
@@ -1038,8 +1040,17 @@ __device__ __forceinline__ R warp_sum(R v) {
 template <typename R>
 __device__ __forceinline__ void two_sum_add(R& hi, R& lo, R x) {
     const R s = hi + x;
-    const R bp = s - hi;
-    lo += (hi - (s - bp)) + (x - bp);
+    if constexpr (sizeof(R) == 8) {
+        // FP64 additions are what the tree costs: with the operand of larger
+        // exponent known (compared as integers) Dekker's two suffice for the
+        // same exact error
+        const bool ge = (__double2hiint(hi) & 0x7fffffff) >= (__double2hiint(x) & 0x7fffffff);
+        const R big = ge ? hi : x, small = ge ? x : hi;
+        lo += small - (s - big);
+    } else {
+        const R bp = s - hi;
+        lo += (hi - (s - bp)) + (x - bp);
+    }
     hi = s;
 }
 
