@@ -79,7 +79,8 @@ typedef struct {
     float   fp64_pivot_ratio;   /* FP32 Cholesky with min/max pivot below this is redone in FP64; 1e-6 */
     int32_t precision_mode;     /* 0: FP32 + FP64 fallback, 1: FP32 only, 2: FP64 throughout        */
     int32_t linear;             /* 1: never relinearise (linear GBP at the initial point)          */
-    int32_t launch_mode;        /* 0: auto (gbp_autotune on first use; a graph whose device, storage,
+    int32_t launch_mode;        /* 0: auto (by size where one configuration is known to be the fastest,
+                                   else gbp_autotune on first use; a graph whose device, storage,
                                    precision and damping modes and sizes match one already tuned in
                                    this process takes that graph's choice), 1: one persistent launch per
                                    gbp_iterate call with a grid barrier between phases, 2: one launch
@@ -290,7 +291,8 @@ typedef struct {
     int32_t n_candidates;           /* candidates timed by the last gbp_autotune                   */
     int32_t cand_mode[GBP_MAX_TUNING_CANDIDATES];
     int32_t cand_shape[GBP_MAX_TUNING_CANDIDATES];
-    double  cand_ms[GBP_MAX_TUNING_CANDIDATES];   /* mean ms per iteration, -1: could not launch  */
+    double  cand_ms[GBP_MAX_TUNING_CANDIDATES];   /* mean ms per iteration, -1: could not launch,
+                                                     0: taken by size without timing              */
 } gbp_tuning;
 
 /* The launch configuration in use and the candidates of the last

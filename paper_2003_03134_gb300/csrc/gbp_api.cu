@@ -101,7 +101,7 @@ struct DevState {
     int32_t* kf_list = nullptr;
     int32_t* kpos = nullptr;
     int32_t* lm_off = nullptr;
-    int32_t* tile_start = nullptr;
+    int32_t* tf = nullptr;
     int4* tidx = nullptr;
     int32_t* big_lm = nullptr;
     int32_t* deferred = nullptr;
@@ -362,10 +362,18 @@ gbp_status build_device(gbp_graph* g, RelayoutSrc<R>* rs = nullptr, const std::v
             kf_list[kpos[f]] = f;
         }
     }
-    // warp tiles: consecutive whole landmarks, at most 32 factors per tile;
-    // a landmark with more factors gets tiles of its own and its belief is
-    // formed in the belief phase.  Variables without factors are orphans.
-    std::vector<int32_t> tiles(1, 0), orphan, big;
+    // warp tiles of whole landmarks, at most 32 factors each; a landmark with
+    // more factors gets tiles of its own and its belief is formed in the
+    // belief phase.  Variables without factors are orphans.  A tile costs the
+    // same whatever it holds, so landmarks are packed best-fit into a few open
+    // tiles (in landmark order; a tile's landmarks stay within a short stretch
+    // of the factor arrays): 30.9 factors a tile at paper scale, 27.4 when a
+    // tile takes what comes next (566 tiles instead of 638, so the resident
+    // kernel holds them with 4 warps a block: 8.5 -> 7.2 us an iteration; 2M
+    // factors 186 -> 178 us).  Which tile a landmark is in changes no sum.
+    constexpr int OPEN_TILES = 8;
+    std::vector<int32_t> tf, tile_lm, orphan, big;   // tile_lm: a landmark of each tile
+    tf.reserve(32 * ((size_t)nf / 31 + 16));
     for (int v = 0; v < nk; ++v)
         if (kf_off[v + 1] == kf_off[v]) orphan.push_back(v);
     {
@@ -377,40 +385,47 @@ gbp_status build_device(gbp_graph* g, RelayoutSrc<R>* rs = nullptr, const std::v
             breaks.push_back(g->part_lm1);
         }
         std::sort(breaks.begin(), breaks.end());
-        int cur = 0;
+        struct Open {
+            size_t tile;
+            int used;
+        };
+        std::vector<Open> open;   // oldest first
+        auto new_tile = [&](int m) {
+            tf.resize(tf.size() + 32, -1);
+            tile_lm.push_back(m);
+            return tile_lm.size() - 1;
+        };
         size_t next_brk = 0;
         for (int m = 0; m < nl; ++m) {
             const int lo = lm_off[m], hi = lm_off[m + 1], d = hi - lo;
-            while (next_brk < breaks.size() && breaks[next_brk] <= m) {
-                if (breaks[next_brk] == m && cur > 0) {
-                    tiles.push_back(lo);
-                    cur = 0;
-                }
-                ++next_brk;
-            }
+            for (; next_brk < breaks.size() && breaks[next_brk] <= m; ++next_brk) open.clear();
             if (d == 0) {
                 orphan.push_back(nk + m);
                 continue;
             }
             if (d > 32) {
-                if (cur > 0) {
-                    tiles.push_back(lo);
-                    cur = 0;
+                for (int x = lo; x < hi; x += 32) {
+                    const size_t t = new_tile(m);
+                    for (int f = x; f < std::min(hi, x + 32); ++f) tf[32 * t + (f - x)] = f;
                 }
-                for (int x = lo + 32; x < hi; x += 32) tiles.push_back(x);
-                tiles.push_back(hi);
                 big.push_back(m);
                 continue;
             }
-            if (cur + d > 32) {
-                tiles.push_back(lo);
-                cur = 0;
+            int best = -1;
+            for (size_t o = 0; o < open.size(); ++o)
+                if (open[o].used + d <= 32 && (best < 0 || open[o].used > open[(size_t)best].used)) best = (int)o;
+            if (best < 0) {
+                if (open.size() == OPEN_TILES) open.erase(open.begin());
+                open.push_back(Open{new_tile(m), 0});
+                best = (int)open.size() - 1;
             }
-            cur += d;
+            Open& o = open[(size_t)best];
+            for (int f = lo; f < hi; ++f) tf[32 * o.tile + o.used + (f - lo)] = f;
+            o.used += d;
+            if (o.used == 32) open.erase(open.begin() + best);
         }
-        if (cur > 0) tiles.push_back(nf);
     }
-    const int n_tiles = (int)tiles.size() - 1;
+    const int n_tiles = (int)tile_lm.size();
     std::vector<R> zr(2 * (size_t)nf), anc(6 * (size_t)nk, R(0));
     for (size_t i = 0; i < zr.size(); ++i) zr[i] = R(g->z[i]);
     // the linearisation's references in R: the rotation rounded, and each
@@ -452,7 +467,7 @@ gbp_status build_device(gbp_graph* g, RelayoutSrc<R>* rs = nullptr, const std::v
     UP(kf_list, kf_list);
     UP(kpos, kpos);
     UP(lm_off, lm_off);
-    UP(tile_start, tiles);
+    UP(tf, tf);
     UP(orphan, orphan);
     UP(big_lm, big);
     UP(kf_birth, g->kf_birth);
@@ -516,7 +531,7 @@ gbp_status build_device(gbp_graph* g, RelayoutSrc<R>* rs = nullptr, const std::v
     d.kf_list = s.kf_list;
     d.kpos = s.kpos;
     d.lm_off = s.lm_off;
-    d.tile_start = s.tile_start;
+    d.tf = s.tf;
     d.tidx = s.tidx;
     d.big_lm = s.big_lm;
     d.deferred = s.deferred;
@@ -536,7 +551,7 @@ gbp_status build_device(gbp_graph* g, RelayoutSrc<R>* rs = nullptr, const std::v
         // at the range's ends); its split landmarks likewise
         int t0 = 0, t1 = 0;
         for (int t = 0; t < n_tiles; ++t) {
-            const int lm = g->fm[tiles[t]];
+            const int lm = tile_lm[t];
             if (lm < g->part_lm0) t0 = t + 1;
             if (lm < g->part_lm1) t1 = t + 1;
         }
@@ -1069,8 +1084,7 @@ gbp_status iterate_phases(gbp_graph* g, int n, float conv_tol, int* done_out) {
 gbp_status iterate_persistent(gbp_graph* g, int n, float conv_tol, int* done_out) {
     const int dm = g->prm.damping_mode;
     const int ps = persistent_shape(g);
-    int na = 0;
-    const bool resident = !g->storage && dm == 0 && resident_grid(g->sf.g, &na) > 0;
+    const bool resident = !g->storage && dm == 0 && resident_grid(g->sf.g) > 0;
     const int grid = resident ? 1 : g->storage ? persistent_grid<double>(g->sd.g, dm, ps) : persistent_grid<float>(g->sf.g, dm, ps);
     if (grid <= 0) return fail(g, GBP_ECUDA, "persistent launch: occupancy query failed");
     cudaError_t e = resident
@@ -1612,6 +1626,38 @@ void tune_cache_store(const gbp_graph* g) {
 }
 }  // namespace
 
+// Sizes at which one configuration won every measurement by more than the
+// candidates' own spread, so that a graph's first gbp_iterate need not time
+// them (16 iterations of 7 candidates, and a copy of the state: 2.7 ms at
+// paper scale, 35 ms at 2M factors, more than the solve itself):
+//   * the resident kernel with one keyframe a block (see gbp_resident.cu):
+//     328 tiles 6.1 us against 9.2 of the best per-phase shape, 591 6.6 / 9.5,
+//     624 8.1 / 9.8, 985 9.0 / 10.2, 1200 10.3 / 11.1; it takes up to 1216;
+//   * at four chips' worth of warps and more (4 x 2432 tiles) the deferring
+//     factor kernel: 10510 tiles 39.5 us against 44.6, 15766 60.4 / 72.0; at
+//     7883 35.0 / 37.0, at 5255 26.0 / 25.0, so between the two lines the
+//     candidates are timed.
+// Recorded as one candidate with time 0.
+constexpr int RULE_LARGE_TILES = 4 * 2432;
+
+static bool choose_by_rule(gbp_graph* g) {
+    if (!tunable(g)) return false;
+    const DevGraph<float>& d = g->sf.g;
+    const int blocks = resident_grid(d);
+    int mode = 0, shape = 0;
+    if (blocks > 0 && d.n_kf <= blocks) mode = 1;
+    else if (d.n_tiles >= RULE_LARGE_TILES) { mode = 2; shape = 4; }
+    if (!mode) return false;
+    g->tuned_mode = mode;
+    if (mode == 2) g->tuned_fshape = shape;
+    g->tuning.n_candidates = 1;
+    g->tuning.cand_mode[0] = mode;
+    g->tuning.cand_shape[0] = shape;
+    g->tuning.cand_ms[0] = 0.0;
+    destroy_exec(g);   // a graph recorded before with the default shapes
+    return true;
+}
+
 gbp_status gbp_iterate(gbp_graph* g, int32_t n_iters, int32_t* iters_done) {
     if (iters_done) *iters_done = 0;
     if (!g) return GBP_EINVAL;
@@ -1624,7 +1670,7 @@ gbp_status gbp_iterate(gbp_graph* g, int32_t n_iters, int32_t* iters_done) {
         return fail(g, GBP_ESTATE, "damping_mode 1 needs a network (gbp_set_damping_model)");
     int mode = g->prm.launch_mode;
     if (mode == 0) {
-        if (!g->tuned_mode && !tune_cache_lookup(g)) {
+        if (!g->tuned_mode && !tune_cache_lookup(g) && !choose_by_rule(g)) {
             st = gbp_autotune(g, 8, nullptr, nullptr);
             if (st != GBP_OK) return st;
         }

@@ -1400,8 +1400,8 @@ __device__ __forceinline__ void damp_store_fixed(const DevGraph<R>& g, const KPa
 }
 
 // ------------------------------------------------------------------------
-// Phase A: one warp, one tile of whole landmarks (at most 32 factors,
-// consecutive in landmark order), one lane per factor.  For each factor:
+// Phase A: one warp, one tile of whole landmarks (at most 32 factors), one
+// lane per factor.  For each factor:
 //   1. its linearisation at x0 (the basis its stored messages are in);
 //   2. both incoming precisions (Sec. 5): the landmark's as prior(t) plus
 //      the other factors' previous messages (segmented warp scans, no
@@ -1427,14 +1427,13 @@ __device__ __forceinline__ float tile_work(const DevGraph<R>& g, const KParams<R
     constexpr bool FEAT = MODE != DAMP_FIXED;
 
     // Every load of the common path is issued in two waves before anything
-    // is stored: the lane's tile entry and the tile's first factor (wave 1),
+    // is stored: the lane's tile entry and factor (wave 1),
     // then the factor's own entries and what the tile entry indexes (wave 2).
     // A store in between (the first linearisation writes the lin record and
     // the keyframe block) would keep later loads behind it.
     const int4 te = g.tidx[(size_t)tile * 32 + lane];
-    const int ts = g.tile_start[tile];
+    const int f = g.tf[(size_t)tile * 32 + lane];
     const bool active = te.x >= 0;
-    const int f = ts + lane;
     const int m = te.z, k = active ? te.x : 0, slot = te.y;
     const bool whole = (te.w & TIDX_WHOLE) != 0;
     const int seg0 = te.w & 31, seg1 = (te.w >> 8) & 31;
@@ -1817,21 +1816,21 @@ __device__ __forceinline__ float tile_work(const DevGraph<R>& g, const KParams<R
 // and ~45 loads a tile besides the stores), not latency or occupancy: 5
 // blocks per SM (96 registers, 130 bytes spilled) take 7 % longer, bringing
 // later tiles into L2 ahead of their warps 5 % longer, and one dependent load
-// less (the tile entry holds what tile_start led to) is worth 2 %.  Reading
+// less (the tile entry holds what the factor arrays would lead to) is worth
+// 2 %.  Reading
 // the gathered records through L1, so that a record's 16-byte pieces share
 // their 32-byte sectors, took 11 % off, the early messages 6 %, 32-byte loads
 // and stores of the records 5 %.  2M factors, a steady iteration (all
-// kernels): 222 -> 186 us (with a relinearisation test due: 233 -> 205); 690k
-// factors in 32 problems: 95 -> 78 us.
+// kernels): 222 -> 186 us (with a relinearisation test due: 233 -> 205), 178
+// (197) with fuller tiles; 690k factors in 32 problems: 95 -> 78, 75.
 
 __device__ __forceinline__ float tile_work_deferring(const DevGraph<float>& g, const KParams<float>& P, int tile, int t,
                                                      int lane) {
     typedef float R;
     const int n_f = g.n_f;
     const int4 te = g.tidx[(size_t)tile * 32 + lane];
-    const int ts = g.tile_start[tile];
+    const int f = g.tf[(size_t)tile * 32 + lane];
     const bool active = te.x >= 0;
-    const int f = ts + lane;
     const int m = te.z, k = active ? te.x : 0, slot = te.y;
     const bool whole = (te.w & TIDX_WHOLE) != 0;
     const int seg0 = te.w & 31, seg1 = (te.w >> 8) & 31;

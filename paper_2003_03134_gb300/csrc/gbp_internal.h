@@ -44,7 +44,7 @@
 //                                message eta, float SoA (HIST x n_f)
 //   CSR keyframe -> factor list (kf_off, kf_list); landmark -> contiguous
 //   factor range (lm_off), since factors are sorted by landmark; warp tiles
-//   of whole landmarks (tile_start); per-variable arrival counters.
+//   of whole landmarks (tf, tidx).
 // Packed symmetric storage: element (i, j), j <= i, at i*(i+1)/2 + j.
 #pragma once
 #include <cuda_runtime.h>
@@ -123,7 +123,8 @@ struct DevGraph {
     const int32_t* kf_list;   // n_f
     const int32_t* kpos;      // n_f: slot of factor f's keyframe message = its position in kf_list
     const int32_t* lm_off;    // n_lm + 1
-    const int32_t* tile_start;// n_tiles + 1: warp tiles of whole landmarks (<= 32 factors each)
+    const int32_t* tf;        // n_tiles x 32: the factor of each lane of a warp tile (-1: none); a tile holds
+                              // whole landmarks (a landmark with more than 32 factors: parts of it alone)
     const int4* tidx;         // n_tiles x 32, a tile's lanes: keyframe (-1: no factor), slot, landmark, and
                               // the lanes of the landmark's factors in the tile (first, last << 8, TIDX_WHOLE
                               // if they are all of its factors; else the lane itself)
@@ -242,8 +243,8 @@ template <typename R> int persistent_grid(const DevGraph<R>& g, int mode, int sh
 template <typename R> cudaError_t launch_persistent(const DevGraph<R>& g, const KParams<R>& p, int n_iters,
                                                     float conv_tol, int check_every, int grid, cudaStream_t s,
                                                     int mode, int shape);
-// resident kernel (gbp_resident.cu): blocks (0 = not for this graph), factor warps per block in *na
-int resident_grid(const DevGraph<float>& g, int* na);
+// resident kernel (gbp_resident.cu): its blocks (0 = not for this graph)
+int resident_grid(const DevGraph<float>& g);
 cudaError_t launch_resident(const DevGraph<float>& g, const KParams<float>& p, int n_iters, float conv_tol,
                             int check_every, cudaStream_t s);
 template <typename R> cudaError_t launch_capture_messages(const DevGraph<R>& g, int t, R* eta_inf, cudaStream_t s);

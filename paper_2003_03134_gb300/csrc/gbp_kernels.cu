@@ -208,21 +208,23 @@ __global__ void __launch_bounds__(FACTOR_BLOCK, MINB)
     }
 }
 
-// The tile entries (gbp_internal.h) from the factor arrays: a warp per tile.
+// The tile entries (gbp_internal.h) from the tiles' factors: a thread per lane.
+// The lanes of a landmark that lies in one tile (at most 32 factors) follow
+// one another in factor order.
 template <typename R>
 __global__ void __launch_bounds__(128) tile_index_kernel(DevGraph<R> g, int n_tiles, int4* __restrict__ tidx) {
-    const int tile = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (tile >= n_tiles) return;
-    const int ts = g.tile_start[tile], te = g.tile_start[tile + 1], f = ts + lane;
+    const size_t i = (size_t)blockIdx.x * 128 + threadIdx.x;
+    if (i >= (size_t)n_tiles * 32) return;
+    const int lane = threadIdx.x & 31, f = g.tf[i];
     int4 e = make_int4(-1, 0, -1, lane | (lane << 8));
-    if (f < te) {
+    if (f >= 0) {
         e.x = g.fk[f];
         e.y = g.kpos[f];
         e.z = g.fm[f];
-        const int lo = g.lm_off[e.z], hi = g.lm_off[e.z + 1];
-        if (lo >= ts && hi <= te) e.w = (lo - ts) | ((hi - ts - 1) << 8) | TIDX_WHOLE;
+        const int lo = g.lm_off[e.z], n = g.lm_off[e.z + 1] - lo, first = lane - (f - lo);
+        if (n <= 32) e.w = first | ((first + n - 1) << 8) | TIDX_WHOLE;
     }
-    tidx[(size_t)tile * 32 + lane] = e;
+    tidx[i] = e;
 }
 
 // Beliefs of iteration 0: b^0 = prior(0) (+ anchor), mean 0.

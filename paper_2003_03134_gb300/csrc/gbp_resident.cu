@@ -27,6 +27,15 @@
 //
 // The arithmetic is that of tile_work and phase_b_item, expression by
 // expression, so the results are bitwise those of the per-phase kernels.
+//
+// Per iteration (200 iterations from reset, launch included) against the
+// per-phase kernels: 10 keyframes, 17 tiles 4.8-5.1 us against 8.0; 60 and
+// ~250 6.3 / 9.9; 125 and 328 6.1 / 9.2; 125 and 591 6.6 / 9.5; 624 (8 factor
+// warps a block) 8.1 / 9.8, 1200 10.3 / 11.1.  Of 9.1 us with 8 factor warps
+// and a relinearisation somewhere in every iteration (clock64 of one block):
+// the gather of the beliefs 1.3, keyframe side, test and relinearisation 2.3,
+// the arrival and its way to the slowest block's belief warps 1.5, the sums
+// and factorisation 2.4, the barrier and the spread of the blocks 1.6.
 #include "gbp_device.cuh"
 
 #include <algorithm>
@@ -114,7 +123,7 @@ __device__ __forceinline__ void load_state(const DevGraph<float>& g, const KPara
     const size_t n_f = g.n_f;
     const int4 te = g.tidx[(size_t)tile * 32 + lane];
     S.active = te.x >= 0;
-    S.f = g.tile_start[tile] + lane;
+    S.f = g.tf[(size_t)tile * 32 + lane];
     S.k = S.active ? te.x : 0;
     S.slot = te.y;
     S.m = te.z;
@@ -328,8 +337,8 @@ __device__ __forceinline__ float kf_sum(const DevGraph<float>& g, const KParams<
     return tid == 0 ? finish_keyframe<float>(g, P, it.k, it.prior, acc, it.mu_old, g.kf_bel_out) : 0.0f;
 }
 
-// NA factor warps per block (a multiple of 4) and FACTOR_BLOCK belief
-// threads, one block per SM.
+// NA factor warps and FACTOR_BLOCK belief threads per block, one block per
+// SM: 255 registers a thread for NA = 4, 168 (with spills) for 8.
 template <int NA>
 __global__ void __launch_bounds__(NA * 32 + NB_BELIEF, 1)
     resident_kernel(const __grid_constant__ DevGraph<float> g, const __grid_constant__ KParams<float> P, int n_iters,
@@ -541,8 +550,6 @@ __global__ void __launch_bounds__(NA * 32 + NB_BELIEF, 1)
     }
 }
 
-constexpr int NA_SMALL = 4, NA_LARGE = 8;
-
 int sm_count() {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
@@ -550,32 +557,38 @@ int sm_count() {
     return sms;
 }
 
+// Factor warps per block: the fewest that hold the tiles (the more registers
+// each); 0: too many tiles.
+int factor_warps(int n_tiles, int sms) {
+    for (int na : {4, 8})
+        if (n_tiles <= sms * na) return na;
+    return 0;
+}
+
 }  // namespace
 
-// Blocks of the resident kernel for this graph and its factor warps per
-// block (*na); 0 where it does not apply: more tiles than the SMs hold at
-// one block each, a landmark split across tiles or a variable without factors
-// (belief-phase items of their own), the warp mapping of the belief phase, a
-// part of a split graph.
-int resident_grid(const DevGraph<float>& g, int* na) {
+// Blocks of the resident kernel for this graph; 0 where it does not apply:
+// more tiles than the SMs hold at one block each, a landmark split across
+// tiles or a variable without factors (belief-phase items of their own), the
+// warp mapping of the belief phase, a part of a split graph.
+int resident_grid(const DevGraph<float>& g) {
     const int sms = sm_count();
     if (sms <= 0 || g.b_warps != NB_BELIEF / 32 || g.n_big > 0 || g.n_orphan > 0 || g.n_tiles < 1) return 0;
     if (g.tile_off != 0 || g.kf_item_off != 0 || g.kf_item_n != g.n_kf) return 0;
-    if (g.n_tiles > sms * NA_LARGE) return 0;
-    *na = g.n_tiles <= sms * NA_SMALL ? NA_SMALL : NA_LARGE;
-    return std::min(sms, std::max((g.n_tiles + *na - 1) / *na, g.n_kf));
+    const int na = factor_warps(g.n_tiles, sms);
+    return na ? std::min(sms, std::max((g.n_tiles + na - 1) / na, g.n_kf)) : 0;
 }
 
 cudaError_t launch_resident(const DevGraph<float>& g, const KParams<float>& p, int n_iters, float conv_tol,
                             int check_every, cudaStream_t s) {
-    int na = 0;
-    const int grid = resident_grid(g, &na);
+    const int grid = resident_grid(g);
     if (grid <= 0) return cudaErrorInvalidConfiguration;
+    const int na = factor_warps(g.n_tiles, sm_count());
     DevGraph<float> gg = g;
     KParams<float> pp = p;
     void* args[] = {&gg, &pp, &n_iters, &conv_tol, &check_every};
-    const void* fn = na == NA_SMALL ? reinterpret_cast<const void*>(resident_kernel<NA_SMALL>)
-                                    : reinterpret_cast<const void*>(resident_kernel<NA_LARGE>);
+    const void* fn = na == 4 ? reinterpret_cast<const void*>(resident_kernel<4>)
+                             : reinterpret_cast<const void*>(resident_kernel<8>);
     return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(na * 32 + NB_BELIEF), args, 0, s);
 }
 
