@@ -200,6 +200,7 @@ struct gbp_graph {
     bool built = false;
     int tuned_mode = 0;                         // autotuner's choice (1 or 2), 0 = not tuned
     int tuned_fshape = -1, tuned_pshape = -1;   // its launch shapes, -1 = not tuned
+    bool tuned_resident = false;                // the choice was mode 1 with the resident kernel
     // one graph split across ranks (gbp_set_partition): the keyframes and
     // landmarks whose beliefs this graph forms; lm1 < 0 = not split
     int part_kf0 = 0, part_kf1 = -1, part_lm0 = 0, part_lm1 = -1;
@@ -1674,6 +1675,16 @@ gbp_status gbp_iterate(gbp_graph* g, int32_t n_iters, int32_t* iters_done) {
             st = gbp_autotune(g, 8, nullptr, nullptr);
             if (st != GBP_OK) return st;
         }
+        const bool resident = g->tuned_mode == 1 && tunable(g) && resident_grid(g->sf.g) > 0;
+        if (g->tuned_resident && !resident && g->tuned_mode == 1) {
+            // the graph has outgrown the resident kernel (keyframes were
+            // added): per-phase launches in the shape of its size, not the
+            // tile-walking persistent kernel
+            g->tuned_mode = 2;
+            g->tuned_fshape = -1;
+            destroy_exec(g);
+        }
+        g->tuned_resident = resident;
         mode = g->tuned_mode;
     }
     int done = 0;

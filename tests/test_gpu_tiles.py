@@ -61,3 +61,23 @@ def test_persistent_launch_gives_the_per_phase_bits(n_problems, params):
                                                   "held_messages", "fp64_resums")])])
     for a, b in zip(*got):
         assert np.array_equal(a, b)
+
+
+def test_a_stream_that_outgrows_the_resident_kernel():
+    """Automatic launches of a graph that grows from a few keyframes past 1216 tiles (~37k factors): the launch
+    configuration changes on the way, the bits are those of per-phase launches throughout."""
+    init, steps = synth.make_stream(5, n_kf=60, n_lm=6000, start_kf=4)
+    got = []
+    for mode in (0, 2):
+        with gbp.Graph(init, huber_nsigma=2.0, launch_mode=mode) as g:
+            g.iterate(3)
+            used = [g.stats()["launch_mode"]]
+            for s in steps:
+                g.add_keyframe(s.obs_lm, s.obs_uv, n_new_lm=s.n_new_lm,
+                               new_lm_xyz=s.new_lm_true if s.n_new_lm else None)
+                g.iterate(2)
+            used.append(g.stats()["launch_mode"])
+            got.append((used, *g.means(), g.relin_iters()))
+    assert got[0][0] == [1, 2], got[0][0]
+    for a, b in zip(got[0][1:], got[1][1:]):
+        assert np.array_equal(a, b)
