@@ -1571,10 +1571,12 @@ gbp_status gbp_reset(gbp_graph* g) {
         std::any_of(g->lm_birth.begin(), g->lm_birth.end(), [](int32_t b) { return b != 0; })) {
         std::fill(g->kf_birth.begin(), g->kf_birth.end(), 0);
         std::fill(g->lm_birth.begin(), g->lm_birth.end(), 0);
+        // on the graph's stream, behind the arrays that gbp_add_keyframe may still
+        // have on their way there (its upload is not waited for)
         int32_t* kb = g->storage ? g->sd.kf_birth : g->sf.kf_birth;
         int32_t* lb = g->storage ? g->sd.lm_birth : g->sf.lm_birth;
-        if (g->n_kf) CK(cudaMemcpy(kb, g->kf_birth.data(), sizeof(int32_t) * g->n_kf, cudaMemcpyHostToDevice));
-        if (g->n_lm) CK(cudaMemcpy(lb, g->lm_birth.data(), sizeof(int32_t) * g->n_lm, cudaMemcpyHostToDevice));
+        if (g->n_kf) CK(cudaMemsetAsync(kb, 0, sizeof(int32_t) * g->n_kf, g->stream));
+        if (g->n_lm) CK(cudaMemsetAsync(lb, 0, sizeof(int32_t) * g->n_lm, g->stream));
     }
     return g->storage ? reset_state<double>(g) : reset_state<float>(g);
 }
