@@ -125,7 +125,8 @@ struct DevState {
     R* anc = nullptr;          // 6 x n_kf: 1 on anchored keyframes, else 0
     int32_t* src_f = nullptr;  // the previous layout's factor of each factor (a keyframe was added)
     float* hist = nullptr;     // learned damping: HIST x n_f message-change history
-    // allocated by themselves
+    // allocated by themselves, not from the pool: what frees one of them does not
+    // tell the pool, whose record of its size would outlive it
     R* uv_ref = nullptr;
     R* prior_s = nullptr;      // prior scale table, prior_anneal_iters + 1 entries
     R* eta_inf = nullptr;      // record schedule: 9 x n_f reference messages (gbp_capture_messages)
@@ -619,7 +620,7 @@ gbp_status build_device(gbp_graph* g, RelayoutSrc<R>* rs = nullptr, const std::v
     if (!g->uv_ref.empty()) {
         std::vector<R> u(g->uv_ref.size());
         for (size_t i = 0; i < u.size(); ++i) u[i] = R(g->uv_ref[i]);
-        CK(g->pool.alloc(&s.uv_ref, u.size(), g->headroom));
+        CK(dev_alloc(&s.uv_ref, u.size()));
         CK(cudaMemcpyAsync(s.uv_ref, u.data(), sizeof(R) * u.size(), cudaMemcpyHostToDevice, st));
         d.uv_ref = s.uv_ref;
         CK(cudaStreamSynchronize(st));

@@ -83,3 +83,28 @@ def test_residuals_follow_the_observation_order_after_a_keyframe_is_added():
             e, want = g.residuals(), np.linalg.norm(z - h, axis=1)
             far = q[:, 2] > 0.5                     # FP32 projections: ~1e-6 relative of up to 1000 px and depth
             assert np.abs(e - want)[far].max() <= 0.05 + 1e-4 * want[far].max()
+
+
+def test_reference_solution_through_precision_switches_and_added_keyframes():
+    """The reference projections are replaced after the layout was rebuilt for another precision, and the freed
+    buffers' addresses serve later layouts: the distance to the reference is that of a graph made afresh."""
+    p = synth.make_walk(4, n_kf=20, n_lm=250)
+    init, steps = synth.stream_plan(p, 16)
+    with gbp.Graph(init, huber_nsigma=2.0) as g:
+        for precision in (2, 0):
+            g.set_reference(init.kf_Rt_true, init.lm_true)
+            g.set_params(precision_mode=precision)
+            g.set_reference(init.kf_Rt_true, init.lm_true)
+            g.set_params(prior_anneal_iters=12)
+            g.iterate(10)
+            with gbp.Graph(init, huber_nsigma=2.0, precision_mode=precision, prior_anneal_iters=12) as f:
+                f.set_reference(init.kf_Rt_true, init.lm_true)
+                f.iterate(10)
+                assert g.stats()["are_ref"] == f.stats()["are_ref"] > 0
+                if precision == 0:
+                    for st in steps:
+                        for h in (f, g):
+                            h.add_keyframe(st.obs_lm, st.obs_uv, n_new_lm=st.n_new_lm)
+                            h.iterate(4)
+                    for a, b in zip(f.means(), g.means()):
+                        assert np.array_equal(a, b)
