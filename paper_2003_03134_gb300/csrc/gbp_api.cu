@@ -1972,7 +1972,9 @@ gbp_status gbp_autotune(gbp_graph* g, int32_t n_trial, int32_t* chosen, double* 
     }
     if (best < 0) return fail(g, GBP_ECUDA, "autotune: no launch configuration ran");
     g->tuned_mode = cand[best].first;
-    // each mode keeps its own best shape (launch_mode may force the other)
+    // each mode keeps its own best shape (launch_mode may force the other); what
+    // was chosen before, by size or by an earlier timing, gives way
+    g->tuned_fshape = g->tuned_pshape = -1;
     for (size_t c = 0; c < cand.size(); ++c) {
         if (ms[c] < 0 || ms[c] != best_mode[cand[c].first - 1]) continue;
         if (cand[c].first == 1 && g->tuned_pshape < 0) g->tuned_pshape = cand[c].second;
