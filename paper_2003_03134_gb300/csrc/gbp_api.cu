@@ -165,6 +165,22 @@ void so3_exp_host(const double w[3], double E[9]) {
 
 }  // namespace
 
+// What the automatic launch mode may choose from depends on whether the
+// resident kernel (gbp_resident.cu) takes the graph, which added keyframes
+// change in both directions: a point without observations or one seen by more
+// than 32 keyframes excludes it, the next keyframe may bring it back.  Each
+// class keeps its own choice, made once a graph.
+enum LaunchClass : int {
+    LC_GENERAL = 0,         // not for the resident kernel
+    LC_RESIDENT = 1,        // resident kernel, one keyframe a block (up to two once the graph has grown)
+    LC_RESIDENT_MANY = 2,   // resident kernel, more keyframes a block: may be slower than per-phase launches
+    N_LAUNCH_CLASSES = 3
+};
+struct LaunchChoice {
+    int mode = 0;                  // 1 or 2, 0 = not chosen yet
+    int fshape = -1, pshape = -1;  // launch shapes, -1 = by size
+};
+
 struct gbp_graph {
     std::string err;
     BufPool pool;                       // buffers of replaced layouts, for the next one
@@ -199,9 +215,8 @@ struct gbp_graph {
     int wexec_every = 0;                        // its check_every
     bool wexec_failed = false;                  // not available for this layout: the host checks
     bool built = false;
-    int tuned_mode = 0;                         // autotuner's choice (1 or 2), 0 = not tuned
-    int tuned_fshape = -1, tuned_pshape = -1;   // its launch shapes, -1 = not tuned
-    bool tuned_resident = false;                // the choice was mode 1 with the resident kernel
+    LaunchChoice choice[N_LAUNCH_CLASSES];      // the automatic mode's choice of each class the graph has been in
+    int lclass = LC_GENERAL;                    // the class it is in (update_launch_class)
     // one graph split across ranks (gbp_set_partition): the keyframes and
     // landmarks whose beliefs this graph forms; lm1 < 0 = not split
     int part_kf0 = 0, part_kf1 = -1, part_lm0 = 0, part_lm1 = -1;
@@ -284,10 +299,12 @@ KParams<R> make_kparams(gbp_graph* g) {
 // else by size (large graphs -- a warp per belief item -- take the deferring
 // kernel at >= 4 blocks per SM, which measured fastest there).
 bool tunable(const gbp_graph* g) { return g->storage == 0 && g->prm.damping_mode == 0; }
+LaunchChoice& tuned(gbp_graph* g) { return g->choice[g->lclass]; }
+const LaunchChoice& tuned(const gbp_graph* g) { return g->choice[g->lclass]; }
 int factor_shape(const gbp_graph* g) {
     if (!tunable(g)) return 0;
     if (g->prm.factor_shape >= 0) return g->prm.factor_shape;
-    if (g->tuned_fshape >= 0) return g->tuned_fshape;
+    if (tuned(g).fshape >= 0) return tuned(g).fshape;
     return g->sf.g.b_warps == 1 ? 4 : 0;
 }
 // The persistent kernel runs in one shape, with no register budget: under
@@ -307,6 +324,25 @@ void destroy_exec(gbp_graph* g) {
         g->wexec = nullptr;
     }
     g->wexec_failed = false;
+}
+
+// The graph's launch class as its layout stands.  A graph that grew while it
+// ran on the resident kernel stays on it up to two keyframes a block: in calls
+// of 20 iterations, as a stream makes them, 160-250 keyframes take 12.5-12.8 us
+// an iteration against 14.5-14.8 per phase (whose launches count more there);
+// one launch of many iterations takes 8.2 against 10.1 at 160, 10.6 / 10.1 at
+// 200, 11.3 / 10.6 at 300, and beyond two a block the resident kernel loses
+// both ways (400: 13.0 / 10.6, 500: 15.2 / 10.6).
+void update_launch_class(gbp_graph* g) {
+    int c = LC_GENERAL;
+    const int blocks = tunable(g) ? resident_grid(g->sf.g) : 0;
+    if (blocks > 0) {
+        const int most = g->lclass == LC_RESIDENT ? 2 * blocks : blocks;
+        c = g->n_kf <= most ? LC_RESIDENT : LC_RESIDENT_MANY;
+    }
+    if (c == g->lclass) return;
+    g->lclass = c;
+    destroy_exec(g);   // a graph recorded with the other class's shape
 }
 
 template <>
@@ -1546,8 +1582,7 @@ gbp_status gbp_set_params(gbp_graph* g, const gbp_params* p) {
     if (check_params(p, why) != GBP_OK) return fail(g, GBP_EINVAL, why);
     bool sigma_changed = p->sigma_px != g->prm.sigma_px;
     if (p->precision_mode != g->prm.precision_mode || p->damping_mode != g->prm.damping_mode) {
-        g->tuned_mode = 0;
-        g->tuned_fshape = g->tuned_pshape = -1;
+        for (LaunchChoice& c : g->choice) c = LaunchChoice();
     }
     g->prm = *p;
     destroy_exec(g);
@@ -1584,14 +1619,14 @@ gbp_status gbp_reset(gbp_graph* g) {
 
 // The auto launch mode's choices, per device and graph shape.  Every
 // candidate gives bitwise identical results, so a graph whose device,
-// storage, precision mode, damping schedule and sizes (keyframes, points, factors, warp
-// tiles, problems) match a graph already tuned in this process takes that
+// storage, precision mode, damping schedule, sizes (keyframes, points, factors, warp
+// tiles, problems) and launch class match a graph already tuned in this process takes that
 // choice instead of timing the candidates again (gbp_autotune, called
 // explicitly, always times them and records its choice here).
 namespace {
-using TuneKey = std::tuple<int, int, int, int, int, int, int, int, int>;
+using TuneKey = std::tuple<int, int, int, int, int, int, int, int, int, int>;
 struct TuneVal {
-    int mode, fshape, pshape;
+    LaunchChoice choice;
     gbp_tuning tuning;
 };
 std::mutex g_tune_mu;
@@ -1603,7 +1638,7 @@ bool tune_key(const gbp_graph* g, TuneKey& key) {
     if (cudaGetDevice(&dev) != cudaSuccess) return false;
     const int n_tiles = g->storage ? g->sd.g.n_tiles : g->sf.g.n_tiles;
     key = TuneKey(dev, g->storage, g->prm.precision_mode, g->prm.damping_mode, g->n_kf, g->n_lm, g->n_f, n_tiles,
-                  (int)g->prob_f0.size());
+                  (int)g->prob_f0.size(), g->lclass);
     return true;
 }
 
@@ -1613,9 +1648,7 @@ bool tune_cache_lookup(gbp_graph* g) {
     std::lock_guard<std::mutex> lock(g_tune_mu);
     auto it = g_tune_cache.find(key);
     if (it == g_tune_cache.end()) return false;
-    g->tuned_mode = it->second.mode;
-    g->tuned_fshape = it->second.fshape;
-    g->tuned_pshape = it->second.pshape;
+    tuned(g) = it->second.choice;
     g->tuning = it->second.tuning;
     destroy_exec(g);   // a graph recorded before with the default shapes
     return true;
@@ -1626,7 +1659,7 @@ void tune_cache_store(const gbp_graph* g) {
     if (!tune_key(g, key)) return;
     std::lock_guard<std::mutex> lock(g_tune_mu);
     if (g_tune_cache.size() >= TUNE_CACHE_MAX && !g_tune_cache.count(key)) g_tune_cache.clear();   // bounded
-    g_tune_cache[key] = TuneVal{g->tuned_mode, g->tuned_fshape, g->tuned_pshape, g->tuning};
+    g_tune_cache[key] = TuneVal{tuned(g), g->tuning};
 }
 }  // namespace
 
@@ -1646,14 +1679,12 @@ constexpr int RULE_LARGE_TILES = 4 * 2432;
 
 static bool choose_by_rule(gbp_graph* g) {
     if (!tunable(g)) return false;
-    const DevGraph<float>& d = g->sf.g;
-    const int blocks = resident_grid(d);
     int mode = 0, shape = 0;
-    if (blocks > 0 && d.n_kf <= blocks) mode = 1;
-    else if (d.n_tiles >= RULE_LARGE_TILES) { mode = 2; shape = 4; }
+    if (g->lclass == LC_RESIDENT) mode = 1;
+    else if (g->sf.g.n_tiles >= RULE_LARGE_TILES) { mode = 2; shape = 4; }
     if (!mode) return false;
-    g->tuned_mode = mode;
-    if (mode == 2) g->tuned_fshape = shape;
+    tuned(g).mode = mode;
+    if (mode == 2) tuned(g).fshape = shape;
     g->tuning.n_candidates = 1;
     g->tuning.cand_mode[0] = mode;
     g->tuning.cand_shape[0] = shape;
@@ -1674,21 +1705,12 @@ gbp_status gbp_iterate(gbp_graph* g, int32_t n_iters, int32_t* iters_done) {
         return fail(g, GBP_ESTATE, "damping_mode 1 needs a network (gbp_set_damping_model)");
     int mode = g->prm.launch_mode;
     if (mode == 0) {
-        if (!g->tuned_mode && !tune_cache_lookup(g) && !choose_by_rule(g)) {
+        update_launch_class(g);
+        if (!tuned(g).mode && !tune_cache_lookup(g) && !choose_by_rule(g)) {
             st = gbp_autotune(g, 8, nullptr, nullptr);
             if (st != GBP_OK) return st;
         }
-        const bool resident = g->tuned_mode == 1 && tunable(g) && resident_grid(g->sf.g) > 0;
-        if (g->tuned_resident && !resident && g->tuned_mode == 1) {
-            // the graph has outgrown the resident kernel (keyframes were
-            // added): per-phase launches in the shape of its size, not the
-            // tile-walking persistent kernel
-            g->tuned_mode = 2;
-            g->tuned_fshape = -1;
-            destroy_exec(g);
-        }
-        g->tuned_resident = resident;
-        mode = g->tuned_mode;
+        mode = tuned(g).mode;
     }
     int done = 0;
     g->last_mode = mode;
@@ -1824,7 +1846,8 @@ gbp_status gbp_profile_iterations(gbp_graph* g, int32_t n_iters, double* ms_out)
     if (st != GBP_OK) return st;
     if (g->prm.damping_mode == 1 && !g->has_model)
         return fail(g, GBP_ESTATE, "damping_mode 1 needs a network (gbp_set_damping_model)");
-    int mode = g->prm.launch_mode ? g->prm.launch_mode : (g->tuned_mode ? g->tuned_mode : 2);
+    update_launch_class(g);
+    int mode = g->prm.launch_mode ? g->prm.launch_mode : (tuned(g).mode ? tuned(g).mode : 2);
     cudaEvent_t ev[2] = {nullptr, nullptr};
     cudaError_t e = cudaSuccess;
     for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaEventCreate(&ev[i]);
@@ -1904,6 +1927,7 @@ gbp_status gbp_autotune(gbp_graph* g, int32_t n_trial, int32_t* chosen, double* 
     if (st != GBP_OK) return st;
     if (g->prm.damping_mode == 1 && !g->has_model)
         return fail(g, GBP_ESTATE, "damping_mode 1 needs a network (gbp_set_damping_model)");
+    update_launch_class(g);
     // candidates: (mode, shape); only the FP32 fixed schedule has several shapes
     std::vector<std::pair<int, int>> cand;
     const int np = tunable(g) ? n_persistent_shapes(g) : 1, nf = tunable(g) ? N_FACTOR_SHAPES : 1;
@@ -1971,16 +1995,17 @@ gbp_status gbp_autotune(gbp_graph* g, int32_t n_trial, int32_t* chosen, double* 
         if (bm < 0 || ms[c] < bm) bm = ms[c];
     }
     if (best < 0) return fail(g, GBP_ECUDA, "autotune: no launch configuration ran");
-    g->tuned_mode = cand[best].first;
+    LaunchChoice choice;
+    choice.mode = cand[best].first;
     // each mode keeps its own best shape (launch_mode may force the other); what
     // was chosen before, by size or by an earlier timing, gives way
-    g->tuned_fshape = g->tuned_pshape = -1;
     for (size_t c = 0; c < cand.size(); ++c) {
         if (ms[c] < 0 || ms[c] != best_mode[cand[c].first - 1]) continue;
-        if (cand[c].first == 1 && g->tuned_pshape < 0) g->tuned_pshape = cand[c].second;
-        if (cand[c].first == 2 && g->tuned_fshape < 0) g->tuned_fshape = cand[c].second;
+        if (cand[c].first == 1 && choice.pshape < 0) choice.pshape = cand[c].second;
+        if (cand[c].first == 2 && choice.fshape < 0) choice.fshape = cand[c].second;
     }
-    if (!tunable(g)) g->tuned_fshape = g->tuned_pshape = 0;
+    if (!tunable(g)) choice.fshape = choice.pshape = 0;
+    tuned(g) = choice;
     gbp_tuning& T = g->tuning;
     T.n_candidates = (int32_t)std::min<size_t>(cand.size(), GBP_MAX_TUNING_CANDIDATES);
     for (int c = 0; c < T.n_candidates; ++c) {
@@ -1989,7 +2014,7 @@ gbp_status gbp_autotune(gbp_graph* g, int32_t n_trial, int32_t* chosen, double* 
         T.cand_ms[c] = ms[c];
     }
     tune_cache_store(g);
-    if (chosen) *chosen = g->tuned_mode;
+    if (chosen) *chosen = choice.mode;
     if (ms_out) {
         ms_out[0] = best_mode[0];
         ms_out[1] = best_mode[1];
@@ -2003,7 +2028,7 @@ gbp_status gbp_get_tuning(const gbp_graph* g, gbp_tuning* out) {
     static const int f_minb[N_FACTOR_SHAPES] = {1, 3, 4, 1, 4, 3};
     static const int p_minb[N_PERSISTENT_SHAPES] = {1};
     *out = g->tuning;
-    out->launch_mode = g->prm.launch_mode ? g->prm.launch_mode : g->tuned_mode;
+    out->launch_mode = g->prm.launch_mode ? g->prm.launch_mode : tuned(g).mode;
     out->factor_shape = factor_shape(g);
     out->persistent_shape = persistent_shape(g);
     out->factor_threads = f_threads[out->factor_shape];

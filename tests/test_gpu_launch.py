@@ -1,5 +1,7 @@
 """The automatic launch mode's choices: what gbp_autotune measured is what runs, a choice holds for the graphs it was
 made for, and every way leads to the bits of per-phase launches."""
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -32,3 +34,84 @@ def test_autotune_puts_the_shape_it_measured_in_use():
             ms = {c["shape"]: c["ms"] for c in t["candidates"] if c["launch_mode"] == 2 and c["ms"] > 0}
             assert chosen == t["launch_mode"] == 2
             assert ms[t["factor_shape"]] == min(ms.values()), t
+
+
+def _growing(seed, n_kf, n_lm, start):
+    """A walk's first `start` keyframes with the points that two of them see, and the later keyframes' observations of
+    those points: (problem, [(obs_lm, obs_uv), ...])."""
+    p = synth.make_walk(seed, n_kf=n_kf, n_lm=n_lm)
+    early = p.obs_kf < start
+    keep = np.bincount(p.obs_lm[early], minlength=p.n_lm) >= 2
+    index = np.cumsum(keep) - 1
+    on = keep[p.obs_lm]
+    sel = early & on
+    init = dataclasses.replace(p, kf_Rt_true=p.kf_Rt_true[:start], kf_Rt_init=p.kf_Rt_init[:start],
+                               lm_true=p.lm_true[keep], lm_init=p.lm_init[keep], obs_kf=p.obs_kf[sel],
+                               obs_lm=index[p.obs_lm[sel]].astype(np.int32), obs_uv=p.obs_uv[sel],
+                               obs_outlier=p.obs_outlier[sel])
+    return init, [(index[p.obs_lm[on & (p.obs_kf == k)]].astype(np.int32), p.obs_uv[on & (p.obs_kf == k)])
+                  for k in range(start, n_kf)]
+
+
+def test_a_stream_returns_to_the_resident_kernel():
+    """A point that nobody sees for one keyframe takes the graph off the resident kernel, its first observation brings
+    it back.  Both configurations are chosen once (the second time off it repeats the first one's record); the bits
+    are those of per-phase launches."""
+    init, steps = _growing(9, 18, 400, 10)
+    out = []
+    for mode in (0, 2):
+        used, records = [], []
+        with gbp.Graph(init, huber_nsigma=2.0, launch_mode=mode) as g:
+            g.iterate(6)
+            used.append(g.stats()["launch_mode"])
+            for i, (obs_lm, obs_uv) in enumerate(steps[:6]):
+                n_lm = gbp.gbp_get_sizes(g.h)[1]
+                unseen = i in (1, 4)
+                if i in (2, 5):
+                    obs_lm = np.append(obs_lm, n_lm - 1).astype(np.int32)
+                    obs_uv = np.concatenate([obs_uv, [[320.0, 240.0]]])
+                g.add_keyframe(obs_lm, obs_uv, n_new_lm=int(unseen),
+                               new_lm_xyz=init.lm_true[:1] + 0.3 if unseen else None)
+                g.iterate(6)
+                used.append(g.stats()["launch_mode"])
+                if unseen:
+                    records.append(g.tuning())
+            out.append((used, records, *g.means(), g.relin_iters()))
+    used, records = out[0][:2]
+    assert used == [1, 1, records[0]["launch_mode"], 1, 1, records[0]["launch_mode"], 1]
+    assert records[0]["n_candidates"] == 7 and records[0] == records[1]
+    for a, b in zip(out[0][2:], out[1][2:]):
+        assert np.array_equal(a, b)
+
+
+def test_a_choice_is_not_handed_to_a_graph_the_resident_kernel_does_not_take():
+    """Two graphs of the same numbers of keyframes, points, factors and tiles, one with a point that nobody sees: what
+    the timing of the first chose (the resident kernel among its candidates) is not what the second starts with."""
+    p = synth.make_circle(4, n_kf=12, n_lm=64, obs_range=(4, 4))
+    other = p.obs_lm.copy()
+    other[p.obs_lm == 63] = 62   # point 62 now has 8 observations, point 63 none
+    q = dataclasses.replace(p, obs_lm=other)
+    with gbp.Graph(p, huber_nsigma=2.0) as a, gbp.Graph(q, huber_nsigma=2.0) as b, \
+            gbp.Graph(q, huber_nsigma=2.0, launch_mode=2) as c:
+        a.autotune(4)
+        for g in (a, b, c):
+            g.iterate(9)
+        assert a.tuning()["n_candidates"] == b.tuning()["n_candidates"] == 7
+        assert a.tuning()["candidates"] != b.tuning()["candidates"]
+        for x, y in zip(b.means(), c.means()):
+            assert np.array_equal(x, y)
+
+
+def test_a_timed_choice_is_reused_for_a_graph_of_the_same_shape():
+    """Graphs whose candidates are timed (FP64 mode, and the FP32 path between the sizes that a rule covers): a second
+    graph of the same sizes takes the first one's choice and its record, times included."""
+    for p, params in ((synth.make_walk(7, n_kf=30, n_lm=300), {"precision_mode": 2}),
+                      (synth.make_loop(2, n_kf=200, n_lm=6000), {})):
+        with gbp.Graph(p, **params) as a, gbp.Graph(p, **params) as b:
+            a.iterate(12)
+            ta = a.tuning()
+            assert ta["n_candidates"] > 1 and all(c["ms"] > 0 for c in ta["candidates"])
+            b.iterate(12)
+            assert b.tuning() == ta
+            for x, y in zip(a.means(), b.means()):
+                assert np.array_equal(x, y)
