@@ -217,6 +217,7 @@ struct gbp_graph {
     bool built = false;
     LaunchChoice choice[N_LAUNCH_CLASSES];      // the automatic mode's choice of each class the graph has been in
     int lclass = LC_GENERAL;                    // the class it is in (update_launch_class)
+    bool resident_refused = false;              // a launch of the resident kernel was refused: not tried again
     // one graph split across ranks (gbp_set_partition): the keyframes and
     // landmarks whose beliefs this graph forms; lm1 < 0 = not split
     int part_kf0 = 0, part_kf1 = -1, part_lm0 = 0, part_lm1 = -1;
@@ -326,6 +327,11 @@ void destroy_exec(gbp_graph* g) {
     g->wexec_failed = false;
 }
 
+// Blocks of the resident kernel for this graph, 0 where it does not apply.
+int resident_blocks(const gbp_graph* g) {
+    return tunable(g) && !g->resident_refused ? resident_grid(g->sf.g) : 0;
+}
+
 // The graph's launch class as its layout stands.  A graph that grew while it
 // ran on the resident kernel stays on it up to two keyframes a block: in calls
 // of 20 iterations, as a stream makes them, 160-250 keyframes take 12.5-12.8 us
@@ -335,7 +341,7 @@ void destroy_exec(gbp_graph* g) {
 // both ways (400: 13.0 / 10.6, 500: 15.2 / 10.6).
 void update_launch_class(gbp_graph* g) {
     int c = LC_GENERAL;
-    const int blocks = tunable(g) ? resident_grid(g->sf.g) : 0;
+    const int blocks = resident_blocks(g);
     if (blocks > 0) {
         const int most = g->lclass == LC_RESIDENT ? 2 * blocks : blocks;
         c = g->n_kf <= most ? LC_RESIDENT : LC_RESIDENT_MANY;
@@ -1118,21 +1124,38 @@ gbp_status iterate_phases(gbp_graph* g, int n, float conv_tol, int* done_out) {
 }
 
 // One cooperative launch for all n iterations; the convergence test (same
-// cadence as above) runs on the device.
-gbp_status iterate_persistent(gbp_graph* g, int n, float conv_tol, int* done_out) {
+// cadence as above) runs on the device.  The resident kernel wants its whole
+// grid on the chip at once, at most one block on each of the device's SMs.
+// Where the driver refuses that (a stream bound to part of the SMs, say),
+// nothing has run; the graph remembers it, and the tile-walking kernel is
+// launched instead, or (refused given) the caller told so that it can choose
+// another mode.
+gbp_status iterate_persistent(gbp_graph* g, int n, float conv_tol, int* done_out, bool* refused = nullptr) {
     const int dm = g->prm.damping_mode;
     const int ps = persistent_shape(g);
-    const bool resident = !g->storage && dm == 0 && resident_grid(g->sf.g) > 0;
-    const int grid = resident ? 1 : g->storage ? persistent_grid<double>(g->sd.g, dm, ps) : persistent_grid<float>(g->sf.g, dm, ps);
-    if (grid <= 0) return fail(g, GBP_ECUDA, "persistent launch: occupancy query failed");
-    cudaError_t e = resident
-        ? launch_resident(g->sf.g, make_kparams<float>(g), n, conv_tol, g->prm.check_every, g->stream)
-        : g->storage
-        ? launch_persistent<double>(g->sd.g, make_kparams<double>(g), n, conv_tol, g->prm.check_every, grid, g->stream,
-                                    dm, ps)
-        : launch_persistent<float>(g->sf.g, make_kparams<float>(g), n, conv_tol, g->prm.check_every, grid, g->stream,
-                                   dm, ps);
-    if (e != cudaSuccess) return cuda_fail(g, e, "cooperative launch");
+    bool resident = resident_blocks(g) > 0;
+    if (resident) {
+        const cudaError_t e = launch_resident(g->sf.g, make_kparams<float>(g), n, conv_tol, g->prm.check_every, g->stream);
+        if (e != cudaSuccess) {
+            (void)cudaGetLastError();
+            g->resident_refused = true;
+            resident = false;
+            if (refused) {
+                *refused = true;
+                return cuda_fail(g, e, "cooperative launch");
+            }
+        }
+    }
+    if (!resident) {
+        const int grid = g->storage ? persistent_grid<double>(g->sd.g, dm, ps) : persistent_grid<float>(g->sf.g, dm, ps);
+        if (grid <= 0) return fail(g, GBP_ECUDA, "persistent launch: occupancy query failed");
+        const cudaError_t e = g->storage
+            ? launch_persistent<double>(g->sd.g, make_kparams<double>(g), n, conv_tol, g->prm.check_every, grid,
+                                        g->stream, dm, ps)
+            : launch_persistent<float>(g->sf.g, make_kparams<float>(g), n, conv_tol, g->prm.check_every, grid,
+                                       g->stream, dm, ps);
+        if (e != cudaSuccess) return cuda_fail(g, e, "cooperative launch");
+    }
     g->launches += 1;
     if (conv_tol > 0.0f) {
         gbp_status st = read_ctl(g);
@@ -1703,20 +1726,28 @@ gbp_status gbp_iterate(gbp_graph* g, int32_t n_iters, int32_t* iters_done) {
     if (g->n_f == 0 && g->n_kf == 0 && g->n_lm == 0) return GBP_OK;
     if (g->prm.damping_mode == 1 && !g->has_model)
         return fail(g, GBP_ESTATE, "damping_mode 1 needs a network (gbp_set_damping_model)");
-    int mode = g->prm.launch_mode;
-    if (mode == 0) {
-        update_launch_class(g);
-        if (!tuned(g).mode && !tune_cache_lookup(g) && !choose_by_rule(g)) {
-            st = gbp_autotune(g, 8, nullptr, nullptr);
-            if (st != GBP_OK) return st;
+    for (;;) {
+        int mode = g->prm.launch_mode;
+        if (mode == 0) {
+            update_launch_class(g);
+            if (!tuned(g).mode && !tune_cache_lookup(g) && !choose_by_rule(g)) {
+                st = gbp_autotune(g, 8, nullptr, nullptr);
+                if (st != GBP_OK) return st;
+            }
+            mode = tuned(g).mode;
         }
-        mode = tuned(g).mode;
+        int done = 0;
+        bool refused = false;
+        g->last_mode = mode;
+        st = mode == 1 ? iterate_persistent(g, n, g->prm.conv_tol, &done, g->prm.launch_mode == 0 ? &refused : nullptr)
+                       : iterate_phases(g, n, g->prm.conv_tol, &done);
+        if (refused) {
+            g->err.clear();
+            continue;   // the graph is now of the class without the resident kernel
+        }
+        if (iters_done) *iters_done = done;
+        return st;
     }
-    int done = 0;
-    g->last_mode = mode;
-    st = mode == 1 ? iterate_persistent(g, n, g->prm.conv_tol, &done) : iterate_phases(g, n, g->prm.conv_tol, &done);
-    if (iters_done) *iters_done = done;
-    return st;
 }
 
 gbp_status gbp_get_means(const gbp_graph* cg, double* kf_mu, double* lm_mu) {
@@ -1995,6 +2026,7 @@ gbp_status gbp_autotune(gbp_graph* g, int32_t n_trial, int32_t* chosen, double* 
         if (bm < 0 || ms[c] < bm) bm = ms[c];
     }
     if (best < 0) return fail(g, GBP_ECUDA, "autotune: no launch configuration ran");
+    update_launch_class(g);   // a refused resident kernel is not this graph's
     LaunchChoice choice;
     choice.mode = cand[best].first;
     // each mode keeps its own best shape (launch_mode may force the other); what

@@ -1,6 +1,10 @@
 """The automatic launch mode's choices: what gbp_autotune measured is what runs, a choice holds for the graphs it was
 made for, and every way leads to the bits of per-phase launches."""
+import ctypes
 import dataclasses
+import glob
+import os
+import subprocess
 
 import numpy as np
 import pytest
@@ -115,3 +119,59 @@ def test_a_timed_choice_is_reused_for_a_graph_of_the_same_shape():
             assert b.tuning() == ta
             for x, y in zip(a.means(), b.means()):
                 assert np.array_equal(x, y)
+
+
+FAKE_LAUNCH = """
+#include <stddef.h>
+typedef struct { unsigned x, y, z; } dim3;
+int fake_refuse_above = 1 << 30;   /* threads a block; a launch with more is refused */
+int __real_cudaLaunchCooperativeKernel(const void*, dim3, dim3, void**, size_t, void*);
+int __wrap_cudaLaunchCooperativeKernel(const void* f, dim3 grid, dim3 block, void** args, size_t shared, void* stream) {
+    if ((int)block.x > fake_refuse_above) return 720;   /* cudaErrorCooperativeLaunchTooLarge */
+    return __real_cudaLaunchCooperativeKernel(f, grid, block, args, shared, stream);
+}
+"""
+
+
+@pytest.fixture
+def refusing_lib(tmp_path, monkeypatch):
+    """The library linked with a cooperative launch that the test can have refused on the host, as the driver refuses
+    one that does not fit the SMs a stream may use.  Sets the number of threads a block above which it is refused."""
+    objs = sorted(glob.glob(os.path.join(build.BUILD_DIR, "*.o")))
+    if not objs:
+        build.build(force=True)
+        objs = sorted(glob.glob(os.path.join(build.BUILD_DIR, "*.o")))
+    (tmp_path / "fake.c").write_text(FAKE_LAUNCH)
+    subprocess.check_call(["gcc", "-c", "-fPIC", "-o", str(tmp_path / "fake.o"), str(tmp_path / "fake.c")])
+    path = str(tmp_path / "libgbp_refusing.so")
+    subprocess.check_call([build.nvcc(), *build.ARCH, "-shared", "-o", path, *objs, str(tmp_path / "fake.o"),
+                           "-Xlinker", "--wrap=cudaLaunchCooperativeKernel"])
+    monkeypatch.setattr(gbp, "LIB_PATH", path)
+    monkeypatch.setattr(gbp, "_lib", None)
+    return ctypes.c_int.in_dll(gbp.lib(), "fake_refuse_above")
+
+
+def test_a_refused_cooperative_launch_is_replaced(refusing_lib):
+    """Automatic launches of a graph for which a rule takes the resident kernel (256 threads a block) untried, and
+    forced persistent launches: refused, the first run per phase and the second on the tile-walking kernel (128
+    threads); with that refused too the forced launch reports the error, as it always did.  Same bits throughout."""
+    p = synth.make_circle(5)
+
+    def solve(mode):
+        with gbp.Graph(p, huber_nsigma=2.0, launch_mode=mode, conv_tol=1e-30) as g:
+            assert [g.iterate(n) for n in (3, 20)] == [3, 20]
+            return g.stats()["launch_mode"], [*g.means(), g.relin_iters()]
+
+    mode, want = solve(0)
+    assert mode == 1   # nothing refused yet
+    for limit in (128, 0):
+        refusing_lib.value = limit
+        for launch_mode in (0, 2) + ((1,) if limit else ()):
+            mode, got = solve(launch_mode)
+            if launch_mode or not limit:
+                assert mode == (launch_mode or 2)
+            for a, b in zip(want, got):
+                assert np.array_equal(a, b)
+    with pytest.raises(gbp.GBPError) as e:
+        solve(1)
+    assert e.value.status == gbp.GBP_ECUDA
