@@ -81,15 +81,23 @@ typedef struct {
     int32_t linear;             /* 1: never relinearise (linear GBP at the initial point)          */
     int32_t launch_mode;        /* 0: auto (by size where one configuration is known to be the fastest,
                                    else gbp_autotune on first use; a graph whose device, storage,
-                                   precision and damping modes and sizes match one already tuned in
-                                   this process takes that graph's choice), 1: one persistent launch per
-                                   gbp_iterate call with a grid barrier between phases, 2: one launch
+                                   precision and damping modes, sizes and kinds of launch that apply
+                                   match one already tuned in this process takes that graph's choice;
+                                   chosen again when added keyframes change what applies), 1: one
+                                   persistent launch per gbp_iterate call: for FP32 graphs with the
+                                   fixed schedule of up to 8 warp tiles an SM whose points all have 1 to
+                                   32 observations the resident kernel (tiles keep their state in
+                                   registers; counted arrivals between the phases), else a kernel that
+                                   walks the tiles with a grid barrier between phases; 2: one launch
                                    per phase (factor kernel, belief kernel) replayed as a CUDA graph.
+                                   A resident launch holds its SMs until its iterations are done: in
+                                   auto mode a graph takes it only while its blocks and those of the
+                                   graphs that run on other streams fit the device together.
                                    All modes give bitwise identical results.                        */
     int32_t damping_mode;       /* 0: the fixed d above (Sec. 5, Sec. 8); 1: per-factor d predicted by
                                    the damping network given to gbp_set_damping_model (see below)   */
     int32_t factor_shape;       /* FP32 fixed schedule, per-phase launches: launch shape of the factor
-                                   kernel, -1 = the autotuner's choice (default; before tuning: 1 for
+                                   kernel, -1 = the autotuner's choice (default; before tuning: 4 for
                                    large graphs, else 0); 0: 128 threads per block, no register
                                    budget; 1: 128 threads, >= 3 blocks per SM; 2: 128 threads, >= 4
                                    blocks per SM; 3: 64 threads, no budget; 4 and 5: 128 threads, >= 4

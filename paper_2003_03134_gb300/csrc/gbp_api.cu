@@ -19,7 +19,9 @@
 #include <cstring>
 #include <new>
 #include <numeric>
+#include <set>
 #include <string>
+#include <utility>
 #include <vector>
 
 using namespace gbp;
@@ -174,7 +176,8 @@ enum LaunchClass : int {
     LC_GENERAL = 0,         // not for the resident kernel
     LC_RESIDENT = 1,        // resident kernel, one keyframe a block (up to two once the graph has grown)
     LC_RESIDENT_MANY = 2,   // resident kernel, more keyframes a block: may be slower than per-phase launches
-    N_LAUNCH_CLASSES = 3
+    LC_SHARED = 3,          // resident kernel, but graphs on other streams need its SMs
+    N_LAUNCH_CLASSES = 4
 };
 struct LaunchChoice {
     int mode = 0;                  // 1 or 2, 0 = not chosen yet
@@ -217,6 +220,7 @@ struct gbp_graph {
     bool built = false;
     LaunchChoice choice[N_LAUNCH_CLASSES];      // the automatic mode's choice of each class the graph has been in
     int lclass = LC_GENERAL;                    // the class it is in (update_launch_class)
+    int use_dev = -1, use_sms = 0;              // its entry in the table of streams (sms_of_other_streams)
     bool resident_refused = false;              // a launch of the resident kernel was refused: not tried again
     // one graph split across ranks (gbp_set_partition): the keyframes and
     // landmarks whose beliefs this graph forms; lm1 < 0 = not split
@@ -332,7 +336,43 @@ int resident_blocks(const gbp_graph* g) {
     return tunable(g) && !g->resident_refused ? resident_grid(g->sf.g) : 0;
 }
 
-// The graph's launch class as its layout stands.  A graph that grew while it
+// The SMs that each stream's graphs take at a time, by device: a graph that
+// the resident kernel takes counts with its blocks, any other with the whole
+// chip; graphs of one stream follow one another, so the largest of them.  A
+// graph is entered by its first iteration and taken out when it is destroyed.
+std::mutex g_use_mu;
+std::map<std::pair<int, cudaStream_t>, std::multiset<int>> g_use;
+
+void drop_stream_use(gbp_graph* g) {   // with g_use_mu held
+    if (g->use_dev < 0) return;
+    auto it = g_use.find({g->use_dev, g->stream});
+    it->second.erase(it->second.find(g->use_sms));
+    if (it->second.empty()) g_use.erase(it);
+    g->use_dev = -1;
+}
+
+int sms_of_other_streams(gbp_graph* g, int sms) {
+    int dev = 0, other = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    std::lock_guard<std::mutex> lock(g_use_mu);
+    if (g->use_dev != dev || g->use_sms != sms) {
+        drop_stream_use(g);
+        g_use[{dev, g->stream}].insert(sms);
+        g->use_dev = dev;
+        g->use_sms = sms;
+    }
+    for (const auto& u : g_use)
+        if (u.first.first == dev && u.first.second != g->stream) other += *u.second.rbegin();
+    return other;
+}
+
+// The graph's launch class as its layout stands.  Resident launches of several
+// streams run beside each other only while all their blocks fit the chip;
+// beyond that each waits for the others to end, where per-phase launches
+// overlap: graphs of 125 keyframes and 566 tiles (142 blocks), 200 iterations
+// each, all of them: 2 streams 2.94 ms resident, 2.30 per phase; 4 streams 5.88
+// / 2.92; 8 streams 11.6 / 4.96; of 68 blocks each 2 streams 1.42 / 2.13, 4
+// streams 2.77 / 2.34; of 10 blocks 8 streams 1.25 / 2.18.  A graph that grew while it
 // ran on the resident kernel stays on it up to two keyframes a block: in calls
 // of 20 iterations, as a stream makes them, 160-250 keyframes take 12.5-12.8 us
 // an iteration against 14.5-14.8 per phase (whose launches count more there);
@@ -341,14 +381,15 @@ int resident_blocks(const gbp_graph* g) {
 // both ways (400: 13.0 / 10.6, 500: 15.2 / 10.6).
 void update_launch_class(gbp_graph* g) {
     int c = LC_GENERAL;
-    const int blocks = resident_blocks(g);
+    const int blocks = resident_blocks(g), sms = sm_count();
+    const int other = sms_of_other_streams(g, blocks > 0 ? blocks : sms);
     if (blocks > 0) {
         const int most = g->lclass == LC_RESIDENT ? 2 * blocks : blocks;
-        c = g->n_kf <= most ? LC_RESIDENT : LC_RESIDENT_MANY;
+        c = blocks + other > sms ? LC_SHARED : g->n_kf <= most ? LC_RESIDENT : LC_RESIDENT_MANY;
     }
-    if (c == g->lclass) return;
+    const int shape = factor_shape(g);
     g->lclass = c;
-    destroy_exec(g);   // a graph recorded with the other class's shape
+    if (factor_shape(g) != shape) destroy_exec(g);   // recorded with the other class's shape
 }
 
 template <>
@@ -1693,6 +1734,9 @@ void tune_cache_store(const gbp_graph* g) {
 //   * the resident kernel with one keyframe a block (see gbp_resident.cu):
 //     328 tiles 6.1 us against 9.2 of the best per-phase shape, 591 6.6 / 9.5,
 //     624 8.1 / 9.8, 985 9.0 / 10.2, 1200 10.3 / 11.1; it takes up to 1216;
+//   * per-phase launches in the shape of the size while graphs on other
+//     streams need the SMs (update_launch_class has the figures; alone, shape
+//     0 is within 1.5 % of the fastest at 600-1200 tiles);
 //   * at four chips' worth of warps and more (4 x 2432 tiles) the deferring
 //     factor kernel: 10510 tiles 39.5 us against 44.6, 15766 60.4 / 72.0; at
 //     7883 35.0 / 37.0, at 5255 26.0 / 25.0, so between the two lines the
@@ -1704,6 +1748,7 @@ static bool choose_by_rule(gbp_graph* g) {
     if (!tunable(g)) return false;
     int mode = 0, shape = 0;
     if (g->lclass == LC_RESIDENT) mode = 1;
+    else if (g->lclass == LC_SHARED) { mode = 2; shape = factor_shape(g); }
     else if (g->sf.g.n_tiles >= RULE_LARGE_TILES) { mode = 2; shape = 4; }
     if (!mode) return false;
     tuned(g).mode = mode;
@@ -1728,8 +1773,8 @@ gbp_status gbp_iterate(gbp_graph* g, int32_t n_iters, int32_t* iters_done) {
         return fail(g, GBP_ESTATE, "damping_mode 1 needs a network (gbp_set_damping_model)");
     for (;;) {
         int mode = g->prm.launch_mode;
+        update_launch_class(g);
         if (mode == 0) {
-            update_launch_class(g);
             if (!tuned(g).mode && !tune_cache_lookup(g) && !choose_by_rule(g)) {
                 st = gbp_autotune(g, 8, nullptr, nullptr);
                 if (st != GBP_OK) return st;
@@ -2176,6 +2221,10 @@ gbp_status gbp_put_split_records(gbp_graph* g, int32_t kind, int32_t n, const in
 
 void gbp_destroy_graph(gbp_graph* g) {
     if (!g) return;
+    {
+        std::lock_guard<std::mutex> lock(g_use_mu);
+        drop_stream_use(g);
+    }
     destroy_exec(g);
     g->sf.release(&g->pool);
     g->sd.release(&g->pool);

@@ -243,6 +243,7 @@ template <typename R> int persistent_grid(const DevGraph<R>& g, int mode, int sh
 template <typename R> cudaError_t launch_persistent(const DevGraph<R>& g, const KParams<R>& p, int n_iters,
                                                     float conv_tol, int check_every, int grid, cudaStream_t s,
                                                     int mode, int shape);
+int sm_count();   // SMs of the current device, 0 if there is none
 // resident kernel (gbp_resident.cu): its blocks (0 = not for this graph)
 int resident_grid(const DevGraph<float>& g);
 cudaError_t launch_resident(const DevGraph<float>& g, const KParams<float>& p, int n_iters, float conv_tol,

@@ -550,13 +550,6 @@ __global__ void __launch_bounds__(NA * 32 + NB_BELIEF, 1)
     }
 }
 
-int sm_count() {
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    return sms;
-}
-
 // Factor warps per block: the fewest that hold the tiles (the more registers
 // each); 0: too many tiles.
 int factor_warps(int n_tiles, int sms) {
@@ -566,6 +559,13 @@ int factor_warps(int n_tiles, int sms) {
 }
 
 }  // namespace
+
+int sm_count() {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    return sms;
+}
 
 // Blocks of the resident kernel for this graph; 0 where it does not apply:
 // more tiles than the SMs hold at one block each, a landmark split across

@@ -5,6 +5,7 @@ import dataclasses
 import glob
 import os
 import subprocess
+import threading
 
 import numpy as np
 import pytest
@@ -175,3 +176,67 @@ def test_a_refused_cooperative_launch_is_replaced(refusing_lib):
     with pytest.raises(gbp.GBPError) as e:
         solve(1)
     assert e.value.status == gbp.GBP_ECUDA
+
+
+def test_graphs_on_several_streams_leave_the_resident_kernel_when_they_do_not_fit(torch):
+    """Resident launches run beside each other while all their blocks (one a keyframe here) fit the SMs; a graph whose
+    blocks and those of other streams' graphs do not, launches per phase until there is room again."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    big = synth.make_walk(2, n_kf=sms // 2 + 10, n_lm=400)
+    small = synth.make_circle(2)
+    s1, s2 = torch.cuda.Stream().cuda_stream, torch.cuda.Stream().cuda_stream
+
+    def graph(p, stream):
+        return gbp.Graph(p, stream=stream, huber_nsigma=2.0)
+
+    def run(g):
+        g.iterate(8)
+        return g.stats()["launch_mode"]
+
+    a = graph(big, s1)
+    assert run(a) == 1
+    same, beside, b = graph(big, s1), graph(small, s2), graph(big, s2)
+    assert run(same) == 1 and run(beside) == 1 and run(a) == 1   # one stream; room for both
+    assert [run(b), run(a), run(same), run(b)] == [2, 2, 2, 2]
+    a.close()
+    assert run(b) == 2
+    same.close()
+    assert run(b) == 1
+    for x, y in zip(b.means(), _means_after(big, 4)):
+        assert np.array_equal(x, y)
+    b.close()
+    beside.close()
+
+
+def _means_after(problem, calls):
+    with gbp.Graph(problem, huber_nsigma=2.0, launch_mode=2) as r:
+        for _ in range(calls):
+            r.iterate(8)
+        return r.means()
+
+
+def test_solves_in_threads_on_their_own_streams_give_the_same_bits(torch):
+    """Four host threads make, solve and close graphs of different sizes at the same time, each on its own stream."""
+    problems = [synth.make_walk(6, n_kf=100, n_lm=500), synth.make_circle(6), synth.make_walk(8, n_kf=60, n_lm=700)]
+    want = [_means_after(p, 3) for p in problems]
+    bad = []
+
+    def work(i):
+        try:
+            stream = torch.cuda.Stream().cuda_stream
+            for r in range(6):
+                j = (i + r) % len(problems)
+                with gbp.Graph(problems[j], stream=stream, huber_nsigma=2.0) as g:
+                    for _ in range(3):
+                        g.iterate(8)
+                    if not all(np.array_equal(x, y) for x, y in zip(g.means(), want[j])):
+                        bad.append((i, r))
+        except Exception as e:   # a thread's exception does not fail the test by itself
+            bad.append((i, repr(e)))
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad
