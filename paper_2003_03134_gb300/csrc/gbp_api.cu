@@ -192,6 +192,7 @@ struct gbp_graph {
     cudaStream_t capture = nullptr;     // private stream used only to record CUDA graphs
     gbp_intrinsics intr{};
     gbp_params prm{};
+    int sms = 0;                                // SMs of the device the graph was made on
     int n_kf = 0, n_lm = 0, n_f = 0;
     // host copy of the problem (internal factor order)
     std::vector<double> kf_R, kf_c, lm_ref;     // references (chart origins)
@@ -381,11 +382,11 @@ int sms_of_other_streams(gbp_graph* g, int sms) {
 // both ways (400: 13.0 / 10.6, 500: 15.2 / 10.6).
 void update_launch_class(gbp_graph* g) {
     int c = LC_GENERAL;
-    const int blocks = resident_blocks(g), sms = sm_count();
-    const int other = sms_of_other_streams(g, blocks > 0 ? blocks : sms);
+    const int blocks = resident_blocks(g);
+    const int other = sms_of_other_streams(g, blocks > 0 ? blocks : g->sms);
     if (blocks > 0) {
         const int most = g->lclass == LC_RESIDENT ? 2 * blocks : blocks;
-        c = blocks + other > sms ? LC_SHARED : g->n_kf <= most ? LC_RESIDENT : LC_RESIDENT_MANY;
+        c = blocks + other > g->sms ? LC_SHARED : g->n_kf <= most ? LC_RESIDENT : LC_RESIDENT_MANY;
     }
     const int shape = factor_shape(g);
     g->lclass = c;
@@ -1484,6 +1485,7 @@ gbp_status create_impl(const gbp_intrinsics* intr, int32_t n_kf, const double* k
     g->intr = *intr;
     gbp_default_params(&g->prm);
     g->stream = reinterpret_cast<cudaStream_t>(cuda_stream);
+    g->sms = sm_count();
     g->n_kf = n_kf;
     g->n_lm = n_lm;
     g->prob_kf0 = prob_kf0;
@@ -1737,19 +1739,20 @@ void tune_cache_store(const gbp_graph* g) {
 //   * per-phase launches in the shape of the size while graphs on other
 //     streams need the SMs (update_launch_class has the figures; alone, shape
 //     0 is within 1.5 % of the fastest at 600-1200 tiles);
-//   * at four chips' worth of warps and more (4 x 2432 tiles) the deferring
-//     factor kernel: 10510 tiles 39.5 us against 44.6, 15766 60.4 / 72.0; at
-//     7883 35.0 / 37.0, at 5255 26.0 / 25.0, so between the two lines the
-//     candidates are timed.
+//   * at four chips' worth of warps and more (4 x 16 an SM: 9728 tiles on 152
+//     SMs) the deferring factor kernel: 10510 tiles 39.5 us against 44.6 of the
+//     best other shape, 12189 45.4 / 49.7, 14472 51.8 / 59.7, 17309 61.3 / 72.1,
+//     22471 85.4 / 100.7, 35340 124.8 / 152.0; at 8950 36.6 / 37.5, at 5255
+//     26.0 / 25.0, so between the two lines the candidates are timed.
 // Recorded as one candidate with time 0.
-constexpr int RULE_LARGE_TILES = 4 * 2432;
+constexpr int RULE_LARGE_TILES_PER_SM = 4 * 16;
 
 static bool choose_by_rule(gbp_graph* g) {
     if (!tunable(g)) return false;
     int mode = 0, shape = 0;
     if (g->lclass == LC_RESIDENT) mode = 1;
     else if (g->lclass == LC_SHARED) { mode = 2; shape = factor_shape(g); }
-    else if (g->sf.g.n_tiles >= RULE_LARGE_TILES) { mode = 2; shape = 4; }
+    else if (g->sms > 0 && g->sf.g.n_tiles >= RULE_LARGE_TILES_PER_SM * g->sms) { mode = 2; shape = 4; }
     if (!mode) return false;
     tuned(g).mode = mode;
     if (mode == 2) tuned(g).fshape = shape;
