@@ -97,12 +97,12 @@ typedef struct {
     int32_t damping_mode;       /* 0: the fixed d above (Sec. 5, Sec. 8); 1: per-factor d predicted by
                                    the damping network given to gbp_set_damping_model (see below)   */
     int32_t factor_shape;       /* FP32 fixed schedule, per-phase launches: launch shape of the factor
-                                   kernel, -1 = the autotuner's choice (default; before tuning: 4 for
-                                   large graphs, else 0); 0: 128 threads per block, no register
-                                   budget; 1: 128 threads, >= 3 blocks per SM; 2: 128 threads, >= 4
-                                   blocks per SM; 3: 64 threads, no budget; 4 and 5: 128 threads, >= 4
-                                   or >= 3 blocks per SM, the rare tiles that need the FP64 redo left
-                                   to a second kernel (so the first holds no registers for it).
+                                   kernel, -1 = the autotuner's choice (default; before tuning by
+                                   size: 4 for large graphs, else 0 or 1); 0: 128 threads per block, no
+                                   register budget; 1: 128 threads, >= 3 blocks per SM; 2: 128 threads,
+                                   >= 4 blocks per SM; 3: 64 threads, no budget; 4 and 5: 128 threads,
+                                   >= 4 or >= 3 blocks per SM, the rare tiles that need the FP64 redo
+                                   left to a second kernel (so the first holds no registers for it).
                                    Every shape gives bitwise identical results.                     */
     int32_t persistent_shape;   /* persistent launches: -1 (default) or 0, the one shape (no
                                    register budget); kept for the autotuner's report.               */

@@ -302,8 +302,13 @@ KParams<R> make_kparams(gbp_graph* g) {
 }
 
 // Launch shapes in use: the parameter if set, else the autotuner's choice,
-// else by size (large graphs -- a warp per belief item -- take the deferring
-// kernel at >= 4 blocks per SM, which measured fastest there).
+// else by size.  Large graphs (a warp per belief item) take the deferring
+// kernel at >= 4 blocks per SM, which measured fastest there.  Smaller ones
+// hold 8 tiles an SM at a time in shape 0 (2 blocks of 4 warps) and 12 in shape
+// 1, whose iterations are slower: shape 1 where it needs fewer waves.  On 152
+// SMs, 150 keyframes: 1162 tiles 10.5 us an iteration (shape 0) against 11.5
+// (shape 1); 1217 13.4 / 11.7; 1521 14.5 / 12.5; 1728 15.1 / 12.7; 1830 15.2 /
+// 15.5; 1936 15.3 / 16.4; 2342 16.4 / 18.1; 2646 19.6 / 18.8.
 bool tunable(const gbp_graph* g) { return g->storage == 0 && g->prm.damping_mode == 0; }
 LaunchChoice& tuned(gbp_graph* g) { return g->choice[g->lclass]; }
 const LaunchChoice& tuned(const gbp_graph* g) { return g->choice[g->lclass]; }
@@ -311,7 +316,10 @@ int factor_shape(const gbp_graph* g) {
     if (!tunable(g)) return 0;
     if (g->prm.factor_shape >= 0) return g->prm.factor_shape;
     if (tuned(g).fshape >= 0) return tuned(g).fshape;
-    return g->sf.g.b_warps == 1 ? 4 : 0;
+    if (g->sf.g.b_warps == 1) return 4;
+    if (g->sms <= 0) return 0;
+    const auto waves = [&](int tiles_per_sm) { return (g->sf.g.n_tiles - 1) / (tiles_per_sm * g->sms); };
+    return waves(12) < waves(8) ? 1 : 0;
 }
 // The persistent kernel runs in one shape, with no register budget: under
 // a budget (>= 3 or >= 4 blocks per SM) it compiled to different rounding
@@ -1736,9 +1744,13 @@ void tune_cache_store(const gbp_graph* g) {
 //   * the resident kernel with one keyframe a block (see gbp_resident.cu):
 //     328 tiles 6.1 us against 9.2 of the best per-phase shape, 591 6.6 / 9.5,
 //     624 8.1 / 9.8, 985 9.0 / 10.2, 1200 10.3 / 11.1; it takes up to 1216;
-//   * per-phase launches in the shape of the size while graphs on other
-//     streams need the SMs (update_launch_class has the figures; alone, shape
-//     0 is within 1.5 % of the fastest at 600-1200 tiles);
+//   * per-phase launches in the shape of the size (factor_shape; alone, shape 0
+//     is within 1.5 % of the fastest at 600-1200 tiles) while graphs on other
+//     streams need the SMs (update_launch_class has the figures), and for a
+//     graph that grew out of the resident kernel: timing it would stop a
+//     stream for 4 ms, 200 of its iterations, and the next 100 keyframes
+//     would change the answer (the persistent launch is not near: 18.7 us at
+//     1217 tiles);
 //   * at four chips' worth of warps and more (4 x 16 an SM: 9728 tiles on 152
 //     SMs) the deferring factor kernel: 10510 tiles 39.5 us against 44.6 of the
 //     best other shape, 12189 45.4 / 49.7, 14472 51.8 / 59.7, 17309 61.3 / 72.1,
@@ -1750,15 +1762,16 @@ constexpr int RULE_LARGE_TILES_PER_SM = 4 * 16;
 static bool choose_by_rule(gbp_graph* g) {
     if (!tunable(g)) return false;
     int mode = 0, shape = 0;
+    const bool grown = g->lclass == LC_GENERAL && g->choice[LC_RESIDENT].mode != 0;
     if (g->lclass == LC_RESIDENT) mode = 1;
-    else if (g->lclass == LC_SHARED) { mode = 2; shape = factor_shape(g); }
+    else if (g->lclass == LC_SHARED || grown) mode = 2;   // fshape stays -1: by size, also as the graph grows
     else if (g->sms > 0 && g->sf.g.n_tiles >= RULE_LARGE_TILES_PER_SM * g->sms) { mode = 2; shape = 4; }
     if (!mode) return false;
     tuned(g).mode = mode;
-    if (mode == 2) tuned(g).fshape = shape;
+    if (shape) tuned(g).fshape = shape;
     g->tuning.n_candidates = 1;
     g->tuning.cand_mode[0] = mode;
-    g->tuning.cand_shape[0] = shape;
+    g->tuning.cand_shape[0] = mode == 2 ? factor_shape(g) : 0;
     g->tuning.cand_ms[0] = 0.0;
     destroy_exec(g);   // a graph recorded before with the default shapes
     return true;

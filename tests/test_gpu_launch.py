@@ -59,9 +59,9 @@ def _growing(seed, n_kf, n_lm, start):
 
 
 def test_a_stream_returns_to_the_resident_kernel():
-    """A point that nobody sees for one keyframe takes the graph off the resident kernel, its first observation brings
-    it back.  Both configurations are chosen once (the second time off it repeats the first one's record); the bits
-    are those of per-phase launches."""
+    """A point that nobody sees for one keyframe takes the graph off the resident kernel, to per-phase launches in the
+    shape of its size without a timing; its first observation brings it back.  The bits are those of per-phase
+    launches."""
     init, steps = _growing(9, 18, 400, 10)
     out = []
     for mode in (0, 2):
@@ -83,8 +83,9 @@ def test_a_stream_returns_to_the_resident_kernel():
                     records.append(g.tuning())
             out.append((used, records, *g.means(), g.relin_iters()))
     used, records = out[0][:2]
-    assert used == [1, 1, records[0]["launch_mode"], 1, 1, records[0]["launch_mode"], 1]
-    assert records[0]["n_candidates"] == 7 and records[0] == records[1]
+    assert used == [1, 1, 2, 1, 1, 2, 1]
+    for r in records:
+        assert (r["n_candidates"], r["factor_shape"], r["candidates"][0]["ms"]) == (1, 0, 0.0)
     for a, b in zip(out[0][2:], out[1][2:]):
         assert np.array_equal(a, b)
 
@@ -120,6 +121,33 @@ def test_a_timed_choice_is_reused_for_a_graph_of_the_same_shape():
             assert b.tuning() == ta
             for x, y in zip(a.means(), b.means()):
                 assert np.array_equal(x, y)
+
+
+def _repeat_points(p, n):
+    """The problem with its points, and their observations, n times over."""
+    return dataclasses.replace(p, lm_true=np.tile(p.lm_true, (n, 1)), lm_init=np.tile(p.lm_init, (n, 1)),
+                               obs_kf=np.tile(p.obs_kf, n), obs_uv=np.tile(p.obs_uv, (n, 1)),
+                               obs_lm=(np.tile(p.obs_lm, n) + np.repeat(np.arange(n), p.n_obs) * p.n_lm).astype(np.int32),
+                               obs_outlier=np.tile(p.obs_outlier, n))
+
+
+@pytest.mark.parametrize("per_sm,shape", [(8, 0), (12, 1), (16, 0)])
+def test_the_factor_shape_by_size_at_the_edges_of_its_waves(torch, per_sm, shape):
+    """Per-phase launches that were never timed: shape 0 holds 8 tiles an SM at a time, shape 1 12; the one that needs
+    fewer waves is taken, on both sides of each edge."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    ring = synth.make_circle(3, n_kf=10, n_lm=8, obs_range=(4, 4))
+    assert ring.n_obs == 32   # a full tile
+    for tiles, want in ((per_sm * sms, shape), (per_sm * sms + 1, 1 - shape)):
+        p = _repeat_points(ring, tiles)
+        with gbp.Graph(p, huber_nsigma=2.0, launch_mode=2) as g:
+            assert g.tuning()["factor_shape"] == want
+            g.iterate(5)
+            got = g.means()
+        with gbp.Graph(p, huber_nsigma=2.0, launch_mode=2, factor_shape=5) as g:
+            g.iterate(5)
+            for a, b in zip(got, g.means()):
+                assert np.array_equal(a, b)
 
 
 FAKE_LAUNCH = """
