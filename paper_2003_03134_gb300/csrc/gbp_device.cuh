@@ -879,10 +879,10 @@ __device__ __forceinline__ float warp_max(float v) {
 
 // Landmark belief b^{t+1} = s(t+1) D + sum of messages (eqs. beliefeta /
 // belieflambda) and its mean (to mu_out too, if given); writes the record,
-// returns |dmu|_inf.
+// returns |dmu|_inf.  An error raised is noted in *bad too, if given.
 template <typename R>
 __device__ __forceinline__ float finish_landmark(const DevGraph<R>& g, const KParams<R>& P, int m, R s, const R* sum,
-                                                 const R* mu_old, R* out_bel, R* mu_out = nullptr) {
+                                                 const R* mu_old, R* out_bel, R* mu_out = nullptr, int* bad = nullptr) {
     R lam[6], eta[3], mu[3], work[6], ratio;
     const R isig2 = P.inv_sigma2;
 #pragma unroll
@@ -913,7 +913,10 @@ __device__ __forceinline__ float finish_landmark(const DevGraph<R>& g, const KPa
         if (!isfinite(mu[i])) ok = false;
         dmu = fmaxf(dmu, float(fabs(mu[i] - mu_old[i])));
     }
-    if (!ok) raise_error(g.ctl, g.n_kf + m);
+    if (!ok) {
+        raise_error(g.ctl, g.n_kf + m);
+        if (bad) *bad = 1;
+    }
     if (mu_out)
 #pragma unroll
         for (int i = 0; i < 3; ++i) mu_out[i] = mu[i];
@@ -963,10 +966,11 @@ __device__ __noinline__ bool kf_record_fp64(R* out) {
 // Keyframe belief b^{t+1} = s(t+1) D + anchor + sum of messages and its
 // mean from the (already reduced) sums; writes the record to out and
 // returns |dmu|_inf against mu_old.
-// prior[i] = (s(t+1) D_i + anchor_scale A_i) / sigma^2, formed by the caller.
+// prior[i] = (s(t+1) D_i + anchor_scale A_i) / sigma^2, formed by the caller;
+// an error raised is noted in *bad too, if given.
 template <typename R>
 __device__ __forceinline__ float finish_keyframe(const DevGraph<R>& g, const KParams<R>& P, int k, const R* prior,
-                                                 const R* sum, const R* mu_old, R* out_bel) {
+                                                 const R* sum, const R* mu_old, R* out_bel, int* bad = nullptr) {
     R lam[21], eta[6], ratio;
 #pragma unroll
     for (int j = 0; j < 21; ++j) lam[j] = sum[j];
@@ -994,7 +998,10 @@ __device__ __forceinline__ float finish_keyframe(const DevGraph<R>& g, const KPa
         if (!isfinite(mu[i])) ok = false;
         dmu = fmaxf(dmu, float(fabs(mu[i] - mu_old[i])));
     }
-    if (!ok) raise_error(g.ctl, k);
+    if (!ok) {
+        raise_error(g.ctl, k);
+        if (bad) *bad = 1;
+    }
     return dmu;
 }
 

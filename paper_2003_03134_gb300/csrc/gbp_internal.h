@@ -192,6 +192,7 @@ enum Ctl : int {
     // 18, 19: the device convergence loop's state (gbp_api.cu)
     CTL_RES_BASE1 = 20,    // resident kernel: its arrival counts at the end of the last launch
     CTL_RES_BASE2 = 21,
+    CTL_RES_ERR_T = 22,    // resident kernel: 1 + the check iteration that first found an error raised, 0 = none
     CTL_RES_CNT1 = 64,     // messages stored: arrivals (a cache line of their own, polled)
     CTL_RES_CNT2 = 96,     // end of iteration: arrivals
     CTL_N = 128

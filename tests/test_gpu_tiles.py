@@ -1,6 +1,7 @@
 """The deferring factor kernel against the general factor phase at the edges of its tiles: landmarks with 31, 32, 33 and
 more factors (split across tiles), tiles of one factor, landmarks without factors, relinearisations in every iteration
 (beta = 0, interval 1) and none (linear)."""
+import ctypes
 import dataclasses
 
 import numpy as np
@@ -81,3 +82,28 @@ def test_a_stream_that_outgrows_the_resident_kernel():
     assert got[0][0] == [1, 2], got[0][0]
     for a, b in zip(got[0][1:], got[1][1:]):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("scale,anneal", [(1e-30, 20), (1e-30, 60), (1e-12, 60), (1e-37, 90)])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_divergence_ends_the_convergence_loop_at_the_next_check(scale, anneal, precision):
+    """Points with one observation, whose prior all but vanishes: their beliefs stop being positive definite in the
+    middle of a solve to a tolerance.  Persistent and per-phase launches leave at the same check, and at the first
+    one of a later call, also when the error came from iterations that were not checked."""
+    p = _problem([1, 4, 5, 6] * 30)
+    got = []
+    for mode in (1, 2):
+        params = dict(launch_mode=mode, prior_final_scale=scale, prior_anneal_iters=anneal, precision_mode=precision)
+        with gbp.Graph(p, conv_tol=1e-12, check_every=5, **params) as g, gbp.Graph(p, **params) as h:
+            rec = []
+            for n in (300, 12):
+                done = ctypes.c_int32(-1)
+                rec.append((gbp.lib().gbp_iterate(g.h, n, ctypes.byref(done)), done.value))
+            assert h.iterate(100) == 100   # nothing is read back
+            h.set_params(conv_tol=1e-12, check_every=7)
+            done = ctypes.c_int32(-1)
+            rec.append((gbp.lib().gbp_iterate(h.h, 50, ctypes.byref(done)), done.value))
+            got.append(rec)
+    assert got[0] == got[1]
+    assert got[0][0][0] == gbp.GBP_EDIVERGED and 0 < got[0][0][1] < 300
+    assert got[0][1:] == [(gbp.GBP_EDIVERGED, 5), (gbp.GBP_EDIVERGED, 7)]
