@@ -812,11 +812,7 @@ gbp_status ensure_exec(gbp_graph* g) {
 // last iteration below conv_tol, no error raised -- and sets the loop's
 // condition.  The kernels, their order and the check points are the host
 // loop's, so the results and the iteration count are the same.  Two control
-// slots past the kernels' own (the Ctl enum ends at CTL_RESUMS) carry the
-// loop's state.
-constexpr int CTL_WL_LEFT = 18;     // check blocks the loop may still run
-constexpr int CTL_WL_TOL = 19;      // conv_tol, float bits
-static_assert(CTL_WL_LEFT > CTL_RESUMS && CTL_WL_TOL < CTL_N, "control slots of the device loop");
+// words of its own (CTL_WL_LEFT, CTL_WL_TOL) carry the loop's state.
 constexpr int WHILE_MAX_BODY = 64;  // longest check block recorded in the loop body
 
 __global__ void while_setup_kernel(int32_t* ctl, int32_t blocks, int32_t tol_bits) {

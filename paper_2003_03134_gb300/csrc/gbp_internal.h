@@ -189,7 +189,8 @@ enum Ctl : int {
     CTL_DEFER_N1 = 15,     // in odd iterations
     CTL_DEFER_DONE = 16,   // blocks of factor_deferred_kernel done (its last block clears the list)
     CTL_RESUMS = 17,       // keyframe incoming precisions summed again exactly from their parts (FP64)
-    // 18, 19: the device convergence loop's state (gbp_api.cu)
+    CTL_WL_LEFT = 18,      // device convergence loop (gbp_api.cu): check blocks it may still run
+    CTL_WL_TOL = 19,       // ... its conv_tol, float bits
     CTL_RES_BASE1 = 20,    // resident kernel: its arrival counts at the end of the last launch
     CTL_RES_BASE2 = 21,
     CTL_RES_ERR_T = 22,    // resident kernel: 1 + the check iteration that first found an error raised, 0 = none
