@@ -948,32 +948,50 @@ gbp_status read_ctl(gbp_graph* g) {
 // copies them on (one launch and one wait: a paper-scale read is all
 // latency); more are copied straight to the caller's pageable arrays, which
 // on this machine's coherent link runs at the rate of pinned ones (4.8 MB:
-// 37 us, where a host copy out of pinned memory takes 160).  Synchronises.
+// 37 us, where a host copy out of pinned memory takes 160).  In two halves,
+// the second after the caller has synchronised, so that the caller can work
+// in between.
 constexpr size_t SMALL_READ = 16384;
 
-gbp_status download_means(gbp_graph* g, bool world, double* kf, double* lm) {
-    const size_t nk = (size_t)g->n_kf * (world ? 12 : 6), nl = 3 * (size_t)g->n_lm;
-    const bool small = nk + nl <= SMALL_READ;
+struct MeansRead {
+    size_t nk, nl;
+    double *kf, *lm;
+    const double* pinned;   // null: copied to kf and lm directly
+};
+
+gbp_status means_enqueue(gbp_graph* g, bool world, double* kf, double* lm, MeansRead& r) {
+    r = MeansRead{(size_t)g->n_kf * (world ? 12 : 6), 3 * (size_t)g->n_lm, kf, lm, nullptr};
     double* d = nullptr;
-    if (small) {
+    if (r.nk + r.nl <= SMALL_READ) {
         if (!g->h_read) CK(cudaMallocHost(reinterpret_cast<void**>(&g->h_read), sizeof(double) * SMALL_READ));
-        d = g->h_read;
+        r.pinned = d = g->h_read;
     } else {
-        gbp_status st = read_buffer(g, nk + nl, &d);
+        gbp_status st = read_buffer(g, r.nk + r.nl, &d);
         if (st != GBP_OK) return st;
     }
-    CK(g->storage ? launch_means<double>(g->sd.g, world, d, d + nk, g->h_ctl, g->stream)
-                  : launch_means<float>(g->sf.g, world, d, d + nk, g->h_ctl, g->stream));
-    if (!small) {
-        if (nk) CK(cudaMemcpyAsync(kf, d, sizeof(double) * nk, cudaMemcpyDeviceToHost, g->stream));
-        if (nl) CK(cudaMemcpyAsync(lm, d + nk, sizeof(double) * nl, cudaMemcpyDeviceToHost, g->stream));
+    CK(g->storage ? launch_means<double>(g->sd.g, world, d, d + r.nk, g->h_ctl, g->stream)
+                  : launch_means<float>(g->sf.g, world, d, d + r.nk, g->h_ctl, g->stream));
+    if (!r.pinned) {
+        if (r.nk) CK(cudaMemcpyAsync(kf, d, sizeof(double) * r.nk, cudaMemcpyDeviceToHost, g->stream));
+        if (r.nl) CK(cudaMemcpyAsync(lm, d + r.nk, sizeof(double) * r.nl, cudaMemcpyDeviceToHost, g->stream));
     }
-    CK(cudaStreamSynchronize(g->stream));
-    if (small) {
-        std::copy(d, d + nk, kf);
-        std::copy(d + nk, d + nk + nl, lm);
+    return GBP_OK;
+}
+
+gbp_status means_finish(gbp_graph* g, const MeansRead& r) {
+    if (r.pinned) {
+        std::copy(r.pinned, r.pinned + r.nk, r.kf);
+        std::copy(r.pinned + r.nk, r.pinned + r.nk + r.nl, r.lm);
     }
     return ctl_status(g);
+}
+
+gbp_status download_means(gbp_graph* g, bool world, double* kf, double* lm) {
+    MeansRead r;
+    const gbp_status st = means_enqueue(g, world, kf, lm, r);
+    if (st != GBP_OK) return st;
+    CK(cudaStreamSynchronize(g->stream));
+    return means_finish(g, r);
 }
 
 bool finite_all(const double* p, size_t n) {
@@ -1042,29 +1060,6 @@ void order_factors(gbp_graph* g, const std::vector<int32_t>& ok, const std::vect
     for (int i = 0; i < n; ++i) g->f_of_obs[g->obs_index[i]] = i;
 }
 
-template <typename R>
-void pull_beliefs(gbp_graph* g, std::vector<double>& kb, std::vector<double>& lb, gbp_status& st) {
-    DevState<R>& s = state<R>(g);
-    std::vector<R> a((size_t)KBEL * g->n_kf), b((size_t)LBEL * g->n_lm);
-    cudaError_t e = cudaMemcpyAsync(a.data(), s.kf_bel, sizeof(R) * a.size(), cudaMemcpyDeviceToHost, g->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(b.data(), s.lm_bel, sizeof(R) * b.size(), cudaMemcpyDeviceToHost, g->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
-    if (e != cudaSuccess) {
-        st = cuda_fail(g, e, "belief download");
-        return;
-    }
-    kb.assign(a.begin(), a.end());
-    lb.assign(b.begin(), b.end());
-    st = GBP_OK;
-}
-
-gbp_status download_beliefs(gbp_graph* g, std::vector<double>& kb, std::vector<double>& lb) {
-    gbp_status st = GBP_OK;
-    if (g->storage) pull_beliefs<double>(g, kb, lb, st);
-    else pull_beliefs<float>(g, kb, lb, st);
-    return st;
-}
-
 // packed lower n x n -> full inverse (double)
 bool packed_inverse(int n, const double* P, double* out) {
     double A[36], L[36] = {0};
@@ -1096,6 +1091,36 @@ bool packed_inverse(int n, const double* P, double* out) {
         for (int i = 0; i < n; ++i) out[i * n + c] = x[i];
     }
     return true;
+}
+
+// World poses and points with the inverses of the beliefs' precisions (either
+// may be null).  The precisions first: the means are converted and read while
+// the host inverts them.
+template <typename R>
+gbp_status read_covariances(gbp_graph* g, double* kf_Rt, double* lm_xyz, double* kf_cov, double* lm_cov) {
+    const DevState<R>& s = state<R>(g);
+    std::vector<R> kb(kf_cov ? (size_t)KBEL * g->n_kf : 0), lb(lm_cov ? (size_t)LBEL * g->n_lm : 0);
+    if (!kb.empty())
+        CK(cudaMemcpyAsync(kb.data(), s.kf_bel, sizeof(R) * kb.size(), cudaMemcpyDeviceToHost, g->stream));
+    if (!lb.empty())
+        CK(cudaMemcpyAsync(lb.data(), s.lm_bel, sizeof(R) * lb.size(), cudaMemcpyDeviceToHost, g->stream));
+    CK(cudaStreamSynchronize(g->stream));
+    MeansRead r;
+    gbp_status st = means_enqueue(g, true, kf_Rt, lm_xyz, r);
+    if (st != GBP_OK) return st;
+    const char* failed = nullptr;
+    double P[21];
+    for (int v = 0; kf_cov && !failed && v < g->n_kf; ++v) {
+        std::copy_n(&kb[(size_t)KBEL * v + KB_LAM], 21, P);
+        if (!packed_inverse(6, P, kf_cov + 36 * (size_t)v)) failed = "keyframe belief not positive definite";
+    }
+    for (int v = 0; lm_cov && !failed && v < g->n_lm; ++v) {
+        std::copy_n(&lb[(size_t)LBEL * v], 6, P);
+        if (!packed_inverse(3, P, lm_cov + 9 * (size_t)v)) failed = "landmark belief not positive definite";
+    }
+    CK(cudaStreamSynchronize(g->stream));
+    st = means_finish(g, r);
+    return failed ? fail(g, GBP_EDIVERGED, failed) : st;
 }
 
 gbp_status compute_uv_ref(gbp_graph* g, const double* kf_Rt, const double* lm) {
@@ -1816,19 +1841,9 @@ gbp_status gbp_get_means(const gbp_graph* cg, double* kf_mu, double* lm_mu) {
 gbp_status gbp_get_beliefs(const gbp_graph* cg, double* kf_Rt, double* lm_xyz, double* kf_cov, double* lm_cov) {
     gbp_graph* g = const_cast<gbp_graph*>(cg);
     if (!g || (g->n_kf && !kf_Rt) || (g->n_lm && !lm_xyz)) return GBP_EINVAL;
-    const gbp_status st = download_means(g, true, kf_Rt, lm_xyz);
-    if (kf_cov || lm_cov) {
-        std::vector<double> kb, lb;
-        const gbp_status dst = download_beliefs(g, kb, lb);
-        if (dst != GBP_OK) return dst;
-        for (int v = 0; kf_cov && v < g->n_kf; ++v)
-            if (!packed_inverse(6, &kb[(size_t)KBEL * v + KB_LAM], kf_cov + 36 * (size_t)v))
-                return fail(g, GBP_EDIVERGED, "keyframe belief not positive definite");
-        for (int v = 0; lm_cov && v < g->n_lm; ++v)
-            if (!packed_inverse(3, &lb[(size_t)LBEL * v], lm_cov + 9 * (size_t)v))
-                return fail(g, GBP_EDIVERGED, "landmark belief not positive definite");
-    }
-    return st;
+    if (!kf_cov && !lm_cov) return download_means(g, true, kf_Rt, lm_xyz);
+    return g->storage ? read_covariances<double>(g, kf_Rt, lm_xyz, kf_cov, lm_cov)
+                      : read_covariances<float>(g, kf_Rt, lm_xyz, kf_cov, lm_cov);
 }
 
 gbp_status gbp_set_reference(gbp_graph* g, const double* ref_kf_Rt, const double* ref_lm) {

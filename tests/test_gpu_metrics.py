@@ -108,3 +108,19 @@ def test_reference_solution_through_precision_switches_and_added_keyframes():
                             h.iterate(4)
                     for a, b in zip(f.means(), g.means()):
                         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("n_lm", [300, 6000])
+def test_beliefs_with_covariances_are_those_without(n_lm):
+    """Poses and points read beside the covariances (one wait for both; up to 16384 doubles of them through pinned
+    memory) are those read alone."""
+    p = synth.make_walk(6, n_kf=24, n_lm=n_lm)
+    with gbp.Graph(p, huber_nsigma=2.0) as g:
+        g.iterate(15)
+        kf, lm = g.beliefs()
+        kf2, lm2, kc, lc = g.beliefs(covariances=True)
+        g.iterate(1)
+        assert not np.array_equal(g.beliefs()[0], kf)
+        assert np.array_equal(kf, kf2) and np.array_equal(lm, lm2)
+        for c in (kc, lc):
+            assert (np.linalg.eigvalsh(c) > 0).all()
