@@ -32,7 +32,8 @@ static_assert(GBP_SPLIT_KF_FLOATS == KBEL, "split keyframe record");
 namespace {
 
 constexpr int GRAPH_CHUNK = 8;   // iterations per captured CUDA graph
-constexpr size_t STAGE_MAX = 4 << 20;   // host arrays of a grown layout up to this many bytes go up in one pinned copy
+constexpr size_t STAGE_MAX = 4 << 20;    // host arrays of a grown layout up to this many bytes go up out of pinned memory
+constexpr size_t STAGE_PIECE = 1 << 20;  // ... at least this many at a time
 
 template <typename T>
 cudaError_t dev_alloc(T** p, size_t n) {
@@ -479,11 +480,14 @@ gbp_status build_device(gbp_graph* g, RelayoutSrc<R>* rs = nullptr, const std::v
             breaks.push_back(g->part_lm1);
         }
         std::sort(breaks.begin(), breaks.end());
-        struct Open {
-            size_t tile;
-            int used;
+        int used[OPEN_TILES] = {}, n_open = 0;   // open tiles, oldest first: lanes taken
+        size_t open[OPEN_TILES] = {};            // ... and which tile it is
+        const auto close = [&](int o) {
+            for (--n_open; o < n_open; ++o) {
+                used[o] = used[o + 1];
+                open[o] = open[o + 1];
+            }
         };
-        std::vector<Open> open;   // oldest first
         auto new_tile = [&](int m) {
             tf.resize(tf.size() + 32, -1);
             tile_lm.push_back(m);
@@ -492,7 +496,7 @@ gbp_status build_device(gbp_graph* g, RelayoutSrc<R>* rs = nullptr, const std::v
         size_t next_brk = 0;
         for (int m = 0; m < nl; ++m) {
             const int lo = lm_off[m], hi = lm_off[m + 1], d = hi - lo;
-            for (; next_brk < breaks.size() && breaks[next_brk] <= m; ++next_brk) open.clear();
+            for (; next_brk < breaks.size() && breaks[next_brk] <= m; ++next_brk) n_open = 0;
             if (d == 0) {
                 orphan.push_back(nk + m);
                 continue;
@@ -505,18 +509,26 @@ gbp_status build_device(gbp_graph* g, RelayoutSrc<R>* rs = nullptr, const std::v
                 big.push_back(m);
                 continue;
             }
-            int best = -1;
-            for (size_t o = 0; o < open.size(); ++o)
-                if (open[o].used + d <= 32 && (best < 0 || open[o].used > open[(size_t)best].used)) best = (int)o;
-            if (best < 0) {
-                if (open.size() == OPEN_TILES) open.erase(open.begin());
-                open.push_back(Open{new_tile(m), 0});
-                best = (int)open.size() - 1;
+            // the fullest open tile with room, the oldest of equals, without a
+            // branch a tile (which mispredicts at most points of many factors);
+            // points of few factors leave few tiles open
+            const auto rank = [&](int o) { return used[o] + d <= 32 ? OPEN_TILES * used[o] + (OPEN_TILES - 1 - o) : 0; };
+            int most = 0;
+            if (n_open == OPEN_TILES)
+                for (int o = 0; o < OPEN_TILES; ++o) most = std::max(most, rank(o));
+            else
+                for (int o = 0; o < n_open; ++o) most = std::max(most, rank(o));
+            int best = OPEN_TILES - 1 - most % OPEN_TILES;
+            if (!most) {
+                if (n_open == OPEN_TILES) close(0);
+                best = n_open++;
+                used[best] = 0;
+                open[best] = new_tile(m);
             }
-            Open& o = open[(size_t)best];
-            for (int f = lo; f < hi; ++f) tf[32 * o.tile + o.used + (f - lo)] = f;
-            o.used += d;
-            if (o.used == 32) open.erase(open.begin() + best);
+            int32_t* const at = tf.data() + 32 * open[best] + used[best];
+            for (int i = 0; i < d; ++i) at[i] = lo + i;
+            used[best] += d;
+            if (used[best] == 32) close(best);
         }
     }
     const int n_tiles = (int)tile_lm.size();
@@ -596,10 +608,20 @@ gbp_status build_device(gbp_graph* g, RelayoutSrc<R>* rs = nullptr, const std::v
     if (staged) {
         if (!g->h_stage) CK(cudaMallocHost(reinterpret_cast<void**>(&g->h_stage), STAGE_MAX));
         if (g->stage_busy) CK(cudaStreamSynchronize(st));
-        for (const Item& it : items)
-            if (it.src && it.bytes) std::memcpy(g->h_stage + it.at, it.src, it.bytes);
-        CK(cudaMemcpyAsync(s.arena, g->h_stage, up_bytes, cudaMemcpyHostToDevice, st));
         g->stage_busy = true;
+        size_t sent = 0, ready = 0;
+        const auto send = [&] {   // in pieces, so that a long upload runs beside the staging of the rest
+            const cudaError_t e = cudaMemcpyAsync(s.arena + sent, g->h_stage + sent, ready - sent, cudaMemcpyHostToDevice, st);
+            sent = ready;
+            return e;
+        };
+        for (const Item& it : items) {
+            if (!it.src || !it.bytes) continue;
+            std::memcpy(g->h_stage + it.at, it.src, it.bytes);
+            ready = it.at + it.bytes;
+            if (ready - sent >= STAGE_PIECE) CK(send());
+        }
+        if (ready > sent) CK(send());
     } else {
         for (const Item& it : items)
             if (it.src && it.bytes)
