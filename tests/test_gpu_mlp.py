@@ -202,3 +202,64 @@ def test_forward_rows_do_not_depend_on_their_place(torch, n, offset):
     assert bool((y[n:] == -1.0).all())
     ref, _ = mlp.forward(p, X.astype(np.float64))
     assert np.abs(y[:n].cpu().numpy() - ref).max() <= 0.02
+
+
+# One wave of mlp_grad_kernel's warps takes 2048 x 32 rows; more go in groups of 128 a warp.
+WAVE_ROWS = 2048 * 32
+
+
+@pytest.mark.parametrize("n", [WAVE_ROWS, WAVE_ROWS + 1, WAVE_ROWS + 97])
+def test_gradient_and_step_around_one_wave_of_rows(torch, n):
+    """Both sides of the switch from a warp per 32 rows to a warp per 128, the last group one row, a group and a
+    row: the gradient against the reference, twice the same bits; an Adam step moves every parameter by what its
+    gradient says, and the packed weights are the new ones."""
+    p = _params(9)
+    X, t = _data(17, n)
+    Xd, td = _dev(torch, X), _dev(torch, t)
+    net = gbp.DampingNet(p)
+    loss, g = net.gradient(Xd.data_ptr(), td.data_ptr(), n)
+    loss2, g2 = net.gradient(Xd.data_ptr(), td.data_ptr(), n)
+    assert loss == loss2
+    np.testing.assert_array_equal(g, g2)
+    rl, rg = mlp.loss_and_grad(p, X.astype(np.float64), t.astype(np.float64))
+    assert abs(loss - rl) <= 0.01 * rl
+    for name, a, b, tol in BLOCKS:
+        assert np.linalg.norm(g[a:b] - rg[a:b]) <= tol * np.linalg.norm(rg[a:b]), name
+    lr = 1e-3
+    net.train_step(Xd.data_ptr(), td.data_ptr(), n, lr)
+    w0, w1 = p.astype(np.float32).astype(np.float64), net.params.astype(np.float64)
+    step = lr * g / (np.abs(g) + 1e-8)
+    # powf may be 4 ulp (2.4e-7) off, which 1 - 0.999^1 = 1e-3 amplifies to 2.4e-4 in the second moment, half of it
+    # in its root; the other roundings are below 1e-6; the new weight rounds once
+    assert (np.abs(w1 - (w0 - step)) <= 1.5e-4 * lr + 2.0 ** -24 * np.abs(w1)).all()
+    other = gbp.DampingNet(w1)
+    y, yo = (torch.empty(1000, dtype=torch.float32, device="cuda") for _ in range(2))
+    net.forward(Xd.data_ptr(), 1000, y.data_ptr())
+    other.forward(Xd.data_ptr(), 1000, yo.data_ptr())
+    torch.cuda.synchronize()
+    assert torch.equal(y, yo)
+    net.close()
+    other.close()
+
+
+def test_grouped_rows_add_up_as_single_ones_do(torch):
+    """Rows whose output is saturated at their target have a gradient of exactly zero.  As many of them behind one
+    wave of rows halve the batch's weights, and nothing else: the grouped gradient of all is, bit for bit, half the
+    ungrouped one of the wave."""
+    p = _params(10)
+    X, t = _data(19, WAVE_ROWS)
+    rng = np.random.default_rng(20)
+    big = (200.0 * rng.normal(size=(4096, 16))).astype(np.float32)
+    y, _ = mlp.forward(p, big.astype(np.float64))
+    big = big[y == y.max()]   # 1 / (1 + exp(-z)) rounds to 1 in 64 bits: z > 36
+    assert len(big) > 500 and abs(y.max() - 0.9) < 1e-15
+    fill = big[np.arange(WAVE_ROWS) % len(big)]
+    net = gbp.DampingNet(p)
+    Xa, ta = _dev(torch, X), _dev(torch, t)
+    Xb = _dev(torch, np.concatenate([X, fill]))
+    tb = _dev(torch, np.concatenate([t, np.full(WAVE_ROWS, 0.9, np.float32)]))
+    la, ga = net.gradient(Xa.data_ptr(), ta.data_ptr(), WAVE_ROWS)
+    lb, gb = net.gradient(Xb.data_ptr(), tb.data_ptr(), 2 * WAVE_ROWS)
+    assert lb == 0.5 * la
+    np.testing.assert_array_equal(gb, np.float32(0.5) * ga)
+    net.close()
