@@ -89,8 +89,9 @@ def kernel_source_hash():
 def ncu_traffic(n_f, regime):
     """DRAM bytes per factor-kernel launch from the committed ncu capture of
     the same regime ("l2_resident" for the paper-scale problem, "hbm" for
-    the batched workload), scaled to this launch's factor count; None if
-    the kernel changed since the capture."""
+    the batched workload; "resident": per iteration of the resident kernel at
+    paper scale), scaled to this launch's factor count; None if the kernel
+    changed since the capture."""
     path = os.path.join(ROOT, "profiles", "factor_kernel_traffic.json")
     try:
         with open(path) as f:
@@ -234,14 +235,32 @@ def oracle_solution(p, max_iters, tol):
     return kf, lm, it, dt, t_1px
 
 
-def roofline(p, iter_ms, fac_ms, mode, regime="l2_resident"):
+def kernels_of(mode, tuning=None, n_obs=0):
+    """The kernels that run an FP32 fixed-schedule iteration in the launch mode gbp_iterate used.  A persistent
+    launch is the resident kernel where that applies: always when the mode was taken by size (one candidate, time 0),
+    never with more observations than 8 full tiles an SM of 152 hold; in between (forced or timed) the record does
+    not say."""
+    if mode != 1:
+        return "factor_kernel<float> + belief_kernel<float>"
+    c = (tuning or {}).get("candidates", [])
+    if len(c) == 1 and c[0]["launch_mode"] == 1 and c[0]["ms"] == 0:
+        return "resident_kernel"
+    if n_obs > 32 * 8 * 152:
+        return "persistent_kernel<float>"
+    return "resident_kernel or persistent_kernel<float>"
+
+
+def roofline(p, iter_ms, fac_ms, mode, regime="l2_resident", tuning=None):
+    """Of one iteration.  traffic is what ncu counted for the kernels named: the factor kernel's launch (per phase),
+    an iteration's share of a launch of 200 (resident kernel), else None."""
     bytes_iter = BYTES_PER_FACTOR * p.n_obs + BYTES_PER_KF * p.n_kf + BYTES_PER_LM * p.n_lm
     impl_iter = bytes_iter + IMPL_EXTRA_PER_FACTOR * p.n_obs
     peak, peak_kind = peaks()
     achieved = bytes_iter / (iter_ms * 1e-3) / 1e9
+    kernel = kernels_of(mode, tuning, p.n_obs)
+    traffic_of = {kernels_of(2): regime, "resident_kernel": "resident"}
     return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-            "traffic": ncu_traffic(p.n_obs, regime),
-            "kernel": "persistent_kernel<float>" if mode == 1 else "factor_kernel<float> + belief_kernel<float>",
+            "traffic": ncu_traffic(p.n_obs, traffic_of.get(kernel, "none")), "kernel": kernel,
             "launch_mode": mode, "bytes_per_iteration": bytes_iter,
             "bytes_rule": f"{BYTES_PER_FACTOR} B/factor + {BYTES_PER_KF} B/keyframe + {BYTES_PER_LM} B/point "
                           "(paper message form)",
@@ -394,7 +413,7 @@ def measure_loop(gbp, stream, p, iters=20, launch_mode=0, factor_shape=-1, with_
         pass
     sz = _Size()
     sz.n_obs, sz.n_kf, sz.n_lm = n_f, n_kf, n_lm
-    roof = roofline(sz, iter_ms, fac_ms, mode, "hbm")
+    roof = roofline(sz, iter_ms, fac_ms, mode, "hbm", tuning)
     bytes_iter = roof["bytes_per_iteration"]
     peak = roof["peak"]
     out = {"workload": f"loop{n_kf}x{n_lm}: {n_kf} keyframes on two laps of a 30 m loop, {n_lm} points, {n_f} "
@@ -473,7 +492,7 @@ def measure_at_scale(gbp, stream, rank=0, world=1, n_problems=256, iters=20, lau
             "value": job_f / (job_ms * 1e-3), "unit": UNIT, "ms_per_iteration": job_ms,
             "ranks": world, "partition": "size-balanced (largest first to the least-loaded rank)",
             "autotune_ms_per_iteration": {"persistent": ms1, "per_phase": ms2}, "tuning": tuning,
-            "roofline": roofline(sz, iter_ms, fac_ms, mode, "hbm"), "fp64_fallbacks": st["fp64_fallbacks"]}
+            "roofline": roofline(sz, iter_ms, fac_ms, mode, "hbm", tuning), "fp64_fallbacks": st["fp64_fallbacks"]}
 
 
 def run_gpu(args, rank, world, local):
@@ -535,7 +554,7 @@ def run_gpu(args, rank, world, local):
     # iterations in the mode gbp_iterate used, and the factor kernel alone)
     g.reset()
     iter_ms, fac_ms = g.profile(64)
-    roof = roofline(p, iter_ms, fac_ms, st_timed["launch_mode"])
+    roof = roofline(p, iter_ms, fac_ms, st_timed["launch_mode"], tuning=tuning)
     loop_pool = loop_job = None
     if rank == 0 and not args.no_loop:
         # the ~2M-factor loop problem takes ~1.5 min to generate: in a spawned

@@ -59,3 +59,28 @@ def test_traffic_only_for_the_captured_kernel_source(tmp_path, monkeypatch):
     monkeypatch.setattr(bench, "kernel_source_hash", lambda: "changed")
     assert bench.ncu_traffic(1000, "l2_resident") is None
 
+
+
+def test_roofline_names_the_kernels_that_ran(tmp_path, monkeypatch):
+    os.makedirs(tmp_path / "profiles")
+    with open(tmp_path / "profiles" / "factor_kernel_traffic.json", "w") as f:
+        json.dump({"kernel_source_hash": "abc", "l2_resident": {"dram_bytes_per_factor": 180.0},
+                   "resident": {"dram_bytes_per_factor": 1.5}}, f)
+    monkeypatch.setattr(bench, "ROOT", str(tmp_path))
+    monkeypatch.setattr(bench, "kernel_source_hash", lambda: "abc")
+
+    class P:
+        n_obs, n_kf, n_lm = 1000, 10, 100
+
+    by_size = {"candidates": [{"launch_mode": 1, "shape": 0, "ms": 0.0}]}
+    timed = {"candidates": [{"launch_mode": m, "shape": 0, "ms": 0.01} for m in (1, 2)]}
+
+    def named(mode, tuning):
+        r = bench.roofline(P(), 0.01, 0.005, mode, tuning=tuning)
+        return r["kernel"], r["traffic"]
+
+    assert named(1, by_size) == ("resident_kernel", 1500.0)
+    assert named(2, timed) == ("factor_kernel<float> + belief_kernel<float>", 180000.0)
+    assert named(1, timed) == ("resident_kernel or persistent_kernel<float>", None)
+    P.n_obs = 1_000_000
+    assert named(1, timed) == ("persistent_kernel<float>", None)
