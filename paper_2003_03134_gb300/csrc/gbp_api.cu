@@ -548,7 +548,8 @@ gbp_status build_device(gbp_graph* g, RelayoutSrc<R>* rs = nullptr, const std::v
     // every array of the layout in one allocation, those with host contents
     // first: when a keyframe is added they travel in one copy out of pinned
     // memory (a copy each, and an allocation each, was most of what adding a
-    // keyframe cost: 0.4 -> 0.27 ms at 60 keyframes)
+    // keyframe cost: a stream at 30-60 keyframes and 960 points 366 -> 157 us a
+    // call, 385 -> 250 until the device is done)
     struct Item {
         void** dst;
         size_t bytes, at;
@@ -1336,8 +1337,8 @@ void order_factors_append(gbp_graph* g, int L1, int K0, int n_obs, const int32_t
 // Incremental SLAM (Sec. 9.2): the grown graph's layout is built on the host
 // from the index arrays alone (no state leaves the device), and the state is
 // gathered on the device from the previous layout's buffers
-// (relayout_kernel); the host reads back only the control block, the latest
-// keyframe's mean and the new variables' prior diagonals.
+// (relayout_kernel); the host reads back only the control block and the latest
+// keyframe's mean, before it starts, and waits for nothing afterwards.
 template <typename R>
 gbp_status add_keyframe_impl(gbp_graph* g, const double* kf_Rt_init, int n_new_lm, const double* new_lm_xyz,
                              int n_obs, const int32_t* obs_lm, const double* obs_uv) {
@@ -1784,9 +1785,8 @@ void tune_cache_store(const gbp_graph* g) {
 // candidates' own spread, so that a graph's first gbp_iterate need not time
 // them (16 iterations of 7 candidates, and a copy of the state: 2.7 ms at
 // paper scale, 35 ms at 2M factors, more than the solve itself):
-//   * the resident kernel with one keyframe a block (see gbp_resident.cu):
-//     328 tiles 6.1 us against 9.2 of the best per-phase shape, 591 6.6 / 9.5,
-//     624 8.1 / 9.8, 985 9.0 / 10.2, 1200 10.3 / 11.1; it takes up to 1216;
+//   * the resident kernel with one keyframe a block (gbp_resident.cu has the
+//     figures, 15 to 1190 tiles); it takes up to 1216;
 //   * per-phase launches in the shape of the size (factor_shape; alone, shape 0
 //     is within 1.5 % of the fastest at 600-1200 tiles) while graphs on other
 //     streams need the SMs (update_launch_class has the figures), and for a

@@ -1818,7 +1818,7 @@ __device__ __forceinline__ float tile_work(const DevGraph<R>& g, const KParams<R
 // The same arithmetic as tile_work, in an order that lets values go early:
 // the message to the landmark as soon as the keyframe side stands (a
 // relinearisation forms it again), then the relinearisation test (it frees
-// the keyframe's mean and the linearisation point).  127 registers, 4 blocks
+// the keyframe's mean and the linearisation point).  124 registers, 4 blocks
 // per SM.  What bounds it is the load/store unit (it carries ~130 shuffles
 // and ~45 loads a tile besides the stores), not latency or occupancy: 5
 // blocks per SM (96 registers, 130 bytes spilled) take 7 % longer, bringing

@@ -28,14 +28,16 @@
 // The arithmetic is that of tile_work and phase_b_item, expression by
 // expression, so the results are bitwise those of the per-phase kernels.
 //
-// Per iteration (200 iterations from reset, launch included) against the
-// per-phase kernels: 10 keyframes, 17 tiles 4.8-5.1 us against 8.0; 60 and
-// ~250 6.3 / 9.9; 125 and 328 6.1 / 9.2; 125 and 591 6.6 / 9.5; 624 (8 factor
-// warps a block) 8.1 / 9.8, 1200 10.3 / 11.1.  Of 9.1 us with 8 factor warps
-// and a relinearisation somewhere in every iteration (clock64 of one block):
-// the gather of the beliefs 1.3, keyframe side, test and relinearisation 2.3,
-// the arrival and its way to the slowest block's belief warps 1.5, the sums
-// and factorisation 2.4, the barrier and the spread of the blocks 1.6.
+// Per iteration (200 iterations from reset, launch included; walks, relinearising
+// somewhere in nearly every iteration) against the per-phase kernels: 10
+// keyframes, 15 tiles 4.7 us against 8.0; 60 and 225 6.7 / 10.1; 125 and 566
+// 7.2 / 10.3; 150 and 608 7.3 / 10.5; with 8 factor warps a block 125 and 634
+// 10.0 / 10.7, 150 and 976 9.8 / 11.0, 150 and 1190 11.2 / 11.7.  Of 9.1 us with
+// 8 factor warps and a relinearisation somewhere in every iteration (clock64 of
+// one block): the gather of the beliefs 1.3, keyframe side, test and
+// relinearisation 2.3, the arrival and its way to the slowest block's belief
+// warps 1.5, the sums and factorisation 2.4, the barrier and the spread of the
+// blocks 1.6.
 #include "gbp_device.cuh"
 
 #include <algorithm>
