@@ -92,7 +92,8 @@ typedef struct {
                                    per phase (factor kernel, belief kernel) replayed as a CUDA graph.
                                    A resident launch holds its SMs until its iterations are done: in
                                    auto mode a graph takes it only while its blocks and those of the
-                                   graphs that run on other streams fit the device together.
+                                   graphs that have iterated on other streams, until they are
+                                   destroyed, fit the device together.
                                    All modes give bitwise identical results.                        */
     int32_t damping_mode;       /* 0: the fixed d above (Sec. 5, Sec. 8); 1: per-factor d predicted by
                                    the damping network given to gbp_set_damping_model (see below)   */
@@ -281,10 +282,11 @@ gbp_status gbp_profile_iterations(gbp_graph* g, int32_t n_iters, double* ms_out)
  * kernel's register budget.  The warp tile (up to 32 factors, whole
  * landmarks) is not tuned: it decides which landmarks are summed across
  * tiles, and so the arithmetic.  *chosen (nullable) receives the chosen
- * mode; ms_out (nullable, 2 doubles) the best mean time per iteration of
- * modes 1 and 2 (-1: no candidate of that mode could launch, e.g. a
- * persistent grid that does not fit).  gbp_get_tuning reports every
- * candidate.  Synchronises the stream. */
+ * mode; it holds until added keyframes change which kinds of launch apply to
+ * the graph (see launch_mode).  ms_out (nullable, 2 doubles) receives the
+ * best mean time per iteration of modes 1 and 2 (-1: no candidate of that
+ * mode could launch, e.g. a persistent grid that does not fit).
+ * gbp_get_tuning reports every candidate.  Synchronises the stream. */
 gbp_status gbp_autotune(gbp_graph* g, int32_t n_trial, int32_t* chosen, double* ms_out);
 
 #define GBP_MAX_TUNING_CANDIDATES 12

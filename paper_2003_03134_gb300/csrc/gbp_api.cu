@@ -172,7 +172,9 @@ void so3_exp_host(const double w[3], double E[9]) {
 // resident kernel (gbp_resident.cu) takes the graph, which added keyframes
 // change in both directions: a point without observations or one seen by more
 // than 32 keyframes excludes it, the next keyframe may bring it back.  Each
-// class keeps its own choice, made once a graph.
+// class keeps its own choice, made once a graph.  And on what else runs: while
+// graphs on other streams need its SMs, resident launches would follow one
+// another.
 enum LaunchClass : int {
     LC_GENERAL = 0,         // not for the resident kernel
     LC_RESIDENT = 1,        // resident kernel, one keyframe a block (up to two once the graph has grown)
@@ -382,13 +384,13 @@ int sms_of_other_streams(gbp_graph* g, int sms) {
 // overlap: graphs of 125 keyframes and 566 tiles (142 blocks), 200 iterations
 // each, all of them: 2 streams 2.94 ms resident, 2.30 per phase; 4 streams 5.88
 // / 2.92; 8 streams 11.6 / 4.96; of 68 blocks each 2 streams 1.42 / 2.13, 4
-// streams 2.77 / 2.34; of 10 blocks 8 streams 1.25 / 2.18.  A graph that grew while it
-// ran on the resident kernel stays on it up to two keyframes a block: in calls
-// of 20 iterations, as a stream makes them, 160-250 keyframes take 12.5-12.8 us
-// an iteration against 14.5-14.8 per phase (whose launches count more there);
-// one launch of many iterations takes 8.2 against 10.1 at 160, 10.6 / 10.1 at
-// 200, 11.3 / 10.6 at 300, and beyond two a block the resident kernel loses
-// both ways (400: 13.0 / 10.6, 500: 15.2 / 10.6).
+// streams 2.77 / 2.34; of 10 blocks 8 streams 1.25 / 2.18.
+// A graph that grew while it ran on the resident kernel stays on it up to two
+// keyframes a block: in calls of 20 iterations, as a stream makes them, 160-250
+// keyframes take 12.5-12.8 us an iteration against 14.5-14.8 per phase (whose
+// launches count more there); one launch of many iterations takes 8.2 against
+// 10.1 at 160, 10.6 / 10.1 at 200, 11.3 / 10.6 at 300, and beyond two a block
+// the resident kernel loses both ways (400: 13.0 / 10.6, 500: 15.2 / 10.6).
 void update_launch_class(gbp_graph* g) {
     int c = LC_GENERAL;
     const int blocks = resident_blocks(g);
@@ -1762,7 +1764,8 @@ bool tune_key(const gbp_graph* g, TuneKey& key) {
 
 bool tune_cache_lookup(gbp_graph* g) {
     TuneKey key;
-    if (!tune_key(g, key)) return false;
+    // what was timed alone says nothing of a chip shared with other streams
+    if (g->lclass == LC_SHARED || !tune_key(g, key)) return false;
     std::lock_guard<std::mutex> lock(g_tune_mu);
     auto it = g_tune_cache.find(key);
     if (it == g_tune_cache.end()) return false;

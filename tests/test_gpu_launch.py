@@ -223,6 +223,8 @@ def test_graphs_on_several_streams_leave_the_resident_kernel_when_they_do_not_fi
 
     a = graph(big, s1)
     assert run(a) == 1
+    with graph(big, s2) as tuned_beside:   # timed where it does not fit, whatever that says is its own
+        tuned_beside.autotune(4)
     same, beside, b = graph(big, s1), graph(small, s2), graph(big, s2)
     assert run(same) == 1 and run(beside) == 1 and run(a) == 1   # one stream; room for both
     assert [run(b), run(a), run(same), run(b)] == [2, 2, 2, 2]
